@@ -904,6 +904,8 @@ int launch_fwd_bf16_single(const void* q, const void* k, const void* v, void* o,
 #else
 int launch_fwd_bf16(const void* q, const void* k, const void* v, void* o, const Problem& p, int* status,
                     cudaStream_t stream, unsigned long long* launches, cudaError_t* cuda_err) {
+  if (p.split_ws != nullptr && decode_kernel_serves(p))
+    return launch_decode_bf16(q, k, v, o, p, status, stream, launches, cuda_err);
   int dev = 0, num_sms = 0;
   *cuda_err = cudaGetDevice(&dev);
   if (*cuda_err != cudaSuccess) return SIGATTN_ERR_CUDA;
