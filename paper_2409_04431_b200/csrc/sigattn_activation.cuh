@@ -115,4 +115,46 @@ __device__ __forceinline__ void sigmoid_block(const float (&a)[N], float (&pr)[N
   else sigmoid_exact<N, WITH_SLOPE>(a, pr, pp);
 }
 
+// Share of the forward's exponentials evaluated on the FMA pipe (every m-th, 0 = none).
+// At D = 128 the shorter instruction stream wins (emulating every 4th measured -6 %); at
+// D = 64, where a tile step has half the tensor work per exponential, unloading the MUFU
+// pipe gains 1-3 % with a causal mask (N = 2048 and 8192) and loses 3-5 % without one
+// (N = 2048 and 8100), so only the causal instantiations do it.
+__host__ __device__ constexpr int fwd_emulate_every(int D, bool causal) { return (D == 64 && causal) ? 8 : 0; }
+
+// NC logits of one row -> NC / 2 packed bf16x2 sigmoid values.
+//   a = s * scale_log2e + c0   (c0 carries the bias and, with ALiBi, the position term)
+// CAUSAL: every key that keeps its weight sits at or before the query, so |i - j| = i - j there and the
+// position term is linear in the column: one FMA per logit from a per-call constant instead of a
+// difference and an FMA with |.| (what a masked key gets instead is blanked afterwards).
+template <int NC, bool ALIBI, bool CAUSAL, int EMULATE_EVERY, bool TWO_SIDED = false>
+__device__ __forceinline__ void sigmoid_cols(const uint32_t (&s)[NC], uint32_t (&out)[NC / 2],
+                                             float scale_log2e, float bias_log2e, float slope_log2e, float row_rel,
+                                             int col_base, bool masked, float mask_limit, float mask_first = 0.0f) {
+  float a[NC];
+  const float c_first = fmaf(-slope_log2e, row_rel - static_cast<float>(col_base), bias_log2e);   // column col_base
+#pragma unroll
+  for (int i = 0; i < NC; ++i) {
+    float c0 = bias_log2e;
+    if (ALIBI && CAUSAL) {
+      c0 = fmaf(slope_log2e, static_cast<float>(i), c_first);
+    } else if (ALIBI) {
+      const float dist = row_rel - static_cast<float>(col_base + i);
+      c0 = fmaf(-slope_log2e, fabsf(dist), bias_log2e);
+    }
+    a[i] = fmaf(__uint_as_float(s[i]), scale_log2e, c0);
+  }
+  float pr[NC];
+  sigmoid_block<NC, false, EMULATE_EVERY>(a, pr, nullptr);
+  if (masked) {  // keys after the query (and, in a padded batch, past the sequence's end) get weight 0
+#pragma unroll
+    for (int i = 0; i < NC; ++i)
+      if (static_cast<float>(col_base + i) > mask_limit ||
+          (TWO_SIDED && static_cast<float>(col_base + i) < mask_first))   // keys before the row's own sequence
+        pr[i] = 0.0f;
+  }
+#pragma unroll
+  for (int i = 0; i < NC / 2; ++i) out[i] = sm100::pack_bf16x2(pr[2 * i], pr[2 * i + 1]);
+}
+
 }  // namespace sigattn

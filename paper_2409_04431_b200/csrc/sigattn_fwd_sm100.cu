@@ -66,22 +66,6 @@ constexpr float kLog2e = 1.4426950408889634f;
 constexpr uint32_t kTmemCols = 256 * kTiles;       // per tile: 128 columns of logits / P, up to 128 of O
 constexpr int kCtasPerSm = (kTiles == 1) ? 2 : 1;
 
-// Share of the forward's exponentials evaluated on the FMA pipe (every m-th, 0 = none).
-// At D = 128 the shorter instruction stream wins (emulating every 4th measured -6 %); at
-// D = 64, where a tile step has half the tensor work per exponential, unloading the MUFU
-// pipe gains 1-3 % with a causal mask (N = 2048 and 8192) and loses 3-5 % without one
-// (N = 2048 and 8100), so only the causal instantiations do it.
-#ifndef SIGATTN_FWD_EMULATE_D64
-#define SIGATTN_FWD_EMULATE_D64 8
-#endif
-#ifndef SIGATTN_FWD_EMULATE_D64_UNMASKED
-#define SIGATTN_FWD_EMULATE_D64_UNMASKED 0
-#endif
-#ifndef SIGATTN_FWD_EMULATE_D128
-#define SIGATTN_FWD_EMULATE_D128 0
-#endif
-
-
 template <int D>
 struct FwdSmem {
   static constexpr int kPanels = D / 64;
@@ -467,41 +451,6 @@ __device__ __forceinline__ void tmem_st_cols(uint32_t addr, uint32_t (&v)[N]) {
   if constexpr (N == 16) tmem_st16(addr, v); else tmem_st32(addr, v);
 }
 
-// NC logits of one row -> NC / 2 packed bf16x2 sigmoid values.
-//   a = s * scale_log2e + c0   (c0 carries the bias and, with ALiBi, the position term)
-// CAUSAL: every key that keeps its weight sits at or before the query, so |i - j| = i - j there and the
-// position term is linear in the column: one FMA per logit from a per-call constant instead of a
-// difference and an FMA with |.| (what a masked key gets instead is blanked afterwards).
-template <int NC, bool ALIBI, bool CAUSAL, int EMULATE_EVERY, bool TWO_SIDED = false>
-__device__ __forceinline__ void sigmoid_cols(const uint32_t (&s)[NC], uint32_t (&out)[NC / 2],
-                                             float scale_log2e, float bias_log2e, float slope_log2e, float row_rel,
-                                             int col_base, bool masked, float mask_limit, float mask_first = 0.0f) {
-  float a[NC];
-  const float c_first = fmaf(-slope_log2e, row_rel - static_cast<float>(col_base), bias_log2e);   // column col_base
-#pragma unroll
-  for (int i = 0; i < NC; ++i) {
-    float c0 = bias_log2e;
-    if (ALIBI && CAUSAL) {
-      c0 = fmaf(slope_log2e, static_cast<float>(i), c_first);
-    } else if (ALIBI) {
-      const float dist = row_rel - static_cast<float>(col_base + i);
-      c0 = fmaf(-slope_log2e, fabsf(dist), bias_log2e);
-    }
-    a[i] = fmaf(__uint_as_float(s[i]), scale_log2e, c0);
-  }
-  float pr[NC];
-  sigmoid_block<NC, false, EMULATE_EVERY>(a, pr, nullptr);
-  if (masked) {  // keys after the query (and, in a padded batch, past the sequence's end) get weight 0
-#pragma unroll
-    for (int i = 0; i < NC; ++i)
-      if (static_cast<float>(col_base + i) > mask_limit ||
-          (TWO_SIDED && static_cast<float>(col_base + i) < mask_first))   // keys before the row's own sequence
-        pr[i] = 0.0f;
-  }
-#pragma unroll
-  for (int i = 0; i < NC / 2; ++i) out[i] = pack_bf16x2(pr[2 * i], pr[2 * i + 1]);
-}
-
 // All activation threads work on the same query tile at a time, alternating between the
 // two tiles of the item: thread (g, r) owns row r and key columns [kCols g, kCols g + kCols)
 // of the tile.  While the groups evaluate one tile, the tensor pipe runs
@@ -597,8 +546,7 @@ __device__ void fwd_act_role(const FwdParams& p, const CUtensorMap* tmO, uint8_t
         // bf16 P goes back over the first half of the columns this thread reads, 32 logits at a time
         // (the packed values of a later run land on logits that an earlier run has consumed)
         const uint32_t tS = tmem + t * kBN + lane_off + g * kCols;
-        constexpr int kEmulateEvery = (D == 128) ? SIGATTN_FWD_EMULATE_D128
-                                      : CAUSAL ? SIGATTN_FWD_EMULATE_D64 : SIGATTN_FWD_EMULATE_D64_UNMASKED;
+        constexpr int kEmulateEvery = fwd_emulate_every(D, CAUSAL);
 #pragma unroll
         for (int c = 0; c < kCols / kRun; ++c) {
           uint32_t sv[kRun];
@@ -906,6 +854,7 @@ int launch_fwd_bf16(const void* q, const void* k, const void* v, void* o, const 
                     cudaStream_t stream, unsigned long long* launches, cudaError_t* cuda_err) {
   if (p.split_ws != nullptr && decode_kernel_serves(p))
     return launch_decode_bf16(q, k, v, o, p, status, stream, launches, cuda_err);
+  if (short_fwd_serves(p)) return launch_short_fwd_bf16(q, k, v, o, p, status, stream, launches, cuda_err);
   int dev = 0, num_sms = 0;
   *cuda_err = cudaGetDevice(&dev);
   if (*cuda_err != cudaSuccess) return SIGATTN_ERR_CUDA;

@@ -55,6 +55,11 @@ int launch_fwd_bf16(const void* q, const void* k, const void* v, void* o, const 
 int launch_fwd_bf16_single(const void* q, const void* k, const void* v, void* o, const Problem& p, int* status,
                            cudaStream_t stream, unsigned long long* launches, cudaError_t* cuda_err);
 
+// Short plain sequences with heads of 64 (see the kernel's file).
+bool short_fwd_serves(const Problem& p);
+int launch_short_fwd_bf16(const void* q, const void* k, const void* v, void* o, const Problem& p, int* status,
+                          cudaStream_t stream, unsigned long long* launches, cudaError_t* cuda_err);
+
 // Few query rows against a cache: keys of a head divided over a cluster, no scratch (see the kernel's file).
 bool decode_kernel_serves(const Problem& p);
 int launch_decode_bf16(const void* q, const void* k, const void* v, void* o, const Problem& p, int* status,
