@@ -170,7 +170,7 @@ sigattn_decode_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid
     }
     __syncwarp();
   } else if (warp == kDecMmaWarp) {
-    if ((threadIdx.x & 31) == 0) {
+    if (elect_one()) {
       const uint32_t idesc_s = make_idesc_bf16(kDecTile, 0, 0, 0) | (static_cast<uint32_t>(rows16 >> 3) << 17);
       constexpr uint32_t kIdescPV = make_idesc_bf16(kDecTile, D, 0, 1);
       const uint64_t q_desc = make_smem_desc_sw128(smem_base + q_off, 16, 1024);
