@@ -60,5 +60,7 @@ __all__ = list(_BINDING_NAMES)
 def __getattr__(name):
     if name in _BINDING_NAMES:
         from . import binding
-        return getattr(binding, name)
+        value = getattr(binding, name)
+        globals()[name] = value   # later uses find the name without coming here (6 us a call otherwise)
+        return value
     raise AttributeError(f"module {__name__!r} has no attribute {name!r}")

@@ -1,17 +1,20 @@
-"""Builds libsigattn.so in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Builds libsigattn.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and the compiled host side of
+the Python binding (_sigattn_host.so) against the installed torch."""
 from __future__ import annotations
 
+import importlib.util
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libsigattn.so")
+HOST_PATH = os.path.join(PKG_DIR, "_sigattn_host.so")
 SOURCES = ["sigattn_api.cu", "sigattn_fp32.cu", "sigattn_fwd_sm100.cu", "sigattn_fwd_single_sm100.cu", "sigattn_bwd_sm100.cu",
-           "sigattn_decode_sm100.cu", "sigattn_short_fwd_sm100.cu",
-           "sigattn_static_scratch.cu", "sigattn_peer.cu"]
+           "sigattn_decode_sm100.cu", "sigattn_short_fwd_sm100.cu", "sigattn_static_scratch.cu", "sigattn_peer.cu"]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
     "-O3", "-std=c++17", "-lineinfo",
@@ -27,10 +30,23 @@ def _nvcc() -> str:
     return path
 
 
+def _host_command() -> list[str]:
+    """g++ command of the host module: torch's own headers and libraries, libsigattn.so from beside it."""
+    torch_dir = list(importlib.util.find_spec("torch").submodule_search_locations)[0]
+    inc = os.path.join(torch_dir, "include")
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
+    return ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+            "-I", sysconfig.get_paths()["include"], "-isystem", inc,
+            "-isystem", os.path.join(inc, "torch", "csrc", "api", "include"), "-isystem", os.path.join(cuda, "include"),
+            os.path.join(CSRC, "host_calls.cpp"), "-o", HOST_PATH, "-L", os.path.join(torch_dir, "lib"),
+            "-ltorch_python", "-ltorch_cpu", "-ltorch", "-lc10", "-lc10_cuda", "-L", PKG_DIR, "-lsigattn",
+            "-Wl,-rpath,$ORIGIN"]
+
+
 def _stale() -> bool:
-    if not os.path.exists(LIB_PATH):
+    if not os.path.exists(LIB_PATH) or not os.path.exists(HOST_PATH):
         return True
-    built = os.path.getmtime(LIB_PATH)
+    built = min(os.path.getmtime(LIB_PATH), os.path.getmtime(HOST_PATH))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
     deps.append(os.path.join(os.path.dirname(PKG_DIR), "include", "sigattn.h"))
     deps.append(os.path.abspath(__file__))
@@ -38,7 +54,7 @@ def _stale() -> bool:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every CUDA source into libsigattn.so (one object per source, in parallel)."""
+    """Compile every CUDA source into libsigattn.so (one object per source, in parallel), then the host module."""
     if not force and not _stale():
         return LIB_PATH
     nvcc = _nvcc()
@@ -65,6 +81,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         raise RuntimeError("libsigattn.so build failed")
     link = [nvcc, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", LIB_PATH, *objs]
     subprocess.run(link, check=True)
+    subprocess.run(_host_command(), check=True)
     return LIB_PATH
 
 

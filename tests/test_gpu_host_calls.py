@@ -1,0 +1,70 @@
+"""The compiled host side of the calls: what it refuses, which stream it launches on, what it returns."""
+import math
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _qkv(B=1, H=2, N=40, D=64, dtype=None):
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(3)
+    return [torch.randn((B, H, N, D), generator=g, device="cuda").to(dtype or torch.bfloat16) for _ in range(4)]
+
+
+def test_refuses_what_the_kernels_could_not_read():
+    import torch
+    import paper_2409_04431_b200 as sa
+    q, k, v, d_o = _qkv()
+    a = (0.125, -3.0)
+    for bad in (k.cpu(), k.float(), k[:, :, :20].contiguous(), k.transpose(1, 2), None, 3):
+        with pytest.raises(ValueError):
+            sa.sigattn_fwd(q, bad, v, *a)
+        with pytest.raises(ValueError):
+            sa.sigattn_bwd(q, k, v, bad, *a)
+    with pytest.raises(TypeError):
+        sa.sigattn_fwd(*(t.half() for t in (q, k, v)), *a)
+    with pytest.raises(ValueError):
+        sa.sigattn_fwd(q, k, v, *a, out=torch.empty_like(q, dtype=torch.float32))
+    with pytest.raises(ValueError):
+        sa.sigattn_bwd(q, k, v, d_o, *a, out=(q, k))
+    with pytest.raises(ValueError):
+        sa.sigattn_bwd(q, k, v, d_o, *a, workspace=torch.empty(1 << 20, device="cuda"))
+    with pytest.raises(sa.SigattnError) as e:
+        sa.sigattn_bwd(q, k, v, d_o, *a, workspace=torch.empty(64, dtype=torch.uint8, device="cuda"))
+    assert e.value.code == -5
+    for bias in (torch.zeros(2, device="cuda"), torch.zeros((1, 2)), torch.zeros((1, 2), dtype=torch.float64, device="cuda")):
+        with pytest.raises(ValueError):
+            sa.sigattn_fwd_gqa(q, k, v, 0.125, bias)
+    with pytest.raises(ValueError):
+        sa.sigattn_fwd_varlen(q, k, v, *a, torch.tensor([40, 40], dtype=torch.int32, device="cuda"))
+
+
+def test_outputs_and_streams():
+    """Given outputs come back as the same objects; the current stream and an explicit one (object or handle) see
+    the launches: work queued behind a long spin on that stream reads what was written before it."""
+    import torch
+    import paper_2409_04431_b200 as sa
+    q, k, v, d_o = _qkv()
+    a = (1.0 / math.sqrt(64), -math.log(40))
+    ref = sa.sigattn_fwd(q, k, v, *a)
+    out = torch.empty_like(q)
+    assert sa.sigattn_fwd(q, k, v, *a, out=out) is out and torch.equal(out, ref)
+    grads = tuple(torch.empty_like(q) for _ in range(3))
+    got = sa.sigattn_bwd(q, k, v, d_o, *a, out=grads)
+    assert all(x is y for x, y in zip(got, grads))
+    assert sa.sigattn_bwd_nk(q, k, v, d_o, *a)[3] is None
+    assert sa.sigattn_bwd_nk(q, k, v, d_o, *a, want_dbias=True)[3].shape == (1, 2)
+    side = torch.cuda.Stream()
+    for how in ("current", "object", "handle"):
+        late = torch.zeros_like(q)
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            late.add_(torch.randn(2048, 2048, device="cuda").mm(torch.randn(2048, 2048, device="cuda"))[0, 0] * 0)
+            late.copy_(q)
+            if how == "current":
+                o = sa.sigattn_fwd(late, k, v, *a)
+        if how != "current":
+            o = sa.sigattn_fwd(late, k, v, *a, stream=side if how == "object" else side.cuda_stream)
+        side.synchronize()
+        assert torch.equal(o, ref), how
