@@ -14,7 +14,8 @@ CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libsigattn.so")
 HOST_PATH = os.path.join(PKG_DIR, "_sigattn_host.so")
 SOURCES = ["sigattn_api.cu", "sigattn_fp32.cu", "sigattn_fwd_sm100.cu", "sigattn_fwd_single_sm100.cu", "sigattn_bwd_sm100.cu",
-           "sigattn_decode_sm100.cu", "sigattn_short_fwd_sm100.cu", "sigattn_static_scratch.cu", "sigattn_peer.cu"]
+           "sigattn_decode_sm100.cu", "sigattn_short_fwd_sm100.cu", "sigattn_short_bwd_sm100.cu",
+           "sigattn_static_scratch.cu", "sigattn_peer.cu"]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
     "-O3", "-std=c++17", "-lineinfo",

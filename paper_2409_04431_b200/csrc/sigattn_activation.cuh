@@ -186,4 +186,45 @@ __device__ __forceinline__ void sigmoid_cols(const uint32_t (&s)[NC], uint32_t (
   for (int i = 0; i < NC / 2; ++i) out[i] = sm100::pack_bf16x2(pr[2 * i], pr[2 * i + 1]);
 }
 
+// ------------------------------------------------------------------ backward
+
+// 32 logits (transposed tile: this thread's key against 32 queries) -> P as bf16x2 for
+// the dV product and P (1 - P) in fp32 for dS.
+//   a = log2(e) * (scale * s + b - slope * |i - j|);  u = 2^a;  P = u / (1 + u);  1 - P = 1 / (1 + u)
+// MASK: 0 no element masked, 1 causal only (queries before mask_lo), 2 both ends (padded batch)
+// CAUSAL: a query that keeps its weight sits at or after the key, so the position term is linear in the
+// query index: one FMA per logit from a per-call constant (a masked query is blanked afterwards).
+template <int MASK, bool ALIBI, bool CAUSAL>
+__device__ __forceinline__ void bwd_sigmoid_chunk(const uint32_t (&s)[32], uint32_t (&p_out)[16], float (&pp)[32],
+                                                  float scale_log2e, float bias_log2e, float slope_log2e,
+                                                  float col_rel, int q_base, float mask_lo, float mask_hi) {
+  float a[32];
+  const float c_first = fmaf(-slope_log2e, static_cast<float>(q_base) - col_rel, bias_log2e);   // query q_base
+#pragma unroll
+  for (int e = 0; e < 32; ++e) {
+    float c0 = bias_log2e;
+    if (ALIBI && CAUSAL) c0 = fmaf(-slope_log2e, static_cast<float>(e), c_first);
+    else if (ALIBI) c0 = fmaf(-slope_log2e, fabsf(static_cast<float>(q_base + e) - col_rel), bias_log2e);
+    a[e] = fmaf(__uint_as_float(s[e]), scale_log2e, c0);
+  }
+  float pr[32];
+  sigmoid_block<32, true, 0, !CAUSAL>(a, pr, pp);
+  if (MASK == 1) {
+#pragma unroll
+    for (int e = 0; e < 32; ++e)
+      if (static_cast<float>(q_base + e) < mask_lo) { pr[e] = 0.0f; pp[e] = 0.0f; }  // query before key
+  }
+  if (MASK == 2) {
+#pragma unroll
+    for (int e = 0; e < 32; ++e)
+      // query before key (causal), or, in a padded batch, past the end of the sequence
+      if (static_cast<float>(q_base + e) < mask_lo || static_cast<float>(q_base + e) >= mask_hi) {
+        pr[e] = 0.0f;
+        pp[e] = 0.0f;
+      }
+  }
+#pragma unroll
+  for (int e = 0; e < 16; ++e) p_out[e] = sm100::pack_bf16x2(pr[2 * e], pr[2 * e + 1]);
+}
+
 }  // namespace sigattn

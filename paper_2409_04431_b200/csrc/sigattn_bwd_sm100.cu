@@ -441,45 +441,6 @@ __device__ void bwd_mma_role(const BwdParams& p, uint32_t smem_base, uint32_t tm
 
 // ------------------------------------------------------------------ activation groups
 
-// 32 logits (transposed tile: this thread's key against 32 queries) -> P as bf16x2 for
-// the dV product and P (1 - P) in fp32 for dS.
-//   a = log2(e) * (scale * s + b - slope * |i - j|);  u = 2^a;  P = u / (1 + u);  1 - P = 1 / (1 + u)
-// MASK: 0 no element masked, 1 causal only (queries before mask_lo), 2 both ends (padded batch)
-// CAUSAL: a query that keeps its weight sits at or after the key, so the position term is linear in the
-// query index: one FMA per logit from a per-call constant (a masked query is blanked afterwards).
-template <int MASK, bool ALIBI, bool CAUSAL>
-__device__ __forceinline__ void bwd_sigmoid_chunk(const uint32_t (&s)[32], uint32_t (&p_out)[16], float (&pp)[32],
-                                                  float scale_log2e, float bias_log2e, float slope_log2e,
-                                                  float col_rel, int q_base, float mask_lo, float mask_hi) {
-  float a[32];
-  const float c_first = fmaf(-slope_log2e, static_cast<float>(q_base) - col_rel, bias_log2e);   // query q_base
-#pragma unroll
-  for (int e = 0; e < 32; ++e) {
-    float c0 = bias_log2e;
-    if (ALIBI && CAUSAL) c0 = fmaf(-slope_log2e, static_cast<float>(e), c_first);
-    else if (ALIBI) c0 = fmaf(-slope_log2e, fabsf(static_cast<float>(q_base + e) - col_rel), bias_log2e);
-    a[e] = fmaf(__uint_as_float(s[e]), scale_log2e, c0);
-  }
-  float pr[32];
-  sigmoid_block<32, true, 0, !CAUSAL>(a, pr, pp);
-  if (MASK == 1) {
-#pragma unroll
-    for (int e = 0; e < 32; ++e)
-      if (static_cast<float>(q_base + e) < mask_lo) { pr[e] = 0.0f; pp[e] = 0.0f; }  // query before key
-  }
-  if (MASK == 2) {
-#pragma unroll
-    for (int e = 0; e < 32; ++e)
-      // query before key (causal), or, in a padded batch, past the end of the sequence
-      if (static_cast<float>(q_base + e) < mask_lo || static_cast<float>(q_base + e) >= mask_hi) {
-        pr[e] = 0.0f;
-        pp[e] = 0.0f;
-      }
-  }
-#pragma unroll
-  for (int e = 0; e < 16; ++e) p_out[e] = pack_bf16x2(pr[2 * e], pr[2 * e + 1]);
-}
-
 // One row of a [128 x D] fp32 accumulator -> bf16 (times `mul`) -> swizzled staging tile.
 template <int D>
 __device__ __forceinline__ void bwd_store_acc_rows(uint32_t t_acc, uint8_t* stage, int tid, float mul) {
@@ -934,6 +895,13 @@ size_t bwd_bf16_workspace_bytes(int B, int H, int N, int D) {
 int launch_bwd_bf16(const void* q, const void* k, const void* v, const void* d_o, void* dq, void* dk, void* dv,
                     const Problem& p, void* workspace, int* status, cudaStream_t stream,
                     unsigned long long* launches, cudaError_t* cuda_err) {
+  if (short_bwd_serves(p)) {
+    const bool timed = (t_ev_start != nullptr && t_ev_stop != nullptr);
+    if (timed) cudaEventRecord(t_ev_start, stream);
+    const int rc = launch_short_bwd_bf16(q, k, v, d_o, dq, dk, dv, p, status, stream, launches, cuda_err);
+    if (timed && rc == SIGATTN_OK) cudaEventRecord(t_ev_stop, stream);
+    return rc;
+  }
   int dev = 0, num_sms = 0;
   *cuda_err = cudaGetDevice(&dev);
   if (*cuda_err != cudaSuccess) return SIGATTN_ERR_CUDA;

@@ -60,6 +60,11 @@ bool short_fwd_serves(const Problem& p);
 int launch_short_fwd_bf16(const void* q, const void* k, const void* v, void* o, const Problem& p, int* status,
                           cudaStream_t stream, unsigned long long* launches, cudaError_t* cuda_err);
 
+bool short_bwd_serves(const Problem& p);
+int launch_short_bwd_bf16(const void* q, const void* k, const void* v, const void* d_o, void* dq, void* dk, void* dv,
+                          const Problem& p, int* status, cudaStream_t stream, unsigned long long* launches,
+                          cudaError_t* cuda_err);
+
 // Few query rows against a cache: keys of a head divided over a cluster, no scratch (see the kernel's file).
 bool decode_kernel_serves(const Problem& p);
 int launch_decode_bf16(const void* q, const void* k, const void* v, void* o, const Problem& p, int* status,
