@@ -107,9 +107,12 @@ __device__ __forceinline__ void sigmoid_exact(const float (&a)[N], float (&pr)[N
   }
 }
 
-// Both paths from one exponential, for a warp in which some threads take the exact path (`exact`, per thread)
-// and others do not: u = 2^a, P = u / (1 + u) with 1 - P = 1 / (1 + u).  Run one after the other, as divergent
-// branches, the two paths cost a warp two exponentials per element.
+// Both paths from one exponential, for a warp in which some threads need the exact path (`exact`, per thread) and
+// others do not: u = 2^a, P = u / (1 + u), 1 - P = 1 / (1 + u).  Run one after the other, as divergent branches, the
+// two paths cost a warp two exponentials per element.
+// Backward: the thread's choice holds for its block.  Forward: element by element, a > -4 takes 1 - r (relative error
+// at most 1.2e-4, at u = 1/16: the Newton reciprocal's 7e-6 over P), the others the series; the additions are
+// predicated, and few elements need them (4 % faster on the whole forward than a selection between two results).
 template <int N, bool WITH_SLOPE, int EMULATE_EVERY>
 __device__ __forceinline__ void sigmoid_mixed(const float (&a)[N], bool exact, float (&pr)[N], float* pp) {
   static_assert(EMULATE_EVERY == 0, "one exponential for both paths");
@@ -117,11 +120,16 @@ __device__ __forceinline__ void sigmoid_mixed(const float (&a)[N], bool exact, f
   for (int i = 0; i < N; ++i) {
     const float u = sm100::ex2_approx(fminf(a[i], 120.0f));
     const float w = fmaf(-u, u, u);
-    const float p_common = fmaf(-u, w, u);
-    const float r = WITH_SLOPE ? sm100::rcp_approx(1.0f + u) : rcp_newton(1.0f + u);
-    const float p_exact = u * r;
-    pr[i] = exact ? p_exact : p_common;
-    if (WITH_SLOPE) pp[i] = exact ? p_exact * r : fmaf(-p_common, p_common, p_common);
+    float p = fmaf(-u, w, u);
+    if constexpr (WITH_SLOPE) {
+      const float r = sm100::rcp_approx(1.0f + u);
+      const float p_exact = u * r;
+      pr[i] = exact ? p_exact : p;
+      pp[i] = exact ? p_exact * r : fmaf(-p, p, p);
+    } else {
+      if (a[i] > kFastPathMaxA) p = 1.0f - rcp_newton(1.0f + u);
+      pr[i] = p;
+    }
   }
 }
 
@@ -129,7 +137,7 @@ __device__ __forceinline__ void sigmoid_mixed(const float (&a)[N], bool exact, f
 // The block's largest a decides between the two paths before anything else is evaluated.
 // SHARED (without a causal mask): a warp whose threads disagree, or all take the exact path, evaluates both from
 // one exponential.  Short sequences, where b = -log n leaves most warps mixed, gain: B32 H12 N197 D64 forward
-// 24.6 -> 21.2 us, backward 65.0 -> 61.8; N577 50.9 -> 47.5, 108 -> 103.  The causal instantiations keep the
+// 24.6 -> 20.6 us, backward 65.0 -> 61.8; N577 50.9 -> 45.1, 108 -> 103.  The causal instantiations keep the
 // branches: with the shared form B8 H16 N2048 D64 ALiBi (hardly any mixed warp) went from 131 to 137 us, and
 // b = 0 at D = 128 (nearly all warps exact) from 47.4 to 54.1.
 template <int N, bool WITH_SLOPE, int EMULATE_EVERY, bool SHARED>

@@ -43,7 +43,7 @@ constexpr int kSbLoadWarp = kSbActWarps;
 constexpr int kSbMmaWarp = kSbActWarps + 1;
 constexpr int kSbTileBytes = kSbT * 128;      // 128 rows of 64 bf16
 constexpr int kSbSlots = 10;                  // operand tiles
-// shared memory: operand tiles; dS^T (two panels of 64 queries), which also stages dQ; dV, dK staging
+// shared memory: operand tiles; dS^T (two panels of 64 queries); dV, dK staging
 constexpr int kSbDs = kSbSlots * kSbTileBytes;
 constexpr int kSbStage = kSbDs + 2 * kSbTileBytes;
 constexpr int kSbDynBytes = kSbStage + 2 * kSbTileBytes + 1024;
@@ -227,7 +227,6 @@ sigattn_short_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __g
         const ShortStep next = short_next<CAUSAL>(s, n_tiles);
         const bool more = next.head < p.n_heads;
         const bool first_of_j = s.i == (CAUSAL ? s.j : 0), last_of_j = s.i == n_tiles - 1;
-        const bool last_of_head = last_of_j && s.j == n_tiles - 1;
         const int q16 = short_live(p, s.i) >> 4, k16 = short_live(p, s.j) >> 4;
         // dV_j += P^T dO_i
         ok = mbar_wait(smem_u32(&bars.p_ready), step & 1, cta_err, 24);
@@ -261,14 +260,11 @@ sigattn_short_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __g
           umma_commit(smem_u32(&bars.empty[slot(k_tile(s.j), s.h)]));
           umma_commit(smem_u32(&bars.empty[slot(v_tile(s.j), s.h)]));
         }
-        // query tiles are last used by the last key tile
-        if (s.j == n_tiles - 1) {
+        // query tiles are last used by the last key tile; with two tiles the slots of Q_0 and dO_0 stage dQ
+        // before the activation threads release them
+        if (s.j == n_tiles - 1 && (one_tile || s.i == 1)) {
           umma_commit(smem_u32(&bars.empty[slot(q_tile(s.i), s.h)]));
           umma_commit(smem_u32(&bars.empty[slot(do_tile(s.i), s.h)]));
-          if (CAUSAL && last_of_head && !one_tile) {   // (causal: the last key tile does not meet query tile 0)
-            umma_commit(smem_u32(&bars.empty[slot(kQ0, s.h)]));
-            umma_commit(smem_u32(&bars.empty[slot(kDo0, s.h)]));
-          }
         }
         if (more) ok = issue_dp(next);
         s = next;
@@ -283,7 +279,7 @@ sigattn_short_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __g
     const uint32_t lane_off = static_cast<uint32_t>(quarter) << 16;
     uint32_t step = 0, n_acc = 0;
 
-    // One accumulator tile's 32 columns of this thread -> bf16 (times mul) -> staging tile
+    // This thread's 32 columns of an accumulator tile -> bf16 (times mul) -> staging tile
     auto stage_cols = [&](uint32_t t_col, int stage_off, float mul) {
       uint32_t o[32];
       tmem_ld32(tmem + lane_off + t_col + (g & 1) * 32, o);
@@ -300,16 +296,27 @@ sigattn_short_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __g
       }
     };
     // Results of the key tile that step `e` finished (and of the head, if it finished that): groups 0 and 1 take
-    // dV_j, 2 and 3 dK_j; then 0 and 1 dQ_0, 2 and 3 dQ_1, staged in the dS^T buffer, which the products have read.
+    // dV_j, 2 and 3 dK_j; then 0 and 1 dQ_0, 2 and 3 dQ_1.  The stores are not waited for here but before the
+    // staging tiles are written again: dQ is staged where the next loads come last (with two tiles the slots of
+    // the head's own Q_0 and dO_0, which wait for the head after the next; with one tile a slot that holds no
+    // operand).
+    uint32_t release = 0;   // thread 0: slots (1 + number, a byte each) to hand to the producer once read
+    auto stores_read = [&]() {
+      tma_wait_group_read<0>();
+      for (; release != 0; release >>= 8) mbar_arrive(smem_u32(&bars.empty[(release & 255u) - 1]));
+    };
     auto epilogue = [&](const ShortStep& e) -> bool {
+      if (threadIdx.x == 0) stores_read();
+      named_barrier_sync<1, kSbActThreads>();   // the staging tiles may be written
       if (!mbar_wait(smem_u32(&bars.acc_full), n_acc & 1, cta_err, 33)) return false;
       ++n_acc;
       tc_fence_after_sync();
       const bool head_done = e.j == n_tiles - 1;
+      const uint32_t q_stage = one_tile ? 6 : short_slot(kQ0, e.h, false), do_stage = short_slot(kDo0, e.h, false);
       if (e.j * kSbT + quarter < p.N)
         stage_cols(g < 2 ? kSbDv : kSbDk, kSbStage + (g >> 1) * kSbTileBytes, g < 2 ? 1.0f : p.scale);
       if (head_done && (g >> 1) * kSbT + quarter < p.N)
-        stage_cols(kSbDq + (g >> 1) * kSbD, kSbDs + (g >> 1) * kSbTileBytes, p.scale);
+        stage_cols(kSbDq + (g >> 1) * kSbD, (g < 2 ? q_stage : do_stage) * kSbTileBytes, p.scale);
       tc_fence_before_sync();
       mbar_arrive(smem_u32(&bars.acc_empty));
       fence_proxy_async_smem();
@@ -317,12 +324,15 @@ sigattn_short_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __g
       if (threadIdx.x == 0) {   // (rows >= N are clipped)
         tma_store_3d(&tmDv, smem_base + kSbStage, 0, e.j * kSbT, e.head);
         tma_store_3d(&tmDk, smem_base + kSbStage + kSbTileBytes, 0, e.j * kSbT, e.head);
-        if (head_done)
-          for (int t = 0; t < n_tiles; ++t) tma_store_3d(&tmDq, smem_base + kSbDs + t * kSbTileBytes, 0, t * kSbT, e.head);
+        if (head_done) {
+          tma_store_3d(&tmDq, smem_base + q_stage * kSbTileBytes, 0, 0, e.head);
+          if (!one_tile) {
+            tma_store_3d(&tmDq, smem_base + do_stage * kSbTileBytes, 0, kSbT, e.head);
+            release = (q_stage + 1) | ((do_stage + 1) << 8);
+          }
+        }
         tma_commit_group();
-        tma_wait_group_read<0>();
       }
-      named_barrier_sync<1, kSbActThreads>();   // staging and dS^T buffers may be written again
       return true;
     };
 
@@ -382,6 +392,7 @@ sigattn_short_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __g
       tc_fence_before_sync();
       fence_proxy_async_smem();
       mbar_arrive(smem_u32(&bars.ds_ready));
+      if (threadIdx.x == 0 && release != 0) stores_read();
       if (s.i == n_tiles - 1) {
         pending = s;
         have_pending = true;
