@@ -54,8 +54,11 @@ struct BwdSmem {
   // (four, which would make stage and phase a mask and a shift, measured no faster)
   static constexpr int kQStages = (D == 64) ? 3 : 2;
   static constexpr int kQOff = 2 * kTileBytes;
-  static constexpr int kDoOff = (2 + kQStages) * kTileBytes;   // one stage
-  static constexpr int kDsOff = (3 + kQStages) * kTileBytes;   // dS^T, 128 x 128 bf16 = two panels
+  // dO stages.  With one stage the next tile's load starts when dV(i) has read this one, and dP^T(i+1) waits for it:
+  // 700 to 1800 of a step's 3860 cycles at D = 64 (clock trace).  Three stages there; D = 128 has no room for more.
+  static constexpr int kDoStages = (D == 64) ? 3 : 1;
+  static constexpr int kDoOff = (2 + kQStages) * kTileBytes;
+  static constexpr int kDsOff = (2 + kQStages + kDoStages) * kTileBytes;   // dS^T, 128 x 128 bf16 = two panels
   static constexpr int kDqOff = kDsOff + 2 * kPanelBytes;   // two fp32 staging boxes of 128 x 32
   static constexpr int kTotal = kDqOff + 2 * kPanelBytes;
   static constexpr int kDynBytes = kTotal + 1024;
@@ -64,7 +67,7 @@ struct BwdSmem {
 struct BwdBarriers {
   uint64_t kv_full, kv_empty;
   uint64_t q_full[3], q_empty[3];
-  uint64_t do_full, do_empty;
+  uint64_t do_full[3], do_empty[3];
   // s_full, p_ready, dq_full, dq_empty: one per region of tensor memory that holds S^T / P^T (see BwdTmem);
   // a region's barriers flip once per use of that region
   uint64_t s_full[2], dp_full;
@@ -270,10 +273,11 @@ __device__ void bwd_load_role(const BwdParams& p, const CUtensorMap* tmQ, const 
     return true;
   };
   auto load_do = [&](int i, int bh) -> bool {
-    if (!mbar_wait(smem_u32(&bars->do_empty), (do_cnt & 1) ^ 1, cta_err, 41)) return false;
-    const uint32_t bar = smem_u32(&bars->do_full);
+    const uint32_t st = do_cnt % L::kDoStages, ph = (do_cnt / L::kDoStages) & 1;
+    if (!mbar_wait(smem_u32(&bars->do_empty[st]), ph ^ 1, cta_err, 41)) return false;
+    const uint32_t bar = smem_u32(&bars->do_full[st]);
     mbar_arrive_expect_tx(bar, L::kTileBytes);
-    load_tile(tmDo, smem_base + L::kDoOff, bar, i * kT, bh);
+    load_tile(tmDo, smem_base + L::kDoOff + st * L::kTileBytes, bar, i * kT, bh);
     ++do_cnt;
     return true;
   };
@@ -343,8 +347,8 @@ __device__ void bwd_mma_role(const BwdParams& p, uint32_t smem_base, uint32_t tm
   // Descriptors are built once; each k-step only advances the start address.
   const uint64_t dK_k = make_smem_desc_sw128(sK, 16, 1024);                 // K_j, K-major (S^T)
   const uint64_t dV_k = make_smem_desc_sw128(sV, 16, 1024);                 // V_j, K-major (dP^T)
-  const uint64_t dDo_k = make_smem_desc_sw128(sDo, 16, 1024);               // dO_i, K-major (dP^T)
-  const uint64_t dDo_mn = make_smem_desc_sw128(sDo, L::kPanelBytes, 1024);  // dO_i, MN-major (dV)
+  const uint64_t dDo_k0 = make_smem_desc_sw128(sDo, 16, 1024);               // dO_i, K-major (dP^T)
+  const uint64_t dDo_mn0 = make_smem_desc_sw128(sDo, L::kPanelBytes, 1024);  // dO_i, MN-major (dV)
   const uint64_t dK_mn = make_smem_desc_sw128(sK, L::kPanelBytes, 1024);    // K_j, MN-major (dQ)
   const uint64_t dDs_mn = make_smem_desc_sw128(sDs, L::kPanelBytes, 1024);  // dS^T, MN-major (dQ)
   // Stage 0 of Q; the other stages are reached by advancing the start address (an array indexed by the
@@ -353,6 +357,8 @@ __device__ void bwd_mma_role(const BwdParams& p, uint32_t smem_base, uint32_t tm
   const uint64_t dQ_mn0 = make_smem_desc_sw128(smem_base + L::kQOff, L::kPanelBytes, 1024);    // Q_i, MN-major (dK)
   auto q_stage = [](uint32_t cnt) -> uint32_t { return cnt % L::kQStages; };
   auto q_phase = [](uint32_t cnt) -> uint32_t { return (cnt / L::kQStages) & 1; };
+  auto do_stage = [](uint32_t cnt) -> uint32_t { return cnt % L::kDoStages; };
+  auto do_phase = [](uint32_t cnt) -> uint32_t { return (cnt / L::kDoStages) & 1; };
   // S^T of global step `step` from the Q tile with running number `qn`.  D = 64: the step's region A last
   // held dQ of two steps earlier, which the drain group must have read.
   auto issue_s = [&](uint32_t step, uint32_t qn, int where) -> bool {
@@ -367,12 +373,12 @@ __device__ void bwd_mma_role(const BwdParams& p, uint32_t smem_base, uint32_t tm
   };
   // dP^T of global step `step`.  D = 128: region B last held dQ of the step before.
   auto issue_dp = [&](uint32_t step, int where) -> bool {
-    if (!mbar_wait(smem_u32(&bars->do_full), do_cnt & 1, cta_err, where)) return false;
+    if (!mbar_wait(smem_u32(&bars->do_full[do_stage(do_cnt)]), do_phase(do_cnt), cta_err, where)) return false;
     if (!TM::kTwoA &&
         !mbar_wait(smem_u32(&bars->dq_empty[0]), (step & 1) ^ 1, cta_err, where + 20))
       return false;
     tc_fence_after_sync();
-    issue_kk(TM::kB, dV_k, dDo_k);
+    issue_kk(TM::kB, dV_k, desc_advance(dDo_k0, do_stage(do_cnt) * L::kTileBytes));
     umma_commit(smem_u32(&bars->dp_full));
     return true;
   };
@@ -400,12 +406,13 @@ __device__ void bwd_mma_role(const BwdParams& p, uint32_t smem_base, uint32_t tm
       if (!mbar_wait(smem_u32(&bars->p_ready[reg]), TM::r_use(step_cnt) & 1, cta_err, 54)) return;
       if (it == 0 && !mbar_wait(smem_u32(&bars->dkv_empty), (item_cnt & 1) ^ 1, cta_err, 55)) return;
       tc_fence_after_sync();
+      const uint64_t dDo_mn = desc_advance(dDo_mn0, do_stage(do_cnt) * L::kTileBytes);
 #pragma unroll
       for (int ks = 0; ks < kT / 16; ++ks) {
         umma_ts(tmem + TM::kDv, tmem + TM::a_col(step_cnt) + (ks >> 2) * 64 + (ks & 3) * 8,
                 desc_advance(dDo_mn, ks * 2048), kIdescAcc, (it > 0 || ks > 0));
       }
-      umma_commit(smem_u32(&bars->do_empty));
+      umma_commit(smem_u32(&bars->do_empty[do_stage(do_cnt)]));
       ++do_cnt;
       // one region A: S^T of the next query tile goes where P^T was
       if (!TM::kTwoA && it + 1 < w.steps && !issue_s(step_cnt + 1, q_cnt + 1, 56)) return;
@@ -709,9 +716,9 @@ sigattn_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     for (int s = 0; s < 3; ++s) {
       mbar_init(smem_u32(&bars.q_full[s]), 1);
       mbar_init(smem_u32(&bars.q_empty[s]), 1);
+      mbar_init(smem_u32(&bars.do_full[s]), 1);
+      mbar_init(smem_u32(&bars.do_empty[s]), 1);
     }
-    mbar_init(smem_u32(&bars.do_full), 1);
-    mbar_init(smem_u32(&bars.do_empty), 1);
     for (int s = 0; s < 2; ++s) {
       mbar_init(smem_u32(&bars.s_full[s]), 1);
       mbar_init(smem_u32(&bars.p_ready[s]), 256);
