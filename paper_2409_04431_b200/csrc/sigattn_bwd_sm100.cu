@@ -48,24 +48,28 @@ struct BwdSmem {
   static constexpr int kPanels = D / 64;
   static constexpr int kPanelBytes = kT * 128;
   static constexpr int kTileBytes = kPanels * kPanelBytes;  // a K, V, Q or dO tile
+  // K, V buffers: at D = 64 two, so that the next item's first products do not wait for this item's results to be
+  // stored (dV is staged in the V buffer, dK in the K buffer)
+  static constexpr int kKvStages = (D == 64) ? 2 : 1;
   static constexpr int kKOff = 0;
   static constexpr int kVOff = kTileBytes;
+  static constexpr int kKvBytes = 2 * kTileBytes;
   // Q stages: two at D = 128 (shared memory is full); three at D = 64, where S^T runs two steps ahead
   // (four, which would make stage and phase a mask and a shift, measured no faster)
   static constexpr int kQStages = (D == 64) ? 3 : 2;
-  static constexpr int kQOff = 2 * kTileBytes;
+  static constexpr int kQOff = kKvStages * kKvBytes;
   // dO stages.  With one stage the next tile's load starts when dV(i) has read this one, and dP^T(i+1) waits for it:
   // 700 to 1800 of a step's 3860 cycles at D = 64 (clock trace).  Three stages there; D = 128 has no room for more.
   static constexpr int kDoStages = (D == 64) ? 3 : 1;
-  static constexpr int kDoOff = (2 + kQStages) * kTileBytes;
-  static constexpr int kDsOff = (2 + kQStages + kDoStages) * kTileBytes;   // dS^T, 128 x 128 bf16 = two panels
+  static constexpr int kDoOff = (2 * kKvStages + kQStages) * kTileBytes;
+  static constexpr int kDsOff = (2 * kKvStages + kQStages + kDoStages) * kTileBytes;   // dS^T, 128 x 128 bf16 = two panels
   static constexpr int kDqOff = kDsOff + 2 * kPanelBytes;   // two fp32 staging boxes of 128 x 32
   static constexpr int kTotal = kDqOff + 2 * kPanelBytes;
   static constexpr int kDynBytes = kTotal + 1024;
 };
 
 struct BwdBarriers {
-  uint64_t kv_full, kv_empty;
+  uint64_t kv_full[2], kv_empty[2];
   uint64_t q_full[3], q_empty[3];
   uint64_t do_full[3], do_empty[3];
   // s_full, p_ready, dq_full, dq_empty: one per region of tensor memory that holds S^T / P^T (see BwdTmem);
@@ -291,16 +295,21 @@ __device__ void bwd_load_role(const BwdParams& p, const CUtensorMap* tmQ, const 
       if (item < 0) continue;
     }
     const BwdItem w = decode_bwd_item<CAUSAL, GROUPED>(p, item);
+    auto load_kv = [&]() -> bool {
+      const uint32_t st = item_cnt % L::kKvStages, ph = (item_cnt / L::kKvStages) & 1;
+      if (!mbar_wait(smem_u32(&bars->kv_empty[st]), ph ^ 1, cta_err, 42)) return false;
+      const uint32_t bar = smem_u32(&bars->kv_full[st]), dst = smem_base + st * L::kKvBytes;
+      mbar_arrive_expect_tx(bar, L::kKvBytes);
+      load_tile(tmK, dst + L::kKOff, bar, w.j * kT, w.bh);
+      load_tile(tmV, dst + L::kVOff, bar, w.j * kT, w.bh);
+      ++item_cnt;
+      return true;
+    };
+    // With one K, V buffer the first Q and dO tiles can be loaded earlier than K and V, with two later.
+    if (L::kKvStages > 1 && !load_kv()) return;
     if (!load_q(w.i_begin, w.bh_q0)) return;
     if (!load_do(w.i_begin, w.bh_q0)) return;
-    if (!mbar_wait(smem_u32(&bars->kv_empty), (item_cnt & 1) ^ 1, cta_err, 42)) return;
-    {
-      const uint32_t bar = smem_u32(&bars->kv_full);
-      mbar_arrive_expect_tx(bar, 2 * L::kTileBytes);
-      load_tile(tmK, smem_base + L::kKOff, bar, w.j * kT, w.bh);
-      load_tile(tmV, smem_base + L::kVOff, bar, w.j * kT, w.bh);
-    }
-    ++item_cnt;
+    if (L::kKvStages == 1 && !load_kv()) return;
     // The remaining steps, head by head.  With two regions A (D = 64) S^T runs a step further ahead than
     // dP^T, so Q stays one tile ahead of dO: dO(s) can only be loaded after dV(s-1), and S^T(s+1) is issued
     // before that product's inputs exist.
@@ -345,11 +354,11 @@ __device__ void bwd_mma_role(const BwdParams& p, uint32_t smem_base, uint32_t tm
     }
   };
   // Descriptors are built once; each k-step only advances the start address.
-  const uint64_t dK_k = make_smem_desc_sw128(sK, 16, 1024);                 // K_j, K-major (S^T)
-  const uint64_t dV_k = make_smem_desc_sw128(sV, 16, 1024);                 // V_j, K-major (dP^T)
+  const uint64_t dK_k0 = make_smem_desc_sw128(sK, 16, 1024);                // K_j, K-major (S^T)
+  const uint64_t dV_k0 = make_smem_desc_sw128(sV, 16, 1024);                // V_j, K-major (dP^T)
   const uint64_t dDo_k0 = make_smem_desc_sw128(sDo, 16, 1024);               // dO_i, K-major (dP^T)
   const uint64_t dDo_mn0 = make_smem_desc_sw128(sDo, L::kPanelBytes, 1024);  // dO_i, MN-major (dV)
-  const uint64_t dK_mn = make_smem_desc_sw128(sK, L::kPanelBytes, 1024);    // K_j, MN-major (dQ)
+  const uint64_t dK_mn0 = make_smem_desc_sw128(sK, L::kPanelBytes, 1024);   // K_j, MN-major (dQ)
   const uint64_t dDs_mn = make_smem_desc_sw128(sDs, L::kPanelBytes, 1024);  // dS^T, MN-major (dQ)
   // Stage 0 of Q; the other stages are reached by advancing the start address (an array indexed by the
   // stage at run time would live in local memory, and this thread pays for every load in full)
@@ -359,6 +368,7 @@ __device__ void bwd_mma_role(const BwdParams& p, uint32_t smem_base, uint32_t tm
   auto q_phase = [](uint32_t cnt) -> uint32_t { return (cnt / L::kQStages) & 1; };
   auto do_stage = [](uint32_t cnt) -> uint32_t { return cnt % L::kDoStages; };
   auto do_phase = [](uint32_t cnt) -> uint32_t { return (cnt / L::kDoStages) & 1; };
+  auto kv_off = [&]() -> uint32_t { return (item_cnt % L::kKvStages) * L::kKvBytes; };   // this item's buffer
   // S^T of global step `step` from the Q tile with running number `qn`.  D = 64: the step's region A last
   // held dQ of two steps earlier, which the drain group must have read.
   auto issue_s = [&](uint32_t step, uint32_t qn, int where) -> bool {
@@ -367,7 +377,7 @@ __device__ void bwd_mma_role(const BwdParams& p, uint32_t smem_base, uint32_t tm
         !mbar_wait(smem_u32(&bars->dq_empty[TM::r_index(step)]), (TM::r_use(step) & 1) ^ 1, cta_err, where + 20))
       return false;
     tc_fence_after_sync();
-    issue_kk(TM::a_col(step), dK_k, desc_advance(dQ_k0, q_stage(qn) * L::kTileBytes));
+    issue_kk(TM::a_col(step), desc_advance(dK_k0, kv_off()), desc_advance(dQ_k0, q_stage(qn) * L::kTileBytes));
     umma_commit(smem_u32(&bars->s_full[TM::r_index(step)]));
     return true;
   };
@@ -378,7 +388,7 @@ __device__ void bwd_mma_role(const BwdParams& p, uint32_t smem_base, uint32_t tm
         !mbar_wait(smem_u32(&bars->dq_empty[0]), (step & 1) ^ 1, cta_err, where + 20))
       return false;
     tc_fence_after_sync();
-    issue_kk(TM::kB, dV_k, desc_advance(dDo_k0, do_stage(do_cnt) * L::kTileBytes));
+    issue_kk(TM::kB, desc_advance(dV_k0, kv_off()), desc_advance(dDo_k0, do_stage(do_cnt) * L::kTileBytes));
     umma_commit(smem_u32(&bars->dp_full));
     return true;
   };
@@ -393,7 +403,8 @@ __device__ void bwd_mma_role(const BwdParams& p, uint32_t smem_base, uint32_t tm
       if (item < 0) continue;
     }
     const BwdItem w = decode_bwd_item<CAUSAL, GROUPED>(p, item);
-    if (!mbar_wait(smem_u32(&bars->kv_full), item_cnt & 1, cta_err, 50)) return;
+    if (!mbar_wait(smem_u32(&bars->kv_full[item_cnt % L::kKvStages]), (item_cnt / L::kKvStages) & 1, cta_err, 50)) return;
+    const uint64_t dK_mn = desc_advance(dK_mn0, kv_off());
 
     // prologue: S^T(0), dP^T(0) and, with two regions A, S^T(1)
     if (!issue_s(step_cnt, q_cnt, 51)) return;
@@ -603,9 +614,10 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
 
     // epilogue: group 0 stores dV_j (staged in the V tile), group 1 stores scale * dK_j (K tile)
     if (!mbar_wait(smem_u32(&bars->dkv_full), item_cnt & 1, cta_err, 64 + wg)) return;
+    const uint32_t kv_stage = item_cnt % L::kKvStages;
     ++item_cnt;
     tc_fence_after_sync();
-    uint8_t* stage = smem + (wg == 0 ? L::kVOff : L::kKOff);
+    uint8_t* stage = smem + kv_stage * L::kKvBytes + (wg == 0 ? L::kVOff : L::kKOff);
     bwd_store_acc_rows<D>(tmem + (wg == 0 ? TM::kDv : TM::kDk) + lane_off, stage, tid, wg == 0 ? 1.0f : p.scale);
     tc_fence_before_sync();
     mbar_arrive(smem_u32(&bars->dkv_empty));
@@ -621,7 +633,7 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
           tma_store_3d(tm, smem_u32(stage + pn * L::kPanelBytes), pn * 64, w.j * kT, w.bh);
       tma_commit_group();
       tma_wait_group_read<0>();
-      mbar_arrive(smem_u32(&bars->kv_empty));
+      mbar_arrive(smem_u32(&bars->kv_empty[kv_stage]));
     }
   }
   if (tid == 0) tma_wait_group<0>();
@@ -711,8 +723,10 @@ sigattn_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 
   if (threadIdx.x == 0) {
     cta_err = 0;
-    mbar_init(smem_u32(&bars.kv_full), 1);
-    mbar_init(smem_u32(&bars.kv_empty), 2);
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(smem_u32(&bars.kv_full[s]), 1);
+      mbar_init(smem_u32(&bars.kv_empty[s]), 2);
+    }
     for (int s = 0; s < 3; ++s) {
       mbar_init(smem_u32(&bars.q_full[s]), 1);
       mbar_init(smem_u32(&bars.q_empty[s]), 1);
