@@ -105,6 +105,7 @@ struct BwdParams {
   int i_split;
   int dkv_add;   // 1: dK_j, dV_j are added (bf16 TMA reduce-adds) into outputs the caller cleared: several calls sum up
   int n_items;
+  int head_group;  // (batch, key/value head) pairs whose items are handed out together
   float scale, scale_log2e, bias_log2e;
   const float* bias_vec;   // one bias per (batch, head) instead of the scalar, or nullptr
   float* dbias;            // receives sum dS per (batch, head), or nullptr
@@ -132,11 +133,11 @@ __device__ __forceinline__ int bwd_snake_rank(int round, int n_items) {
 
 __device__ __forceinline__ int bwd_num_rounds(int n_items) { return (n_items + gridDim.x - 1) / gridDim.x; }
 
-// Dynamic schedule for batches without padding, where an item's cost follows the position of its
-// key tile inside its own sequence and the static order above no longer sorts by cost: the CTAs
-// draw items from a global counter in key-tile order (every sequence hands out its expensive key
-// tiles first).  One thread per CTA draws; the MMA thread, the activation groups and the drain
-// group read the item from a two-slot ring.  false: a bounded wait expired; *item < 0: none left.
+// Dynamic schedule: the CTAs draw items from a global counter in the order of their numbers.  Used where the static
+// order above does not sort by cost: in batches without padding, where the cost follows the position of the key tile
+// inside its own sequence, and when heads are handed out in groups.  One thread per CTA draws; the MMA thread, the
+// activation groups and the drain group read the item from a two-slot ring.  false: a bounded wait expired;
+// *item < 0: none left.
 constexpr int kBwdSchedConsumers = 1 + 256 + 128;
 __device__ __forceinline__ bool bwd_sched_draw(const BwdParams& p, BwdBarriers* bars, int round, int* item,
                                                volatile int* cta_err) {
@@ -177,24 +178,19 @@ __device__ __forceinline__ int bwd_seq_of_row(const int* __restrict__ cu, int n_
 template <bool CAUSAL, bool GROUPED>
 __device__ __forceinline__ BwdItem decode_bwd_item(const BwdParams& p, int item) {
   BwdItem w;
-  w.j = item / p.BH;  // ascending key tile = descending work when causal
-  w.bh = item - w.j * p.BH;
-  int sub = 0;
-  if (GROUPED && p.n_sub > 1) {   // item = (key tile, key/value head, part of its query heads)
-    const int per_j = p.BH * p.n_sub;
-    w.j = item / per_j;
-    const int r = item - w.j * per_j;
-    w.bh = r / p.n_sub;
-    sub = r - w.bh * p.n_sub;
-  }
-  int part = 0;
-  if (GROUPED && p.i_split > 1) {   // item = (key tile, head, half of its query tiles)
-    const int per_j = p.BH * 2;
-    w.j = item / per_j;
-    const int r = item - w.j * per_j;
-    w.bh = r >> 1;
-    part = r & 1;
-  }
+  // Items are numbered group of heads by group of heads (see the launcher; one group = all heads), within a group by
+  // ascending key tile = descending work when causal, then head, then part.
+  const int parts = GROUPED ? (p.n_sub > 1 ? p.n_sub : p.i_split) : 1;
+  const int per_group = p.head_group * p.n_tiles_k * parts;
+  const int g0 = item / per_group * p.head_group;
+  const int per_tile = min(p.head_group, p.BH - g0) * parts;
+  int r = item - g0 * p.n_tiles_k * parts;
+  w.j = r / per_tile;
+  r -= w.j * per_tile;
+  w.bh = g0 + (GROUPED ? r / parts : r);
+  const int of_parts = GROUPED ? r - (w.bh - g0) * parts : 0;
+  const int sub = (GROUPED && p.n_sub > 1) ? of_parts : 0;     // part of the query heads of a key/value head
+  const int part = (GROUPED && p.i_split > 1) ? of_parts : 0;  // half of the query tiles
   w.bh_q0 = GROUPED ? (w.bh / p.H_kv) * p.H + (w.bh % p.H_kv) * p.group + sub * p.heads_per_sub : w.bh;
   // causal: the first query tile whose last row, at position 128 i + 127 + pos0, reaches key 128 j
   // padded batch: query tiles past the sequence's end are not visited at all
@@ -257,7 +253,7 @@ struct BwdTmem {
 
 // ------------------------------------------------------------------ producer
 
-template <int D, bool CAUSAL, bool GROUPED, bool DYNAMIC>
+template <int D, bool CAUSAL, bool GROUPED>
 __device__ void bwd_load_role(const BwdParams& p, const CUtensorMap* tmQ, const CUtensorMap* tmK,
                               const CUtensorMap* tmV, const CUtensorMap* tmDo, uint32_t smem_base,
                               BwdBarriers* bars, volatile int* cta_err) {
@@ -285,9 +281,10 @@ __device__ void bwd_load_role(const BwdParams& p, const CUtensorMap* tmQ, const 
     ++do_cnt;
     return true;
   };
-  for (int round = 0, rounds = bwd_num_rounds(p.n_items); DYNAMIC || round < rounds; ++round) {
+  const bool dynamic = p.sched_counter != nullptr;
+  for (int round = 0, rounds = bwd_num_rounds(p.n_items); dynamic || round < rounds; ++round) {
     int item;
-    if (DYNAMIC) {
+    if (dynamic) {
       if (!bwd_sched_draw(p, bars, round, &item, cta_err)) return;
       if (item < 0) break;
     } else {
@@ -333,7 +330,7 @@ __device__ void bwd_load_role(const BwdParams& p, const CUtensorMap* tmQ, const 
 // a single thread is active, and every product costs the thread more.  Measured, whole backward, us:
 // B8 H12 N4096 D64 1540 -> 1385, B8 H16 N2048 D64 causal ALiBi 353 -> 331, B2 H16 N4096 D128 causal 389 -> 387.
 // (The role run by the whole warp with an election per batch of products: 1405, 339, 392.)
-template <int D, bool CAUSAL, bool GROUPED, bool DYNAMIC>
+template <int D, bool CAUSAL, bool GROUPED>
 __device__ void bwd_mma_role(const BwdParams& p, uint32_t smem_base, uint32_t tmem, BwdBarriers* bars,
                              volatile int* cta_err) {
   using L = BwdSmem<D>;
@@ -393,9 +390,10 @@ __device__ void bwd_mma_role(const BwdParams& p, uint32_t smem_base, uint32_t tm
     return true;
   };
 
-  for (int round = 0, rounds = bwd_num_rounds(p.n_items); DYNAMIC || round < rounds; ++round) {
+  const bool dynamic = p.sched_counter != nullptr;
+  for (int round = 0, rounds = bwd_num_rounds(p.n_items); dynamic || round < rounds; ++round) {
     int item;
-    if (DYNAMIC) {
+    if (dynamic) {
       if (!bwd_sched_take(bars, round, &item, cta_err)) return;
       if (item < 0) break;
     } else {
@@ -488,14 +486,15 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
                              uint8_t* smem, uint32_t tmem, BwdBarriers* bars, volatile int* cta_err) {
   using L = BwdSmem<D>;
   using TM = BwdTmem<D>;
-  constexpr bool GROUPED = KIND >= 1, DYNAMIC = KIND == 2;
+  constexpr bool GROUPED = KIND >= 1;
   const int tid = threadIdx.x & 127;  // key row within the tile
   const uint32_t lane_off = static_cast<uint32_t>(((threadIdx.x >> 5) & 3) * 32) << 16;
   uint32_t step_cnt = 0, item_cnt = 0;
 
-  for (int round = 0, rounds = bwd_num_rounds(p.n_items); DYNAMIC || round < rounds; ++round) {
+  const bool dynamic = p.sched_counter != nullptr;
+  for (int round = 0, rounds = bwd_num_rounds(p.n_items); dynamic || round < rounds; ++round) {
     int item;
-    if (DYNAMIC) {
+    if (dynamic) {
       if (!bwd_sched_take(bars, round, &item, cta_err)) return;
       if (item < 0) break;
     } else {
@@ -641,7 +640,7 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
 
 // ------------------------------------------------------------------ dQ drain group
 
-template <int D, bool CAUSAL, bool GROUPED, bool DYNAMIC>
+template <int D, bool CAUSAL, bool GROUPED>
 __device__ void bwd_drain_role(const BwdParams& p, const CUtensorMap* tmW, uint8_t* smem, uint32_t tmem,
                                BwdBarriers* bars, volatile int* cta_err) {
   using L = BwdSmem<D>;
@@ -649,9 +648,10 @@ __device__ void bwd_drain_role(const BwdParams& p, const CUtensorMap* tmW, uint8
   const int tid = threadIdx.x & 127;  // query row within the tile
   const uint32_t lane_off = static_cast<uint32_t>(((threadIdx.x >> 5) & 3) * 32) << 16;
   uint32_t step_cnt = 0;
-  for (int round = 0, rounds = bwd_num_rounds(p.n_items); DYNAMIC || round < rounds; ++round) {
+  const bool dynamic = p.sched_counter != nullptr;
+  for (int round = 0, rounds = bwd_num_rounds(p.n_items); dynamic || round < rounds; ++round) {
     int item;
-    if (DYNAMIC) {
+    if (dynamic) {
       if (!bwd_sched_take(bars, round, &item, cta_err)) return;
       if (item < 0) break;
     } else {
@@ -768,15 +768,15 @@ sigattn_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   const uint32_t tmem = tmem_base_slot;
 
   if (warp == kBwdLoadWarp) {
-    if ((threadIdx.x & 31) == 0) bwd_load_role<D, CAUSAL, GROUPED, KIND == 2>(p, &tmQ, &tmK, &tmV, &tmDo, smem_base, &bars, &cta_err);
+    if ((threadIdx.x & 31) == 0) bwd_load_role<D, CAUSAL, GROUPED>(p, &tmQ, &tmK, &tmV, &tmDo, smem_base, &bars, &cta_err);
     __syncwarp();
   } else if (warp == kBwdMmaWarp) {
-    if (elect_one()) bwd_mma_role<D, CAUSAL, GROUPED, KIND == 2>(p, smem_base, tmem, &bars, &cta_err);
+    if (elect_one()) bwd_mma_role<D, CAUSAL, GROUPED>(p, smem_base, tmem, &bars, &cta_err);
     __syncwarp();
   } else if (warp < 8) {
     bwd_act_role<D, CAUSAL, ALIBI, DBIAS, KIND>(p, &tmDk, &tmDv, warp >> 2, smem, tmem, &bars, &cta_err);
   } else {
-    bwd_drain_role<D, CAUSAL, GROUPED, KIND == 2>(p, &tmW, smem, tmem, &bars, &cta_err);
+    bwd_drain_role<D, CAUSAL, GROUPED>(p, &tmW, smem, tmem, &bars, &cta_err);
   }
 
   tc_fence_before_sync();
@@ -852,6 +852,9 @@ sigattn_bwd_scale_rows_kernel(const uint4* __restrict__ d_o, const float* __rest
     out[i] = make_uint4(scale_bf16x2(x.x, r), scale_bf16x2(x.y, r), scale_bf16x2(x.z, r), scale_bf16x2(x.w, r));
   }
 }
+
+// What the items in work at a time may touch of Q, dO and the dQ accumulator.
+constexpr size_t kBwdL2Share = 64u << 20;
 
 // Work-item counters of the dynamic schedule: one per launch in flight, handed out round robin.
 constexpr int kBwdSchedSlots = 1024;
@@ -1015,7 +1018,25 @@ int launch_bwd_bf16(const void* q, const void* k, const void* v, const void* d_o
     if (*cuda_err != cudaSuccess) return SIGATTN_ERR_CUDA;
   }
 
-  if (p.cu_seqlens != nullptr) {
+  // Which heads are in work at a time.  Every item of a head reads the head's Q and dO and adds to its fp32 dQ
+  // (8 N D bytes a head), so what all running items touch should stay in L2 (126 MB): heads are handed out in groups
+  // of about 64 MB, drawn dynamically (the costs then fall group by group).  Long sequences run at the power limit,
+  // where every byte that does not go to HBM is time.  Whole backward in a sustained loop, us, all heads at once /
+  // groups of 128, 64, 32, 16 MB:
+  //   B1 H32 N16384 D128 causal (512 MB)   7250 / 6040  5960  5970  6040
+  //   B8 H12 N4096 D64 (192 MB)            1640 / 1410  1320  1305  1305
+  //   B8 H16 N2048 D64 causal ALiBi (128)   322 /        310   311   314
+  //   B2 H16 N4096 D128 causal (128)        455 /        441   444   445
+  // A padded batch touches less than its shape says, and its items' costs differ: groups pay from about three times
+  // that on (lengths N/4 to N, D64: B32 H16 N2500, 625 MB, 2300 -> 1970; B32 H8 N1500, 187 MB, 495 -> 505).
+  // (Packed documents have their own locality: the key tiles in work belong to a few documents.)
+  const size_t head_bytes = static_cast<size_t>(bp.group) * p.N * p.D * 8;
+  bp.head_group = bp.BH;
+  if (p.cu_seqlens == nullptr && head_bytes * bp.BH > (p.seqlens != nullptr ? 3 * kBwdL2Share : kBwdL2Share)) {
+    const size_t heads = kBwdL2Share / head_bytes;
+    if (heads < static_cast<size_t>(bp.BH)) bp.head_group = heads < 1 ? 1 : static_cast<int>(heads);
+  }
+  if (p.cu_seqlens != nullptr || bp.head_group < bp.BH) {
     static std::atomic<unsigned> next_slot{0};
     int* counters = nullptr;
     *cuda_err = cudaGetSymbolAddress(reinterpret_cast<void**>(&counters), g_bwd_sched_counters);
