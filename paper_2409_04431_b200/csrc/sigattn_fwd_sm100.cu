@@ -123,6 +123,7 @@ struct FwdParams {
   float* split_ws;
   int o_reduce;    // 1: split items of the unpacked general mode add bf16 tiles into O instead of storing them
   int n_items;
+  int head_group;  // heads whose items are handed out together
   float scale_log2e, bias_log2e;
   const float* bias_vec;   // one bias per (batch, head) instead of the scalar, or nullptr
   const float* slopes;
@@ -148,8 +149,8 @@ __device__ __forceinline__ int snake_rank(int round, int n_items) {
 
 __device__ __forceinline__ int num_rounds(int n_items) { return (n_items + gridDim.x - 1) / gridDim.x; }
 
-// Dynamic schedule.  The static snake order balances the CTAs only if the items' costs fall with
-// their rank.  In a padded batch the cost of an item also depends on the length of its sequence,
+// Dynamic schedule (used when the launcher gives a counter).  The static snake order balances the CTAs only if the
+// items' costs fall with their rank.  In a padded batch the cost of an item also depends on the length of its sequence,
 // and in a batch without padding the cost of a causal item follows its position inside its own
 // sequence, a sawtooth over the rows.  The general instantiations therefore draw their items from
 // a global counter instead, in row order from the last row down (every sequence then hands out
@@ -194,8 +195,13 @@ __device__ __forceinline__ int seq_of_row(const int* __restrict__ cu, int n_seqs
 template <bool CAUSAL>
 __device__ __forceinline__ Item decode_item(const FwdParams& p, int item) {
   Item w;
-  int rank = item / p.BH;
-  w.bh = item - rank * p.BH;
+  // Items are numbered group of heads by group of heads (one group = all heads unless the launcher says otherwise),
+  // within a group by decreasing cost, then head.
+  const int g0 = item / (p.head_group * p.n_pairs * p.n_splits) * p.head_group;
+  const int gn = min(p.head_group, p.BH - g0);
+  const int in_group = item - g0 * p.n_pairs * p.n_splits;
+  int rank = in_group / gn;
+  w.bh = g0 + in_group - rank * gn;
   const int split = rank / p.n_pairs;   // 0 unless the keys are split
   rank -= split * p.n_pairs;
   const int pair = CAUSAL ? (p.n_pairs - 1 - rank) : rank;
@@ -264,15 +270,16 @@ __device__ __forceinline__ Item decode_item(const FwdParams& p, int item) {
 
 // ------------------------------------------------------------------ producer
 
-template <int D, bool CAUSAL, bool DYNAMIC>
+template <int D, bool CAUSAL>
 __device__ void fwd_load_role(const FwdParams& p, const CUtensorMap* tmQ, const CUtensorMap* tmK,
                               const CUtensorMap* tmV, uint32_t smem_base, FwdBarriers* bars, volatile int* cta_err) {
   using L = FwdSmem<D>;
   uint32_t kv_cnt = 0;
   uint32_t q_iter[2] = {0, 0};
-  for (int round = 0, rounds = num_rounds(p.n_items); DYNAMIC || round < rounds; ++round) {
+  const bool dynamic = p.sched_counter != nullptr;
+  for (int round = 0, rounds = num_rounds(p.n_items); dynamic || round < rounds; ++round) {
     int item;
-    if (DYNAMIC) {
+    if (dynamic) {
       if (!sched_draw(p, bars, round, &item, cta_err)) return;
       if (item < 0) break;
     } else {
@@ -323,7 +330,7 @@ __device__ void fwd_load_role(const FwdParams& p, const CUtensorMap* tmQ, const 
 // thread is active and feeds the products' descriptors to the tensor pipe directly.  Measured against the
 // predicated form, forward, us: B8 H16 N2048 D64 causal ALiBi 142 -> 134, B8 H12 N4096 D64 620-650 -> 597-607,
 // B2 H16 N4096 D128 causal 134 -> 132.
-template <int D, bool CAUSAL, bool DYNAMIC>
+template <int D, bool CAUSAL>
 __device__ void fwd_mma_role(const FwdParams& p, uint32_t smem_base, uint32_t tmem, FwdBarriers* bars,
                              volatile int* cta_err) {
   using L = FwdSmem<D>;
@@ -365,9 +372,10 @@ __device__ void fwd_mma_role(const FwdParams& p, uint32_t smem_base, uint32_t tm
   auto kv_addr = [&](uint32_t cnt) { return smem_base + L::kKvOff + (cnt % L::kStages) * L::kTileBytes; };
   auto kv_release = [&](uint32_t cnt) { umma_commit(smem_u32(&bars->kv_empty[cnt % L::kStages])); };
 
-  for (int round = 0, rounds = num_rounds(p.n_items); DYNAMIC || round < rounds; ++round) {
+  const bool dynamic = p.sched_counter != nullptr;
+  for (int round = 0, rounds = num_rounds(p.n_items); dynamic || round < rounds; ++round) {
     int item;
-    if (DYNAMIC) {
+    if (dynamic) {
       if (!sched_take(bars, round, &item, cta_err)) return;
       if (item < 0) break;
     } else {
@@ -475,10 +483,10 @@ __device__ void fwd_act_role(const FwdParams& p, const CUtensorMap* tmO, uint8_t
   const uint32_t lane_off = static_cast<uint32_t>(((threadIdx.x >> 5) & 3) * 32) << 16;
   uint32_t s_cnt0 = 0, s_cnt1 = 0, it[2] = {0, 0};
 
-  constexpr bool DYNAMIC = (MODE >= 2);
-  for (int round = 0, rounds = num_rounds(p.n_items); DYNAMIC || round < rounds; ++round) {
+  const bool dynamic = p.sched_counter != nullptr;
+  for (int round = 0, rounds = num_rounds(p.n_items); dynamic || round < rounds; ++round) {
     int item;
-    if (DYNAMIC) {
+    if (dynamic) {
       if (!sched_take(bars, round, &item, cta_err)) return;
       if (item < 0) break;
     } else {
@@ -707,10 +715,10 @@ sigattn_fwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   const uint32_t tmem = tmem_base_slot;
 
   if (warp == kLoadWarp) {
-    if ((threadIdx.x & 31) == 0) fwd_load_role<D, CAUSAL, MODE >= 2>(p, &tmQ, &tmK, &tmV, smem_base, &bars, &cta_err);
+    if ((threadIdx.x & 31) == 0) fwd_load_role<D, CAUSAL>(p, &tmQ, &tmK, &tmV, smem_base, &bars, &cta_err);
     __syncwarp();
   } else if (warp == kMmaWarp) {
-    if (elect_one()) fwd_mma_role<D, CAUSAL, MODE >= 2>(p, smem_base, tmem, &bars, &cta_err);
+    if (elect_one()) fwd_mma_role<D, CAUSAL>(p, smem_base, tmem, &bars, &cta_err);
     __syncwarp();
   } else {
     fwd_act_role<D, CAUSAL, ALIBI, MODE>(p, &tmO, smem, tmem, &bars, &cta_err);
@@ -775,6 +783,10 @@ int choose_key_splits(int base_items, int n_kv, int num_sms) {
 // (1024 launches may overlap on different streams before two of them share a counter; a kernel that
 // sees its counter run past what one launch can draw sets the device status word).
 constexpr int kSchedSlots = 1024;
+
+// K and V of all heads beyond which heads are handed out in groups, and of one group.
+constexpr size_t kFwdL2Most = 80u << 20, kFwdL2Share = 32u << 20;
+
 __device__ int g_fwd_sched_counters[kSchedSlots];
 #endif
 
@@ -834,6 +846,7 @@ int launch_fwd_bf16_single(const void* q, const void* k, const void* v, void* o,
   fp.n_splits = 1;
   fp.tiles_per_split = fp.n_kv_total;
   fp.n_items = fp.n_pairs * fp.BH;
+  fp.head_group = fp.BH;
   fp.scale_log2e = p.scale * kLog2e;
   fp.bias_log2e = p.bias * kLog2e;
   fp.bias_vec = p.bias_vec;
@@ -949,7 +962,23 @@ int launch_fwd_bf16(const void* q, const void* k, const void* v, void* o, const 
                                    o_splits > 1);
   if (!packed && !general && fwd_single_tile_shape(p, num_sms))
     return launch_fwd_bf16_single(q, k, v, o, p, status, stream, launches, cuda_err);
-  if (general) {   // the general instantiations draw their work items from a counter
+  // Which heads are in work at a time.  Every item of a head reads the head's K and V (4 N_k D bytes), so those of all
+  // running items should stay in L2 (126 MB, shared with Q and O passing through): heads are handed out in groups
+  // of about 32 MB, drawn dynamically, once all of them together exceed 80 MB (a padded batch, which touches less
+  // than its shape says: three times that).  In a sustained loop, at the power limit, us, all heads at once / groups
+  // of 67, 33, 17, 8 MB:
+  //   B1 H32 N16384 D128 causal (268 MB)  2170 / 2030  2000  2050
+  //   B8 H12 N4096 D64 (100 MB)            645 /  606   584   585   588
+  //   B2 H16 N4096 D128 causal (67)        150 /        150   152   167
+  //   B8 H16 N2048 D64 causal ALiBi (67)   130 /  135   136   136   144
+  fp.head_group = fp.BH;
+  const size_t kv_bytes = static_cast<size_t>(p.key_rows()) * p.D * 4;
+  if (!packed && p.cu_seqlens == nullptr && fp.n_splits == 1 &&
+      kv_bytes * BH_kv > (p.seqlens != nullptr ? 3 * kFwdL2Most : kFwdL2Most)) {
+    const size_t heads = kv_bytes < kFwdL2Share ? kFwdL2Share / kv_bytes * group : group;
+    if (heads < BH) fp.head_group = static_cast<int>(heads);
+  }
+  if (general || fp.head_group < fp.BH) {   // (the general instantiations always draw their work items from a counter)
     static std::atomic<unsigned> next_slot{0};
     int* counters = nullptr;
     *cuda_err = cudaGetSymbolAddress(reinterpret_cast<void**>(&counters), g_fwd_sched_counters);
