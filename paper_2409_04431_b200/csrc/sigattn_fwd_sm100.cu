@@ -270,13 +270,13 @@ __device__ __forceinline__ Item decode_item(const FwdParams& p, int item) {
 
 // ------------------------------------------------------------------ producer
 
-template <int D, bool CAUSAL>
+template <int D, bool CAUSAL, bool GENERAL>   // GENERAL: always dynamic
 __device__ void fwd_load_role(const FwdParams& p, const CUtensorMap* tmQ, const CUtensorMap* tmK,
                               const CUtensorMap* tmV, uint32_t smem_base, FwdBarriers* bars, volatile int* cta_err) {
   using L = FwdSmem<D>;
   uint32_t kv_cnt = 0;
   uint32_t q_iter[2] = {0, 0};
-  const bool dynamic = p.sched_counter != nullptr;
+  const bool dynamic = GENERAL || p.sched_counter != nullptr;
   for (int round = 0, rounds = num_rounds(p.n_items); dynamic || round < rounds; ++round) {
     int item;
     if (dynamic) {
@@ -330,7 +330,7 @@ __device__ void fwd_load_role(const FwdParams& p, const CUtensorMap* tmQ, const 
 // thread is active and feeds the products' descriptors to the tensor pipe directly.  Measured against the
 // predicated form, forward, us: B8 H16 N2048 D64 causal ALiBi 142 -> 134, B8 H12 N4096 D64 620-650 -> 597-607,
 // B2 H16 N4096 D128 causal 134 -> 132.
-template <int D, bool CAUSAL>
+template <int D, bool CAUSAL, bool GENERAL>
 __device__ void fwd_mma_role(const FwdParams& p, uint32_t smem_base, uint32_t tmem, FwdBarriers* bars,
                              volatile int* cta_err) {
   using L = FwdSmem<D>;
@@ -372,7 +372,7 @@ __device__ void fwd_mma_role(const FwdParams& p, uint32_t smem_base, uint32_t tm
   auto kv_addr = [&](uint32_t cnt) { return smem_base + L::kKvOff + (cnt % L::kStages) * L::kTileBytes; };
   auto kv_release = [&](uint32_t cnt) { umma_commit(smem_u32(&bars->kv_empty[cnt % L::kStages])); };
 
-  const bool dynamic = p.sched_counter != nullptr;
+  const bool dynamic = GENERAL || p.sched_counter != nullptr;
   for (int round = 0, rounds = num_rounds(p.n_items); dynamic || round < rounds; ++round) {
     int item;
     if (dynamic) {
@@ -483,7 +483,7 @@ __device__ void fwd_act_role(const FwdParams& p, const CUtensorMap* tmO, uint8_t
   const uint32_t lane_off = static_cast<uint32_t>(((threadIdx.x >> 5) & 3) * 32) << 16;
   uint32_t s_cnt0 = 0, s_cnt1 = 0, it[2] = {0, 0};
 
-  const bool dynamic = p.sched_counter != nullptr;
+  const bool dynamic = GENERAL || p.sched_counter != nullptr;
   for (int round = 0, rounds = num_rounds(p.n_items); dynamic || round < rounds; ++round) {
     int item;
     if (dynamic) {
@@ -715,10 +715,10 @@ sigattn_fwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   const uint32_t tmem = tmem_base_slot;
 
   if (warp == kLoadWarp) {
-    if ((threadIdx.x & 31) == 0) fwd_load_role<D, CAUSAL>(p, &tmQ, &tmK, &tmV, smem_base, &bars, &cta_err);
+    if ((threadIdx.x & 31) == 0) fwd_load_role<D, CAUSAL, (MODE >= 2)>(p, &tmQ, &tmK, &tmV, smem_base, &bars, &cta_err);
     __syncwarp();
   } else if (warp == kMmaWarp) {
-    if (elect_one()) fwd_mma_role<D, CAUSAL>(p, smem_base, tmem, &bars, &cta_err);
+    if (elect_one()) fwd_mma_role<D, CAUSAL, (MODE >= 2)>(p, smem_base, tmem, &bars, &cta_err);
     __syncwarp();
   } else {
     fwd_act_role<D, CAUSAL, ALIBI, MODE>(p, &tmO, smem, tmem, &bars, &cta_err);
