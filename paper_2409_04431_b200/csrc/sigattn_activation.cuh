@@ -133,22 +133,51 @@ __device__ __forceinline__ void sigmoid_mixed(const float (&a)[N], bool exact, f
   }
 }
 
+// The same for warps of causal kernels, with the results of the divergent branches to the last bit: a thread needs
+// only 2^a (common path) or 2^-a (exact path), so one exponential of the argument with the thread's sign serves both.
+template <int N, bool WITH_SLOPE, int EMULATE_EVERY>
+__device__ __forceinline__ void sigmoid_signed(const float (&a)[N], bool exact, float (&pr)[N], float* pp) {
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const bool emulate = EMULATE_EVERY > 0 && i % (EMULATE_EVERY > 0 ? EMULATE_EVERY : 1) == EMULATE_EVERY - 1;
+    float v = sm100::ex2_approx(fminf(exact ? -a[i] : a[i], 120.0f));
+    if (emulate && !exact) v = ex2_emulated(a[i]);
+    const float w = fmaf(-v, v, v);
+    const float p_common = fmaf(-v, w, v);
+    const float r = WITH_SLOPE ? sm100::rcp_approx(1.0f + v) : rcp_newton(1.0f + v);
+    pr[i] = exact ? r : p_common;
+    if (WITH_SLOPE) pp[i] = exact ? r * (v * r) : fmaf(-p_common, p_common, p_common);
+  }
+}
+
+// How a warp evaluates a block whose threads need different paths.
+enum Mixing {
+  kBranches,   // one path after the other
+  kShared,     // sigmoid_mixed
+  kSigned      // sigmoid_signed
+};
+
+// Which form a kernel uses.  Short sequences, where b = -log n leaves most warps mixed, gain from one exponential:
+// without a mask B32 H12 N197 D64 forward 24.6 -> 20.6 us, backward 65.0 -> 61.8; N577 50.9 -> 45.1, 108 -> 103.
+// Causal instantiations keep the branches: B8 H16 N2048 D64 ALiBi (hardly any mixed warp) went from 131 to 137 us
+// with the shared form, and b = 0 at D = 128 (nearly all warps exact) from 47.4 to 54.1.  Documents packed without
+// padding (RAGGED) are mostly short whatever the mask.
+__host__ __device__ constexpr Mixing mixing(bool causal, bool ragged) {
+  return !causal ? kShared : ragged ? kSigned : kBranches;
+}
+
 // a[N] (already scaled by log2 e) -> P[N]; if WITH_SLOPE also P (1 - P) in pp[N].
 // The block's largest a decides between the two paths before anything else is evaluated.
-// SHARED (without a causal mask): a warp whose threads disagree, or all take the exact path, evaluates both from
-// one exponential.  Short sequences, where b = -log n leaves most warps mixed, gain: B32 H12 N197 D64 forward
-// 24.6 -> 20.6 us, backward 65.0 -> 61.8; N577 50.9 -> 45.1, 108 -> 103.  The causal instantiations keep the
-// branches: with the shared form B8 H16 N2048 D64 ALiBi (hardly any mixed warp) went from 131 to 137 us, and
-// b = 0 at D = 128 (nearly all warps exact) from 47.4 to 54.1.
-template <int N, bool WITH_SLOPE, int EMULATE_EVERY, bool SHARED>
+template <int N, bool WITH_SLOPE, int EMULATE_EVERY, Mixing MIXING>
 __device__ __forceinline__ void sigmoid_block(const float (&a)[N], float (&pr)[N], float* pp) {
   const bool exact = max_tree<N>(a) > kFastPathMaxA;
-  if constexpr (SHARED) {
-    if (!__any_sync(0xffffffffu, exact)) sigmoid_common<N, WITH_SLOPE, EMULATE_EVERY>(a, pr, pp);
-    else sigmoid_mixed<N, WITH_SLOPE, EMULATE_EVERY>(a, exact, pr, pp);
-  } else {
+  if constexpr (MIXING == kBranches) {
     if (!exact) sigmoid_common<N, WITH_SLOPE, EMULATE_EVERY>(a, pr, pp);
     else sigmoid_exact<N, WITH_SLOPE>(a, pr, pp);
+  } else {   // (the warp is converged here)
+    if (!__any_sync(0xffffffffu, exact)) sigmoid_common<N, WITH_SLOPE, EMULATE_EVERY>(a, pr, pp);
+    else if constexpr (MIXING == kShared) sigmoid_mixed<N, WITH_SLOPE, EMULATE_EVERY>(a, exact, pr, pp);
+    else sigmoid_signed<N, WITH_SLOPE, EMULATE_EVERY>(a, exact, pr, pp);
   }
 }
 
@@ -182,7 +211,7 @@ __device__ __forceinline__ void sigmoid_cols(const uint32_t (&s)[NC], uint32_t (
     a[i] = fmaf(__uint_as_float(s[i]), scale_log2e, c0);
   }
   float pr[NC];
-  sigmoid_block<NC, false, EMULATE_EVERY, !CAUSAL>(a, pr, nullptr);
+  sigmoid_block<NC, false, EMULATE_EVERY, mixing(CAUSAL, TWO_SIDED)>(a, pr, nullptr);
   if (masked) {  // keys after the query (and, in a padded batch, past the sequence's end) get weight 0
 #pragma unroll
     for (int i = 0; i < NC; ++i)
@@ -202,7 +231,7 @@ __device__ __forceinline__ void sigmoid_cols(const uint32_t (&s)[NC], uint32_t (
 // MASK: 0 no element masked, 1 causal only (queries before mask_lo), 2 both ends (padded batch)
 // CAUSAL: a query that keeps its weight sits at or after the key, so the position term is linear in the
 // query index: one FMA per logit from a per-call constant (a masked query is blanked afterwards).
-template <int MASK, bool ALIBI, bool CAUSAL>
+template <int MASK, bool ALIBI, bool CAUSAL, bool RAGGED = false>
 __device__ __forceinline__ void bwd_sigmoid_chunk(const uint32_t (&s)[32], uint32_t (&p_out)[16], float (&pp)[32],
                                                   float scale_log2e, float bias_log2e, float slope_log2e,
                                                   float col_rel, int q_base, float mask_lo, float mask_hi) {
@@ -216,7 +245,7 @@ __device__ __forceinline__ void bwd_sigmoid_chunk(const uint32_t (&s)[32], uint3
     a[e] = fmaf(__uint_as_float(s[e]), scale_log2e, c0);
   }
   float pr[32];
-  sigmoid_block<32, true, 0, !CAUSAL>(a, pr, pp);
+  sigmoid_block<32, true, 0, mixing(CAUSAL, RAGGED)>(a, pr, pp);
   if (MASK == 1) {
 #pragma unroll
     for (int e = 0; e < 32; ++e)

@@ -540,7 +540,9 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
       if (ragged) {
         mask_lo = static_cast<float>(q_lo - i * kT);
         mask_hi = static_cast<float>(q_hi - i * kT);
-        diag = i * kT < q_lo || (i + 1) * kT > q_hi;   // the tile is not wholly inside this key's queries
+        // the tile is not wholly inside the queries of some key of this warp (decided by the warp: threads that
+        // disagree would run the masked and the plain evaluation one after the other, 5200 cycles instead of 2200)
+        diag = __any_sync(0xffffffffu, i * kT < q_lo || (i + 1) * kT > q_hi);
       }
       float pp0[32], pp1[32];
       if (!mbar_wait(smem_u32(&bars->s_full[TM::r_index(step_cnt)]), TM::r_use(step_cnt) & 1, cta_err, 60 + wg))
@@ -554,14 +556,14 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
         tmem_wait_ld();
         float(&ppc)[32] = (c == 0) ? pp0 : pp1;
         if (GROUPED && diag)
-          bwd_sigmoid_chunk<2, ALIBI, CAUSAL>(s, pk, ppc, p.scale_log2e, bias_log2e, slope_log2e, col_rel, gc * 32, mask_lo,
-                                      mask_hi);
+          bwd_sigmoid_chunk<2, ALIBI, CAUSAL, ragged>(s, pk, ppc, p.scale_log2e, bias_log2e, slope_log2e, col_rel, gc * 32,
+                                                      mask_lo, mask_hi);
         else if (CAUSAL && diag)
-          bwd_sigmoid_chunk<1, ALIBI, CAUSAL>(s, pk, ppc, p.scale_log2e, bias_log2e, slope_log2e, col_rel, gc * 32, col_rel,
-                                      0.0f);
+          bwd_sigmoid_chunk<1, ALIBI, CAUSAL, ragged>(s, pk, ppc, p.scale_log2e, bias_log2e, slope_log2e, col_rel, gc * 32,
+                                                      col_rel, 0.0f);
         else
-          bwd_sigmoid_chunk<0, ALIBI, CAUSAL>(s, pk, ppc, p.scale_log2e, bias_log2e, slope_log2e, col_rel, gc * 32, 0.0f,
-                                      0.0f);
+          bwd_sigmoid_chunk<0, ALIBI, CAUSAL, ragged>(s, pk, ppc, p.scale_log2e, bias_log2e, slope_log2e, col_rel, gc * 32,
+                                                      0.0f, 0.0f);
         tmem_st16(tmem + TM::a_col(step_cnt) + lane_off + wg * 64 + c * 16, pk);
       }
       tmem_wait_st();
