@@ -180,15 +180,24 @@ __device__ __forceinline__ BwdItem decode_bwd_item(const BwdParams& p, int item)
   BwdItem w;
   // Items are numbered group of heads by group of heads (see the launcher; one group = all heads), within a group by
   // ascending key tile = descending work when causal, then head, then part.
+  // (Divisions only where they are needed: every role decodes every item, and the thread that issues the products
+  // pays for each instruction.  Two more of them cost 15 % at N = 577, five short items a head.)
   const int parts = GROUPED ? (p.n_sub > 1 ? p.n_sub : p.i_split) : 1;
-  const int per_group = p.head_group * p.n_tiles_k * parts;
-  const int g0 = item / per_group * p.head_group;
-  const int per_tile = min(p.head_group, p.BH - g0) * parts;
-  int r = item - g0 * p.n_tiles_k * parts;
+  int g0 = 0, r = item, per_tile = p.BH * parts;
+  if (p.head_group < p.BH) {
+    const int per_group = p.head_group * p.n_tiles_k * parts, gr = item / per_group;
+    g0 = gr * p.head_group;
+    r -= gr * per_group;
+    per_tile = min(p.head_group, p.BH - g0) * parts;
+  }
   w.j = r / per_tile;
   r -= w.j * per_tile;
-  w.bh = g0 + (GROUPED ? r / parts : r);
-  const int of_parts = GROUPED ? r - (w.bh - g0) * parts : 0;
+  int of_parts = 0;
+  if (GROUPED && parts > 1) {
+    of_parts = r % parts;
+    r /= parts;
+  }
+  w.bh = g0 + r;
   const int sub = (GROUPED && p.n_sub > 1) ? of_parts : 0;     // part of the query heads of a key/value head
   const int part = (GROUPED && p.i_split > 1) ? of_parts : 0;  // half of the query tiles
   w.bh_q0 = GROUPED ? (w.bh / p.H_kv) * p.H + (w.bh % p.H_kv) * p.group + sub * p.heads_per_sub : w.bh;

@@ -197,11 +197,16 @@ __device__ __forceinline__ Item decode_item(const FwdParams& p, int item) {
   Item w;
   // Items are numbered group of heads by group of heads (one group = all heads unless the launcher says otherwise),
   // within a group by decreasing cost, then head.
-  const int g0 = item / (p.head_group * p.n_pairs * p.n_splits) * p.head_group;
-  const int gn = min(p.head_group, p.BH - g0);
-  const int in_group = item - g0 * p.n_pairs * p.n_splits;
-  int rank = in_group / gn;
-  w.bh = g0 + in_group - rank * gn;
+  int g0 = 0, gn = p.BH, rank = item;
+  if (p.head_group < p.BH) {
+    const int per_group = p.head_group * p.n_pairs, gr = item / per_group;   // (never with split keys)
+    g0 = gr * p.head_group;
+    gn = min(p.head_group, p.BH - g0);
+    rank -= gr * per_group;
+  }
+  w.bh = g0 + rank;
+  rank /= gn;
+  w.bh -= rank * gn;
   const int split = rank / p.n_pairs;   // 0 unless the keys are split
   rank -= split * p.n_pairs;
   const int pair = CAUSAL ? (p.n_pairs - 1 - rank) : rank;
