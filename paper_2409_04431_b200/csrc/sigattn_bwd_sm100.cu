@@ -21,9 +21,8 @@
 // converted to bf16 (times scale) after the main kernel: the two helper steps that
 // survive from the paper's backward.  scale is also folded into dK's epilogue.
 //
-// Warp roles (448 threads): warps 0-7 two activation groups (query columns 0-63 and
-// 64-127 of the tile; every thread owns one key row), warps 8-11 dQ drain group,
-// warp 12 TMA producer, warp 13 MMA issuer.
+// Warp roles (see BwdRoles): activation groups of four warps (every thread owns one key row and a share of the
+// tile's query columns), at D = 128 a dQ drain group, a TMA producer, an MMA issuer.
 #include <atomic>
 
 #include "sigattn_internal.h"
@@ -38,9 +37,32 @@ namespace {
 using namespace sm100;
 
 constexpr int kT = 128;  // tile edge: keys per item (TMEM lanes) and queries per step
-constexpr int kBwdThreads = 448;
-constexpr int kBwdLoadWarp = 12;
-constexpr int kBwdMmaWarp = 13;
+
+// Warp roles.  Narrow: two activation groups of four warps (64 query columns a thread) and a drain group.  Wide
+// (D = 64): four activation groups (32 query columns a thread) that also drain dQ, and a thread that issues its adds.
+// Four warps per scheduler instead of two cover the latency of the activation and feed the exponentials evenly where
+// the warps take different paths, and each path's code is half as long (two chunks of 32 logits on both paths do not
+// fit the instruction cache well); but 512 threads wait, drain and arrive where 256 and 128 did.  The launcher
+// chooses (see there).  The 512 activation threads have 96 registers each: room for 32 columns and no more.
+template <int D, bool WIDE>
+struct BwdRoles {
+  static_assert(D == 64 || !WIDE, "at D = 128 the step is bound by the products and the drain");
+  static constexpr bool kDrainGroup = !WIDE;
+  static constexpr int kGroups = WIDE ? 4 : 2;                 // activation groups
+  static constexpr int kCols = kT / kGroups;                   // query columns of a thread
+  static constexpr int kActThreads = 128 * kGroups;
+  static constexpr int kDrainThreads = kDrainGroup ? 128 : kActThreads;
+  static constexpr int kLoadWarp = 4 * kGroups + (kDrainGroup ? 4 : 0);
+  static constexpr int kMmaWarp = kLoadWarp + 1;
+  static constexpr int kStoreWarp = kMmaWarp + 1;              // wide: issues the dQ adds
+  static constexpr int kThreads = 32 * (kMmaWarp + (kDrainGroup ? 1 : 2));
+  static constexpr int kSchedConsumers = 1 + kActThreads + (kDrainGroup ? 128 : 1);   // see the dynamic schedule
+  // first packed column of k-step ks (16 queries = 8 columns): a group packs its bf16 values over the first half
+  // of its own columns
+  __device__ static __forceinline__ uint32_t packed_col(int ks) {
+    return (ks / (kCols / 16)) * kCols + (ks % (kCols / 16)) * 8;
+  }
+};
 constexpr float kLog2eB = 1.4426950408889634f;
 
 template <int D>
@@ -78,6 +100,7 @@ struct BwdBarriers {
   uint64_t p_ready[2], ds_ready;
   uint64_t dq_full[2], dq_empty[2];
   uint64_t dkv_full, dkv_empty;
+  uint64_t stage_full, stage_empty;   // wide: the dQ staging boxes between the activation groups and the storing thread
   // dynamic schedule (batches without padding): the TMA thread draws the next work item from a
   // global counter and hands it to the other roles through this two-slot ring
   uint64_t sched_full[2], sched_empty[2];
@@ -138,7 +161,6 @@ __device__ __forceinline__ int bwd_num_rounds(int n_items) { return (n_items + g
 // inside its own sequence, and when heads are handed out in groups.  One thread per CTA draws; the MMA thread, the
 // activation groups and the drain group read the item from a two-slot ring.  false: a bounded wait expired;
 // *item < 0: none left.
-constexpr int kBwdSchedConsumers = 1 + 256 + 128;
 __device__ __forceinline__ bool bwd_sched_draw(const BwdParams& p, BwdBarriers* bars, int round, int* item,
                                                volatile int* cta_err) {
   const uint32_t slot = round & 1, phase = (round >> 1) & 1;
@@ -339,7 +361,7 @@ __device__ void bwd_load_role(const BwdParams& p, const CUtensorMap* tmQ, const 
 // a single thread is active, and every product costs the thread more.  Measured, whole backward, us:
 // B8 H12 N4096 D64 1540 -> 1385, B8 H16 N2048 D64 causal ALiBi 353 -> 331, B2 H16 N4096 D128 causal 389 -> 387.
 // (The role run by the whole warp with an election per batch of products: 1405, 339, 392.)
-template <int D, bool CAUSAL, bool GROUPED>
+template <int D, bool CAUSAL, bool GROUPED, bool WIDE>
 __device__ void bwd_mma_role(const BwdParams& p, uint32_t smem_base, uint32_t tmem, BwdBarriers* bars,
                              volatile int* cta_err) {
   using L = BwdSmem<D>;
@@ -427,7 +449,7 @@ __device__ void bwd_mma_role(const BwdParams& p, uint32_t smem_base, uint32_t tm
       const uint64_t dDo_mn = desc_advance(dDo_mn0, do_stage(do_cnt) * L::kTileBytes);
 #pragma unroll
       for (int ks = 0; ks < kT / 16; ++ks) {
-        umma_ts(tmem + TM::kDv, tmem + TM::a_col(step_cnt) + (ks >> 2) * 64 + (ks & 3) * 8,
+        umma_ts(tmem + TM::kDv, tmem + TM::a_col(step_cnt) + BwdRoles<D, WIDE>::packed_col(ks),
                 desc_advance(dDo_mn, ks * 2048), kIdescAcc, (it > 0 || ks > 0));
       }
       umma_commit(smem_u32(&bars->do_empty[do_stage(do_cnt)]));
@@ -443,7 +465,7 @@ __device__ void bwd_mma_role(const BwdParams& p, uint32_t smem_base, uint32_t tm
       const uint64_t q_mn = desc_advance(dQ_mn0, st * L::kTileBytes);
 #pragma unroll
       for (int ks = 0; ks < kT / 16; ++ks) {
-        umma_ts(tmem + TM::kDk, tmem + TM::kB + (ks >> 2) * 64 + (ks & 3) * 8, desc_advance(q_mn, ks * 2048),
+        umma_ts(tmem + TM::kDk, tmem + TM::kB + BwdRoles<D, WIDE>::packed_col(ks), desc_advance(q_mn, ks * 2048),
                 kIdescAcc, (it > 0 || ks > 0));
       }
 #pragma unroll
@@ -466,12 +488,14 @@ __device__ void bwd_mma_role(const BwdParams& p, uint32_t smem_base, uint32_t tm
 
 // ------------------------------------------------------------------ activation groups
 
-// One row of a [128 x D] fp32 accumulator -> bf16 (times `mul`) -> swizzled staging tile.
-template <int D>
-__device__ __forceinline__ void bwd_store_acc_rows(uint32_t t_acc, uint8_t* stage, int tid, float mul) {
+// One row of a [128 x D] fp32 accumulator -> bf16 (times `mul`) -> swizzled staging tile: share `part` of its
+// columns (32-column runs part, part + parts, ...).
+template <int D, bool WIDE>
+__device__ __forceinline__ void bwd_store_acc_rows(uint32_t t_acc, uint8_t* stage, int tid, float mul, int part) {
   using L = BwdSmem<D>;
+  constexpr int kParts = BwdRoles<D, WIDE>::kGroups / 2;
 #pragma unroll 1
-  for (int c = 0; c < D / 32; ++c) {
+  for (int c = part; c < D / 32; c += kParts) {
     uint32_t o[32];
     tmem_ld32(t_acc + c * 32, o);
     tmem_wait_ld();
@@ -490,15 +514,42 @@ __device__ __forceinline__ void bwd_store_acc_rows(uint32_t t_acc, uint8_t* stag
 }
 
 // KIND: 0 plain, 1 general (grouped heads, padded batch), 2 general plus a batch stored without padding
-template <int D, bool CAUSAL, bool ALIBI, bool DBIAS, int KIND>
-__device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const CUtensorMap* tmDv, int wg,
+template <int D, bool CAUSAL, bool ALIBI, bool DBIAS, int KIND, bool WIDE>
+__device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const CUtensorMap* tmDv,
+                             int wg,
                              uint8_t* smem, uint32_t tmem, BwdBarriers* bars, volatile int* cta_err) {
   using L = BwdSmem<D>;
   using TM = BwdTmem<D>;
+  using R = BwdRoles<D, WIDE>;
   constexpr bool GROUPED = KIND >= 1;
+  constexpr int kCols = R::kCols;
   const int tid = threadIdx.x & 127;  // key row within the tile
   const uint32_t lane_off = static_cast<uint32_t>(((threadIdx.x >> 5) & 3) * 32) << 16;
   uint32_t step_cnt = 0, item_cnt = 0;
+
+  // Without a drain group: the dQ tile of global step `step`, 16 of its 64 columns per group, to the two staging
+  // boxes, from where one thread of another warp adds it to the fp32 accumulator (with barriers among the 512 threads
+  // instead a drain cost 1000 of a step's 3520 cycles).  Done after the P phase of the following step, by when the
+  // products have completed it.
+  auto drain = [&](uint32_t step) -> bool {
+    const uint32_t reg = TM::r_index(step);
+    if (!mbar_wait(smem_u32(&bars->dq_full[reg]), TM::r_use(step) & 1, cta_err, 70 + wg)) return false;
+    tc_fence_after_sync();
+    uint32_t o[16];
+    tmem_ld16(tmem + TM::dq_col(step) + lane_off + wg * 16, o);
+    tmem_wait_ld();
+    tc_fence_before_sync();
+    mbar_arrive(smem_u32(&bars->dq_empty[reg]));
+    if (!mbar_wait(smem_u32(&bars->stage_empty), (step & 1) ^ 1, cta_err, 74)) return false;
+    uint8_t* box = smem + L::kDqOff + (wg >> 1) * L::kPanelBytes + tid * 128;
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      *reinterpret_cast<uint4*>(box + ((((wg & 1) * 4 + e) ^ (tid & 7)) * 16)) =
+          make_uint4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]);
+    fence_proxy_async_smem();
+    mbar_arrive(smem_u32(&bars->stage_full));
+    return true;
+  };
 
   const bool dynamic = p.sched_counter != nullptr;
   for (int round = 0, rounds = bwd_num_rounds(p.n_items); dynamic || round < rounds; ++round) {
@@ -553,17 +604,17 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
         // disagree would run the masked and the plain evaluation one after the other, 5200 cycles instead of 2200)
         diag = __any_sync(0xffffffffu, i * kT < q_lo || (i + 1) * kT > q_hi);
       }
-      float pp0[32], pp1[32];
+      float pp[kCols / 32][32];
       if (!mbar_wait(smem_u32(&bars->s_full[TM::r_index(step_cnt)]), TM::r_use(step_cnt) & 1, cta_err, 60 + wg))
         return;
       tc_fence_after_sync();
 #pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        const int gc = wg * 2 + c;  // 32-query chunk of the tile
+      for (int c = 0; c < kCols / 32; ++c) {
+        const int gc = wg * (kCols / 32) + c;  // 32-query chunk of the tile
         uint32_t s[32], pk[16];
         tmem_ld32(tmem + TM::a_col(step_cnt) + lane_off + gc * 32, s);
         tmem_wait_ld();
-        float(&ppc)[32] = (c == 0) ? pp0 : pp1;
+        float(&ppc)[32] = pp[c];
         if (GROUPED && diag)
           bwd_sigmoid_chunk<2, ALIBI, CAUSAL, ragged>(s, pk, ppc, p.scale_log2e, bias_log2e, slope_log2e, col_rel, gc * 32,
                                                       mask_lo, mask_hi);
@@ -573,25 +624,28 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
         else
           bwd_sigmoid_chunk<0, ALIBI, CAUSAL, ragged>(s, pk, ppc, p.scale_log2e, bias_log2e, slope_log2e, col_rel, gc * 32,
                                                       0.0f, 0.0f);
-        tmem_st16(tmem + TM::a_col(step_cnt) + lane_off + wg * 64 + c * 16, pk);
+        tmem_st16(tmem + TM::a_col(step_cnt) + lane_off + wg * kCols + c * 16, pk);
       }
       tmem_wait_st();
       tc_fence_before_sync();
       mbar_arrive(smem_u32(&bars->p_ready[TM::r_index(step_cnt)]));
+      if constexpr (!R::kDrainGroup) {
+        if ((g > 0 || it > 0) && !drain(step_cnt - 1)) return;
+      }
 
       // dS^T = P (1 - P) dP^T -> bf16 -> shared memory [key][query], 128-byte swizzle
       if (!mbar_wait(smem_u32(&bars->dp_full), step_cnt & 1, cta_err, 62 + wg)) return;
       tc_fence_after_sync();
-      uint8_t* ds_row = smem + L::kDsOff + wg * L::kPanelBytes + tid * 128;
+      uint8_t* ds_row = smem + L::kDsOff + (wg * kCols >> 6) * L::kPanelBytes + tid * 128;
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {  // 16 queries at a time
+      for (int c = 0; c < kCols / 16; ++c) {  // 16 queries at a time
         uint32_t dp[16];
-        tmem_ld16(tmem + TM::kB + lane_off + wg * 64 + c * 16, dp);
+        tmem_ld16(tmem + TM::kB + lane_off + wg * kCols + c * 16, dp);
         tmem_wait_ld();
         uint32_t ds[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-          const float* f = ((c < 2) ? pp0 : pp1) + (c & 1) * 16 + 2 * e;
+          const float* f = pp[c >> 1] + (c & 1) * 16 + 2 * e;
           const float ds0 = f[0] * __uint_as_float(dp[2 * e]), ds1 = f[1] * __uint_as_float(dp[2 * e + 1]);
           if (DBIAS) ds_sum += ds0 + ds1;
           ds[e] = pack_bf16x2(ds0, ds1);
@@ -599,12 +653,12 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
         // one copy to shared memory (A operand of dQ, MN-major) ...
 #pragma unroll
         for (int g = 0; g < 2; ++g) {
-          const int chunk = c * 2 + g;
+          const int chunk = ((wg * kCols & 63) >> 3) + c * 2 + g;
           *reinterpret_cast<uint4*>(ds_row + ((chunk ^ (tid & 7)) * 16)) =
               make_uint4(ds[4 * g + 0], ds[4 * g + 1], ds[4 * g + 2], ds[4 * g + 3]);
         }
         // ... and one to tensor memory (A operand of dK), over dP^T columns already consumed
-        tmem_st8(tmem + TM::kB + lane_off + wg * 64 + c * 8, ds);
+        tmem_st8(tmem + TM::kB + lane_off + wg * kCols + c * 8, ds);
       }
       tmem_wait_st();
       tc_fence_before_sync();   // the dP^T reads above precede the dQ MMA that overwrites region B
@@ -622,19 +676,25 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
     }
     }   // query heads
 
-    // epilogue: group 0 stores dV_j (staged in the V tile), group 1 stores scale * dK_j (K tile)
+    if constexpr (!R::kDrainGroup) {
+      if (!drain(step_cnt - 1)) return;
+    }
+
+    // epilogue: the first half of the groups stores dV_j (staged in the V tile), the other half scale * dK_j (K tile)
     if (!mbar_wait(smem_u32(&bars->dkv_full), item_cnt & 1, cta_err, 64 + wg)) return;
     const uint32_t kv_stage = item_cnt % L::kKvStages;
     ++item_cnt;
     tc_fence_after_sync();
-    uint8_t* stage = smem + kv_stage * L::kKvBytes + (wg == 0 ? L::kVOff : L::kKOff);
-    bwd_store_acc_rows<D>(tmem + (wg == 0 ? TM::kDv : TM::kDk) + lane_off, stage, tid, wg == 0 ? 1.0f : p.scale);
+    const bool is_dv = wg < R::kGroups / 2;
+    uint8_t* stage = smem + kv_stage * L::kKvBytes + (is_dv ? L::kVOff : L::kKOff);
+    bwd_store_acc_rows<D, WIDE>(tmem + (is_dv ? TM::kDv : TM::kDk) + lane_off, stage, tid, is_dv ? 1.0f : p.scale,
+                          wg % (R::kGroups / 2));
     tc_fence_before_sync();
     mbar_arrive(smem_u32(&bars->dkv_empty));
     fence_proxy_async_smem();
-    if (wg == 0) named_barrier_sync<1, 128>(); else named_barrier_sync<2, 128>();
-    if (tid == 0) {
-      const CUtensorMap* tm = (wg == 0) ? tmDv : tmDk;
+    if (is_dv) named_barrier_sync<1, R::kActThreads / 2>(); else named_barrier_sync<2, R::kActThreads / 2>();
+    if (tid == 0 && wg % (R::kGroups / 2) == 0) {
+      const CUtensorMap* tm = is_dv ? tmDv : tmDk;
 #pragma unroll
       for (int pn = 0; pn < L::kPanels; ++pn)
         if (GROUPED && (p.n_sub > 1 || p.i_split > 1 || p.dkv_add))   // the parts (or successive calls) add their shares
@@ -714,14 +774,49 @@ __device__ void bwd_drain_role(const BwdParams& p, const CUtensorMap* tmW, uint8
   if (tid == 0) tma_wait_group<0>();
 }
 
+// Wide: one thread adds the staged dQ tiles to the fp32 accumulator.
+template <int D, bool CAUSAL, bool GROUPED>
+__device__ void bwd_store_role(const BwdParams& p, const CUtensorMap* tmW, uint32_t smem_base, BwdBarriers* bars,
+                               volatile int* cta_err) {
+  using L = BwdSmem<D>;
+  uint32_t step_cnt = 0;
+  const bool dynamic = p.sched_counter != nullptr;
+  for (int round = 0, rounds = bwd_num_rounds(p.n_items); dynamic || round < rounds; ++round) {
+    int item;
+    if (dynamic) {
+      if (!bwd_sched_take(bars, round, &item, cta_err)) return;
+      if (item < 0) break;
+    } else {
+      item = bwd_snake_rank(round, p.n_items);
+      if (item < 0) continue;
+    }
+    const BwdItem w = decode_bwd_item<CAUSAL, GROUPED>(p, item);
+    int it = 0, bh_q = w.bh_q0;
+    for (int s = 0; s < w.steps; ++s, ++step_cnt) {
+      if (!mbar_wait(smem_u32(&bars->stage_full), step_cnt & 1, cta_err, 75)) return;
+      tma_reduce_add_3d(tmW, smem_base + L::kDqOff, 0, (w.i_begin + it) * kT, bh_q);
+      tma_reduce_add_3d(tmW, smem_base + L::kDqOff + L::kPanelBytes, 32, (w.i_begin + it) * kT, bh_q);
+      tma_commit_group();
+      tma_wait_group_read<0>();
+      mbar_arrive(smem_u32(&bars->stage_empty));
+      if (++it == w.n) {   // the next query head of the group
+        it = 0;
+        ++bh_q;
+      }
+    }
+  }
+  tma_wait_group<0>();
+}
+
 // ------------------------------------------------------------------ kernels
 
-template <int D, bool CAUSAL, bool ALIBI, bool DBIAS, int KIND>
-__global__ void __launch_bounds__(kBwdThreads, 1)
+template <int D, bool CAUSAL, bool ALIBI, bool DBIAS, int KIND, bool WIDE>
+__global__ void __launch_bounds__(BwdRoles<D, WIDE>::kThreads, 1)
 sigattn_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                         const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmDo,
                         const __grid_constant__ CUtensorMap tmDk, const __grid_constant__ CUtensorMap tmDv,
                         const __grid_constant__ CUtensorMap tmW, const BwdParams p) {
+  using R = BwdRoles<D, WIDE>;
   constexpr bool GROUPED = KIND >= 1;
   extern __shared__ uint8_t smem_raw[];
   __shared__ BwdBarriers bars;
@@ -746,21 +841,23 @@ sigattn_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(smem_u32(&bars.s_full[s]), 1);
-      mbar_init(smem_u32(&bars.p_ready[s]), 256);
+      mbar_init(smem_u32(&bars.p_ready[s]), R::kActThreads);
       mbar_init(smem_u32(&bars.dq_full[s]), 1);
-      mbar_init(smem_u32(&bars.dq_empty[s]), 128);
+      mbar_init(smem_u32(&bars.dq_empty[s]), R::kDrainThreads);
     }
     mbar_init(smem_u32(&bars.dp_full), 1);
-    mbar_init(smem_u32(&bars.ds_ready), 256);
+    mbar_init(smem_u32(&bars.ds_ready), R::kActThreads);
     mbar_init(smem_u32(&bars.dkv_full), 1);
-    mbar_init(smem_u32(&bars.dkv_empty), 256);
+    mbar_init(smem_u32(&bars.stage_full), R::kActThreads);
+    mbar_init(smem_u32(&bars.stage_empty), 1);
+    mbar_init(smem_u32(&bars.dkv_empty), R::kActThreads);
     for (int s = 0; s < 2; ++s) {
       mbar_init(smem_u32(&bars.sched_full[s]), 1);
-      mbar_init(smem_u32(&bars.sched_empty[s]), kBwdSchedConsumers);
+      mbar_init(smem_u32(&bars.sched_empty[s]), BwdRoles<D, WIDE>::kSchedConsumers);
     }
     fence_mbar_init();
   }
-  if (warp == kBwdLoadWarp && elect_one()) {
+  if (warp == R::kLoadWarp && elect_one()) {
     tma_prefetch_desc(&tmQ);
     tma_prefetch_desc(&tmK);
     tma_prefetch_desc(&tmV);
@@ -769,7 +866,7 @@ sigattn_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     tma_prefetch_desc(&tmDv);
     tma_prefetch_desc(&tmW);
   }
-  if (warp == kBwdMmaWarp) {
+  if (warp == R::kMmaWarp) {
     tmem_alloc(smem_u32(&tmem_base_slot), 512);
     tmem_relinquish();
   }
@@ -778,16 +875,19 @@ sigattn_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   tc_fence_after_sync();
   const uint32_t tmem = tmem_base_slot;
 
-  if (warp == kBwdLoadWarp) {
+  if (warp == R::kLoadWarp) {
     if ((threadIdx.x & 31) == 0) bwd_load_role<D, CAUSAL, GROUPED>(p, &tmQ, &tmK, &tmV, &tmDo, smem_base, &bars, &cta_err);
     __syncwarp();
-  } else if (warp == kBwdMmaWarp) {
-    if (elect_one()) bwd_mma_role<D, CAUSAL, GROUPED>(p, smem_base, tmem, &bars, &cta_err);
+  } else if (warp == R::kMmaWarp) {
+    if (elect_one()) bwd_mma_role<D, CAUSAL, GROUPED, WIDE>(p, smem_base, tmem, &bars, &cta_err);
     __syncwarp();
-  } else if (warp < 8) {
-    bwd_act_role<D, CAUSAL, ALIBI, DBIAS, KIND>(p, &tmDk, &tmDv, warp >> 2, smem, tmem, &bars, &cta_err);
-  } else {
+  } else if (warp < 4 * R::kGroups) {
+    bwd_act_role<D, CAUSAL, ALIBI, DBIAS, KIND, WIDE>(p, &tmDk, &tmDv, warp >> 2, smem, tmem, &bars, &cta_err);
+  } else if constexpr (R::kDrainGroup) {
     bwd_drain_role<D, CAUSAL, GROUPED>(p, &tmW, smem, tmem, &bars, &cta_err);
+  } else {
+    if (elect_one()) bwd_store_role<D, CAUSAL, GROUPED>(p, &tmW, smem_base, &bars, &cta_err);
+    __syncwarp();
   }
 
   tc_fence_before_sync();
@@ -796,7 +896,7 @@ sigattn_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     if (threadIdx.x == 0) atomicExch(p.status, 200 + cta_err);
     __nanosleep(100000);
   }
-  if (warp == kBwdMmaWarp) tmem_dealloc(tmem, 512);
+  if (warp == R::kMmaWarp) tmem_dealloc(tmem, 512);
 }
 
 // dQ (bf16) = scale * workspace (fp32): the conversion step that follows the main kernel.
@@ -871,10 +971,10 @@ constexpr size_t kBwdL2Share = 64u << 20;
 constexpr int kBwdSchedSlots = 1024;
 __device__ int g_bwd_sched_counters[kBwdSchedSlots];
 
-template <int D, bool CAUSAL, bool ALIBI, bool DBIAS, int KIND>
+template <int D, bool CAUSAL, bool ALIBI, bool DBIAS, int KIND, bool WIDE>
 int launch_bwd_variant(const CUtensorMap* maps, const BwdParams& bp, int num_sms, cudaStream_t stream,
                        cudaError_t* cuda_err) {
-  auto kernel = sigattn_bwd_bf16_kernel<D, CAUSAL, ALIBI, DBIAS, KIND>;
+  auto kernel = sigattn_bwd_bf16_kernel<D, CAUSAL, ALIBI, DBIAS, KIND, WIDE>;
   // The shared-memory opt-in is a per-device attribute of the kernel: one bit per device ordinal
   // (a process may drive several GPUs); ordinals past 63 simply set it on every launch.
   static std::atomic<unsigned long long> configured{0};
@@ -888,7 +988,7 @@ int launch_bwd_variant(const CUtensorMap* maps, const BwdParams& bp, int num_sms
     configured.fetch_or(bit, std::memory_order_relaxed);
   }
   const int grid = bp.n_items < num_sms ? bp.n_items : num_sms;
-  kernel<<<grid, kBwdThreads, BwdSmem<D>::kDynBytes, stream>>>(maps[0], maps[1], maps[2], maps[3], maps[4], maps[5],
+  kernel<<<grid, BwdRoles<D, WIDE>::kThreads, BwdSmem<D>::kDynBytes, stream>>>(maps[0], maps[1], maps[2], maps[3], maps[4], maps[5],
                                                                 maps[6], bp);
   *cuda_err = cudaGetLastError();
   return *cuda_err == cudaSuccess ? SIGATTN_OK : SIGATTN_ERR_CUDA;
@@ -1074,9 +1174,22 @@ int launch_bwd_bf16(const void* q, const void* k, const void* v, const void* d_o
   // the bias gradient costs the activation groups a running sum (4-5 % of the kernel), so it
   // is compiled in only where it is asked for; likewise the loop over a group's query heads and
   // the per-sequence lengths (kind 1) and the lookups of a batch without padding (kind 2)
+  // Wide or narrow (see BwdRoles).  Short sequences have b = -log n near the common path's limit, so many warps take
+  // both activation paths, and items of few steps; there four groups pay.  Long ones are bound by the other work of
+  // those groups.  The line is drawn by the length a typical row sees.  Whole backward, us, narrow / wide, H12 or 16:
+  //   no mask: B16 N300 54 / 52, B16 N577 122 / 101, B16 N1025 250 / 245, B16 N1500 387 / 401, B8 N2048 335 / 353;
+  //   causal: B16 N512 97 / 90, B8 N1024 115 / 106, B8 N2048 292 / 292, B2 N4096 246 / 251;
+  //   padded, lengths N/4 to N: N400 64 / 58, N1500 249 / 227, N2500 1010 / 967;
+  //   packed documents: 60 in 16384 rows 337 / 291, 16 in 16384 507 / 462, 5 in 8000 253 / 280.
+  const int typical_rows = p.cu_seqlens != nullptr ? p.N / p.n_seqs
+                           : p.seqlens != nullptr  ? p.N / 2
+                           : p.causal              ? p.N / 3 * 2 : p.N;
+  const bool wide = p.D == 64 && typical_rows <= 1280;
+#define SIGATTN_BWD_SHAPE(DD, CC, AA, BB, KK)                                                              \
+  ((DD == 64 && wide) ? launch_bwd_variant<DD, CC, AA, BB, KK, DD == 64>(maps, bp, num_sms, stream, cuda_err) \
+                      : launch_bwd_variant<DD, CC, AA, BB, KK, false>(maps, bp, num_sms, stream, cuda_err))
 #define SIGATTN_BWD_KIND(DD, CC, AA, KK)                                                                   \
-  ((p.dbias != nullptr) ? launch_bwd_variant<DD, CC, AA, true, KK>(maps, bp, num_sms, stream, cuda_err)    \
-                        : launch_bwd_variant<DD, CC, AA, false, KK>(maps, bp, num_sms, stream, cuda_err))
+  ((p.dbias != nullptr) ? SIGATTN_BWD_SHAPE(DD, CC, AA, true, KK) : SIGATTN_BWD_SHAPE(DD, CC, AA, false, KK))
 #define SIGATTN_BWD_CASE(DD, CC, AA)                                                                       \
   rc = (bp.cu_seqlens != nullptr)                  ? SIGATTN_BWD_KIND(DD, CC, AA, 2)                        \
        : (bp.group > 1 || bp.seqlens != nullptr || bp.i_split > 1 || bp.dkv_add) ? SIGATTN_BWD_KIND(DD, CC, AA, 1) \
@@ -1090,6 +1203,7 @@ int launch_bwd_bf16(const void* q, const void* k, const void* v, const void* d_o
   }
 #undef SIGATTN_BWD_CASE
 #undef SIGATTN_BWD_KIND
+#undef SIGATTN_BWD_SHAPE
   if (rc != SIGATTN_OK) return rc;
   if (timed) cudaEventRecord(t_ev_stop, stream);
   *launches += 1;

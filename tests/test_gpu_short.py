@@ -48,3 +48,31 @@ def test_short_many_heads_equal_the_general_kernels(B, N, causal):
     sa.sigattn_check()
     assert torch.equal(a[1], b[1]) and torch.equal(a[2], b[2])
     assert float((a[0].float() - b[0].float()).norm() / b[0].float().norm()) < 1e-3   # dQ: fp32 sums in another order
+
+
+@pytest.mark.parametrize("kind,H,H_kv,N", [
+    ("plain", 3, 3, 300), ("causal", 3, 3, 700), ("grouped", 4, 2, 385), ("padded", 2, 2, 520), ("packed", 2, 1, 900),
+])
+def test_wide_backward_at_64(kind, H, H_kv, N):
+    """The four-group shape of the backward (typical sequences up to 1280 rows, heads of 64): every kind of call that
+    reaches it, with a ragged last tile, several query tiles per item and several items per thread block."""
+    import torch
+    import paper_2409_04431_b200 as sa
+    B, D, causal = (1 if kind == "packed" else 2), 64, kind in ("causal", "packed")
+    q, _, _, d_o = inputs.random_case(B, H, N, D, 500 + N)
+    _, k, v, _ = inputs.random_case(B, H_kv, N, D, 501 + N)
+    tq, tk, tv, tdo = (to_device(t, "bf16") for t in (q, k, v, d_o))
+    scale, bias, more = 1.0 / math.sqrt(D), -math.log(N), {}
+    if kind == "padded":
+        lens = [N, N // 3]
+        out = sa.sigattn_bwd_varlen(tq, tk, tv, tdo, scale, bias, torch.tensor(lens, dtype=torch.int32, device="cuda"), causal)
+        more = {"seqlens": lens}
+    elif kind == "packed":
+        cu = np.array([0, 10, 300, 301, N], dtype=np.int32)
+        out = sa.sigattn_bwd_ragged(tq, tk, tv, tdo, torch.from_numpy(cu).cuda(), scale, bias, causal)
+        more = {"cu_seqlens": cu}
+    else:
+        out = sa.sigattn_bwd_gqa(tq, tk, tv, tdo, scale, bias, causal, want_dbias=True)
+    sa.sigattn_check()
+    for name, g, r in zip(("dQ", "dK", "dV"), out, oracle.sigattn_bwd(q, k, v, d_o, scale, bias, causal, None, **more)):
+        assert_bf16_close(to_host(g), r, name)
