@@ -121,6 +121,7 @@ struct FwdParams {
   // the partial results simply add up.  n_splits = 1: off.
   int n_splits, tiles_per_split;
   float* split_ws;
+  int split_cut;   // unpacked general mode, two parts: the first one's share of the key tiles, in 1/256
   int o_reduce;    // 1: split items of the unpacked general mode add bf16 tiles into O instead of storing them
   int n_items;
   int head_group;  // heads whose items are handed out together
@@ -256,13 +257,12 @@ __device__ __forceinline__ Item decode_item(const FwdParams& p, int item) {
     // the diagonal, which is fully masked (or out of range and read as zeros), and add zeros.
     const int n0 = w.n[0], n1 = w.n[1];
     if (n0 >= 2 * p.n_splits && (n1 == 0 || n1 >= n0)) {
-      // part s takes key tiles [s n0 / S, (s + 1) n0 / S): never empty since n0 >= 2 S; the last
-      // part of tile 1 runs on to n1
-      const int first = split * n0 / p.n_splits, end = (split + 1) * n0 / p.n_splits;
-      const bool last = split == p.n_splits - 1;
-      w.j0 = first;
-      w.n[0] = end - first;
-      w.n[1] = n1 == 0 ? 0 : (last ? n1 : end) - first;
+      // part 0 takes the first split_cut / 256 of the key tiles, part 1 the others (never empty since n0 >= 4;
+      // for tile 1 it runs on to n1)
+      const int cut = min(n0 - 1, max(1, n0 * p.split_cut >> 8));
+      w.j0 = split == 0 ? 0 : cut;
+      w.n[0] = split == 0 ? cut : n0 - cut;
+      w.n[1] = n1 == 0 ? 0 : (split == 0 ? cut : n1 - cut);
     } else if (split > 0) {
       w.j0 = max(n0, n1);
       w.n[0] = n0 > 0 ? 1 : 0;
@@ -949,6 +949,32 @@ int launch_fwd_bf16(const void* q, const void* k, const void* v, void* o, const 
   fp.n_kv_total = (p.key_rows() + kBN - 1) / kBN;
   fp.n_splits = o_splits > 1 ? o_splits : n_splits;
   fp.o_reduce = o_splits > 1 ? 1 : 0;
+  fp.split_cut = 128;
+  if (o_splits > 1) {
+    // Where the items are cut.  The first parts are handed out first, one to an SM; the SMs left over take the second
+    // parts.  Halves suit a causal sequence, whose items' costs fall to nothing.  With items of about equal cost (no
+    // mask, or queries far behind the first key) and more than half as many items as SMs halves would make two full
+    // rounds; there the SMs left over take k second parts each, and both kinds of SM should end together:
+    // m + o = k (n - m + o), m of an item's n tiles in the first part, o tiles' worth of start and epilogue an item.
+    // Queries at the end of 8192 keys, H32 H_kv8 D128: 1024 (128 items) 135 -> 128 us, 700 (96 items) 134 -> 101.
+    constexpr double kItemTiles = 2.5;
+    long long tiles = 0;
+    int longest = 1;
+    for (int pair = 0; pair < fp.n_pairs; ++pair) {
+      const int end = (pair + 1) * 2 * kBM + fp.pos0;   // keys before this are seen by the pair's last row
+      int n = fp.n_kv_total;
+      if (p.causal) n = end <= 0 ? 1 : (end + kBN - 1) / kBN < n ? (end + kBN - 1) / kBN : n;
+      tiles += n;
+      if (n > longest) longest = n;
+    }
+    const int items = fp.n_pairs * fp.BH, left_over = num_sms - items;
+    if (left_over > 0 && 20 * tiles >= 17ll * longest * fp.n_pairs) {
+      const int k = (items + left_over - 1) / left_over;
+      const double second = (longest - (k - 1) * kItemTiles) / (k + 1);
+      const int cut = static_cast<int>(256.0 * (longest - second) / longest + 0.5);
+      fp.split_cut = cut < 128 ? 128 : cut > 250 ? 250 : cut;
+    }
+  }
   fp.tiles_per_split = (fp.n_kv_total + n_splits - 1) / n_splits;
   fp.split_ws = accumulate ? p.split_ws : nullptr;
   fp.n_items = fp.n_pairs * fp.BH * fp.n_splits;
