@@ -25,6 +25,7 @@
 // tile's query columns), at D = 128 a dQ drain group, a TMA producer, an MMA issuer.
 #include <atomic>
 
+#include "launch.h"
 #include "sigattn_internal.h"
 #include "sigattn_activation.cuh"
 #include "sm100_primitives.cuh"
@@ -54,7 +55,6 @@ struct BwdRoles {
   static constexpr int kDrainThreads = kDrainGroup ? 128 : kActThreads;
   static constexpr int kLoadWarp = 4 * kGroups + (kDrainGroup ? 4 : 0);
   static constexpr int kMmaWarp = kLoadWarp + 1;
-  static constexpr int kStoreWarp = kMmaWarp + 1;              // wide: issues the dQ adds
   static constexpr int kThreads = 32 * (kMmaWarp + (kDrainGroup ? 1 : 2));
   static constexpr int kSchedConsumers = 1 + kActThreads + (kDrainGroup ? 128 : 1);   // see the dynamic schedule
   // first packed column of k-step ks (16 queries = 8 columns): a group packs its bf16 values over the first half
@@ -874,6 +874,8 @@ sigattn_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = tmem_base_slot;
+  grid_dependency_wait();
+  grid_dependency_trigger();
 
   if (warp == R::kLoadWarp) {
     if ((threadIdx.x & 31) == 0) bwd_load_role<D, CAUSAL, GROUPED>(p, &tmQ, &tmK, &tmV, &tmDo, smem_base, &bars, &cta_err);
@@ -902,6 +904,8 @@ sigattn_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 // dQ (bf16) = scale * workspace (fp32): the conversion step that follows the main kernel.
 __global__ void __launch_bounds__(256)
 sigattn_bwd_convert_dq_kernel(const float4* __restrict__ ws, uint2* __restrict__ dq, size_t n_vec4, float scale) {
+  grid_dependency_wait();
+  grid_dependency_trigger();
   const size_t stride = static_cast<size_t>(gridDim.x) * blockDim.x;
   for (size_t i = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n_vec4; i += stride) {
     const float4 v = ws[i];
@@ -988,9 +992,8 @@ int launch_bwd_variant(const CUtensorMap* maps, const BwdParams& bp, int num_sms
     configured.fetch_or(bit, std::memory_order_relaxed);
   }
   const int grid = bp.n_items < num_sms ? bp.n_items : num_sms;
-  kernel<<<grid, BwdRoles<D, WIDE>::kThreads, BwdSmem<D>::kDynBytes, stream>>>(maps[0], maps[1], maps[2], maps[3], maps[4], maps[5],
-                                                                maps[6], bp);
-  *cuda_err = cudaGetLastError();
+  *cuda_err = launch_after(kernel, dim3(grid), BwdRoles<D, WIDE>::kThreads, BwdSmem<D>::kDynBytes, stream, 0, maps[0], maps[1],
+                           maps[2], maps[3], maps[4], maps[5], maps[6], bp);
   return *cuda_err == cudaSuccess ? SIGATTN_OK : SIGATTN_ERR_CUDA;
 }
 
@@ -1015,9 +1018,8 @@ int launch_acc_to_bf16(const float* acc, void* out, size_t n, float mul, cudaStr
   if (*cuda_err != cudaSuccess) return SIGATTN_ERR_CUDA;
   const size_t n_vec4 = n / 4;
   const size_t want = n_vec4 / 256 + 1, cap = static_cast<size_t>(num_sms) * 8;
-  sigattn_bwd_convert_dq_kernel<<<static_cast<int>(want < cap ? want : cap), 256, 0, stream>>>(
-      reinterpret_cast<const float4*>(acc), static_cast<uint2*>(out), n_vec4, mul);
-  *cuda_err = cudaGetLastError();
+  *cuda_err = launch_after(sigattn_bwd_convert_dq_kernel, dim3(static_cast<unsigned>(want < cap ? want : cap)), 256, 0, stream, 0,
+                           reinterpret_cast<const float4*>(acc), static_cast<uint2*>(out), n_vec4, mul);
   if (*cuda_err != cudaSuccess) return SIGATTN_ERR_CUDA;
   *launches += 1;
   return SIGATTN_OK;
@@ -1228,9 +1230,8 @@ int launch_bwd_bf16(const void* q, const void* k, const void* v, const void* d_o
   }
   const int blocks = static_cast<int>(n_vec4 / 256 + 1 < static_cast<size_t>(num_sms) * 8 ? n_vec4 / 256 + 1
                                                                                             : static_cast<size_t>(num_sms) * 8);
-  sigattn_bwd_convert_dq_kernel<<<blocks, 256, 0, stream>>>(static_cast<const float4*>(workspace),
-                                                            static_cast<uint2*>(dq), n_vec4, p.scale);
-  *cuda_err = cudaGetLastError();
+  *cuda_err = launch_after(sigattn_bwd_convert_dq_kernel, dim3(blocks), 256, 0, stream, 0, static_cast<const float4*>(workspace),
+                           static_cast<uint2*>(dq), n_vec4, p.scale);
   if (*cuda_err != cudaSuccess) return SIGATTN_ERR_CUDA;
   *launches += 1;
   return SIGATTN_OK;

@@ -26,6 +26,7 @@
 //   B = 32, N_k = 4096   115 -> 85 us;   B = 1, N_k = 2000   14.9 -> 8.3 us;   B = 1, N_k = 65536   63 -> 52 us
 #include <atomic>
 
+#include "launch.h"
 #include "sigattn_internal.h"
 #include "sm100_primitives.cuh"
 #include "tensor_map.h"
@@ -131,6 +132,7 @@ sigattn_decode_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid
     tmem_alloc(smem_u32(&tmem_base_slot), kDecTmemCols);
     tmem_relinquish();
   }
+  grid_dependency_wait();
   if (threadIdx.x < rows16) {
     // rows past the end only fill the tile; their weights are never used
     const int r = min(static_cast<int>(threadIdx.x), p.rows - 1);
@@ -144,6 +146,7 @@ sigattn_decode_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = tmem_base_slot;
+  grid_dependency_trigger();   // (after the allocation of tensor memory: see launch.h)
   const uint32_t tmem_o = tmem + 128;
 
   if (warp == kDecLoadWarp) {
@@ -336,19 +339,8 @@ int launch_decode_variant(const CUtensorMap& tmQ, const CUtensorMap& tmK, const 
     if (*cuda_err != cudaSuccess) return SIGATTN_ERR_CUDA;
     configured.fetch_or(bit, std::memory_order_relaxed);
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(shares), static_cast<unsigned>(heads));
-  cfg.blockDim = dim3(kDecThreads);
-  cfg.dynamicSmemBytes = smem_bytes;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = static_cast<unsigned>(dp.cluster);
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  *cuda_err = cudaLaunchKernelEx(&cfg, kernel, tmQ, tmK, tmV, dp);
+  *cuda_err = launch_after(kernel, dim3(static_cast<unsigned>(shares), static_cast<unsigned>(heads)), kDecThreads, smem_bytes,
+                           stream, static_cast<unsigned>(dp.cluster), tmQ, tmK, tmV, dp);
   return *cuda_err == cudaSuccess ? SIGATTN_OK : SIGATTN_ERR_CUDA;
 }
 

@@ -21,6 +21,7 @@
 // table in Appendix F.1 / Algorithm 2, with the factor scale = 1/sqrt(d) in dQ and dK.
 #include <atomic>
 
+#include "launch.h"
 #include "sigattn_internal.h"
 #include "../../include/sigattn.h"
 
@@ -275,6 +276,8 @@ template <int D>
 __global__ void __launch_bounds__(kThreads) fwd_fp32_kernel(const Fp32Args p) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   const int blocks = (p.N + kOwn - 1) / kOwn, head = blockIdx.x / blocks;
+  grid_dependency_wait();
+  grid_dependency_trigger();
   fp32_pass<D, kForward>(p, *reinterpret_cast<Fp32Smem<D>*>(smem_raw), (blockIdx.x - head * blocks) * kOwn, head);
 }
 
@@ -282,6 +285,8 @@ template <int D>
 __global__ void __launch_bounds__(kThreads) bwd_fp32_kernel(const Fp32Args p) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   Fp32Smem<D>& sm = *reinterpret_cast<Fp32Smem<D>*>(smem_raw);
+  grid_dependency_wait();
+  grid_dependency_trigger();
   if (static_cast<int>(blockIdx.x) < p.dq_blocks) {
     const int blocks = (p.N + kOwn - 1) / kOwn, head = blockIdx.x / blocks;
     fp32_pass<D, kGradQ>(p, sm, (blockIdx.x - head * blocks) * kOwn, head);
@@ -347,8 +352,7 @@ int launch_fp32(const Fp32Args& a, long long blocks, cudaStream_t stream, cudaEr
     if (*cuda_err != cudaSuccess) return SIGATTN_ERR_CUDA;
     configured.fetch_or(bit, std::memory_order_relaxed);
   }
-  kernel<<<static_cast<unsigned>(blocks), kThreads, sizeof(Fp32Smem<D>), stream>>>(a);
-  *cuda_err = cudaGetLastError();
+  *cuda_err = launch_after(kernel, dim3(static_cast<unsigned>(blocks)), kThreads, sizeof(Fp32Smem<D>), stream, 0, a);
   return *cuda_err == cudaSuccess ? SIGATTN_OK : SIGATTN_ERR_CUDA;
 }
 

@@ -27,6 +27,7 @@
 // tanh form is not used.
 #include <atomic>
 
+#include "launch.h"
 #include "sigattn_internal.h"
 #include "sigattn_activation.cuh"
 #include "sm100_primitives.cuh"
@@ -718,6 +719,8 @@ sigattn_fwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = tmem_base_slot;
+  grid_dependency_wait();
+  grid_dependency_trigger();
 
   if (warp == kLoadWarp) {
     if ((threadIdx.x & 31) == 0) fwd_load_role<D, CAUSAL, (MODE >= 2)>(p, &tmQ, &tmK, &tmV, smem_base, &bars, &cta_err);
@@ -813,8 +816,7 @@ int launch_fwd_variant(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUt
   }
   const int slots = num_sms * kCtasPerSm;
   const int grid = fp.n_items < slots ? fp.n_items : slots;
-  kernel<<<grid, kFwdThreads, FwdSmem<D>::kDynBytes, stream>>>(tmQ, tmK, tmV, tmO, fp);
-  *cuda_err = cudaGetLastError();
+  *cuda_err = launch_after(kernel, dim3(grid), kFwdThreads, FwdSmem<D>::kDynBytes, stream, 0, tmQ, tmK, tmV, tmO, fp);
   return *cuda_err == cudaSuccess ? SIGATTN_OK : SIGATTN_ERR_CUDA;
 }
 

@@ -22,6 +22,7 @@
 // launcher.
 #include <atomic>
 
+#include "launch.h"
 #include "sigattn_internal.h"
 #include "sigattn_activation.cuh"
 #include "sm100_primitives.cuh"
@@ -158,6 +159,8 @@ sigattn_short_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __g
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = tmem_base_slot;
+  grid_dependency_wait();
+  grid_dependency_trigger();
 
   if (warp == kSbLoadWarp) {
     if (elect_one()) {
@@ -429,8 +432,8 @@ int launch_short_bwd_variant(const CUtensorMap (&m)[7], const ShortBwdParams& sp
     configured.fetch_or(bit, std::memory_order_relaxed);
   }
   const int grid = sp.n_heads < num_sms ? sp.n_heads : num_sms;
-  kernel<<<grid, kSbThreads, kSbDynBytes, stream>>>(m[0], m[1], m[2], m[3], m[4], m[5], m[6], sp);
-  *cuda_err = cudaGetLastError();
+  *cuda_err = launch_after(kernel, dim3(grid), kSbThreads, kSbDynBytes, stream, 0, m[0], m[1], m[2], m[3], m[4], m[5],
+                           m[6], sp);
   return *cuda_err == cudaSuccess ? SIGATTN_OK : SIGATTN_ERR_CUDA;
 }
 

@@ -17,6 +17,7 @@
 // 197 28.7 -> 25.8, 256 29.5 -> 28.8; causal B64 H16 N200 59.7 -> 47.7; B1 H12 N50 8.3 -> 6.2, N197 10.3 -> 9.8.
 #include <atomic>
 
+#include "launch.h"
 #include "sigattn_internal.h"
 #include "sigattn_activation.cuh"
 #include "sm100_primitives.cuh"
@@ -121,6 +122,8 @@ sigattn_short_fwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __g
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = tmem_base_slot;
+  grid_dependency_wait();
+  grid_dependency_trigger();
 
   if (warp == kSfLoadWarp) {
     if ((threadIdx.x & 31) == 0) {
@@ -273,8 +276,8 @@ int launch_short_fwd_variant(const CUtensorMap (&maps)[4], const ShortFwdParams&
     configured.fetch_or(bit, std::memory_order_relaxed);
   }
   const int slots = 2 * num_sms;
-  kernel<<<sp.n_units < slots ? sp.n_units : slots, kSfThreads, kSfDynBytes, stream>>>(maps[0], maps[1], maps[2], maps[3], sp);
-  *cuda_err = cudaGetLastError();
+  *cuda_err = launch_after(kernel, dim3(sp.n_units < slots ? sp.n_units : slots), kSfThreads, kSfDynBytes, stream, 0,
+                           maps[0], maps[1], maps[2], maps[3], sp);
   return *cuda_err == cudaSuccess ? SIGATTN_OK : SIGATTN_ERR_CUDA;
 }
 
