@@ -11,6 +11,7 @@
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <memory>
 #include <stdexcept>
 #include <string>
 
@@ -22,6 +23,10 @@ PyObject* g_error = nullptr;   // binding.SigattnError
 
 // A Python exception has been set.
 struct PyError {};
+
+struct Release {
+  void operator()(PyObject* o) const { Py_DECREF(o); }
+};
 
 [[noreturn]] void fail(PyObject* type, const std::string& text) {
   PyErr_SetString(type, text.c_str());
@@ -288,20 +293,20 @@ PyObject* host_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const at::Tensor& d_o = like(a[4], q, "d_o", "q");
     const c10::cuda::OptionalCUDAGuard guard(q.device());
     at::Tensor g[3];
-    PyObject* given[3] = {nullptr, nullptr, nullptr};
+    std::unique_ptr<PyObject, Release> given[3];   // (an iterable other than a list or a tuple may hold no reference itself)
     if (a[12] == Py_None) {
       g[0] = at::empty_like(q);
       g[1] = at::empty_like(*c.k);
       g[2] = at::empty_like(*c.v);
     } else {
       static const char* names[3] = {"dq", "dk", "dv"};
-      PyObject* seq = PySequence_Fast(a[12], "out must be (dq, dk, dv)");
+      const std::unique_ptr<PyObject, Release> seq(PySequence_Fast(a[12], "out must be (dq, dk, dv)"));
       if (!seq) throw PyError();
-      const bool three = PySequence_Fast_GET_SIZE(seq) == 3;
-      for (int i = 0; three && i < 3; ++i) given[i] = PySequence_Fast_GET_ITEM(seq, i);   // (kept alive by the caller's `out`)
-      Py_DECREF(seq);
-      if (!three) bad("out must be (dq, dk, dv)");
-      for (int i = 0; i < 3; ++i) g[i] = like(given[i], i == 0 ? q : *c.k, names[i], i == 0 ? "q" : "k");
+      if (PySequence_Fast_GET_SIZE(seq.get()) != 3) bad("out must be (dq, dk, dv)");
+      for (int i = 0; i < 3; ++i) {
+        given[i].reset(Py_NewRef(PySequence_Fast_GET_ITEM(seq.get(), i)));
+        g[i] = like(given[i].get(), i == 0 ? q : *c.k, names[i], i == 0 ? "q" : "k");
+      }
     }
     const auto f32 = q.options().dtype(at::kFloat);
     at::Tensor dbias, dtemp, hold;
@@ -357,7 +362,7 @@ PyObject* host_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const int extra = c.mode == kPlain ? 0 : c.mode == kDtemp ? 2 : 1;
     PyObject* out = PyTuple_New(3 + extra);
     if (!out) throw PyError();
-    for (int i = 0; i < 3; ++i) PyTuple_SET_ITEM(out, i, given[i] ? Py_NewRef(given[i]) : THPVariable_Wrap(std::move(g[i])));
+    for (int i = 0; i < 3; ++i) PyTuple_SET_ITEM(out, i, given[i] ? given[i].release() : THPVariable_Wrap(std::move(g[i])));
     if (extra == 2) PyTuple_SET_ITEM(out, 3, THPVariable_Wrap(std::move(dtemp)));
     if (extra) PyTuple_SET_ITEM(out, 2 + extra, db ? THPVariable_Wrap(std::move(dbias)) : Py_NewRef(Py_None));
     return out;

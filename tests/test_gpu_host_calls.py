@@ -68,3 +68,28 @@ def test_outputs_and_streams():
             o = sa.sigattn_fwd(late, k, v, *a, stream=side if how == "object" else side.cuda_stream)
         side.synchronize()
         assert torch.equal(o, ref), how
+
+
+@pytest.mark.parametrize("how", ["list", "generator", "map", "stacked tensor"])
+def test_gradients_into_any_iterable_of_three(how):
+    """`out` may be whatever unpacks into three tensors; what the call hands back is alive and is what it wrote, also
+    where the iterable kept no reference to the tensors (freed ones would be handed out again by the allocations here)."""
+    import torch
+    import paper_2409_04431_b200 as sa
+    q, k, v, d_o = _qkv(N=300)
+    a = (1.0 / math.sqrt(64), -math.log(300))
+    ref = sa.sigattn_bwd(q, k, v, d_o, *a)
+    out = {"list": lambda: [torch.empty_like(q) for _ in range(3)], "generator": lambda: (torch.empty_like(q) for _ in range(3)),
+           "map": lambda: map(torch.empty_like, (q, k, v)), "stacked tensor": lambda: torch.empty((3, *q.shape), dtype=q.dtype, device="cuda")}[how]()
+    got = sa.sigattn_bwd(q, k, v, d_o, *a, out=out)
+    later = [torch.full_like(q, 7.0) for _ in range(6)]
+    assert len(got) == 3 and len(later) == 6 and all(isinstance(x, torch.Tensor) for x in got)
+    assert torch.equal(got[1], ref[1]) and torch.equal(got[2], ref[2])
+    assert float((got[0].float() - ref[0].float()).norm() / ref[0].float().norm()) < 1e-3   # dQ: fp32 sums in another order
+    if how == "stacked tensor":
+        assert all(x.data_ptr() == out[i].data_ptr() for i, x in enumerate(got))
+    for wrong in ((q, k), (q, k, v, d_o), iter([q, k])):
+        with pytest.raises(ValueError):
+            sa.sigattn_bwd(q, k, v, d_o, *a, out=wrong)
+    with pytest.raises(TypeError):
+        sa.sigattn_bwd(q, k, v, d_o, *a, out=3)
