@@ -78,6 +78,7 @@ enum Mode : long { kPlain = 0, kBiasVec, kGqa, kNk, kShard, kVarlen, kRagged, kR
 struct Call {
   Mode mode;
   const at::Tensor *q, *k, *v;
+  const void *qp, *kp, *vp;   // their data
   int B, H, H_kv, N_q, N_k, D, dtype;
   float scale, bias = 0.0f;
   const float* bias_vec = nullptr;
@@ -183,23 +184,44 @@ Call parse(PyObject* mode, PyObject* q_, PyObject* k_, PyObject* v_, PyObject* s
     c.slopes = s->const_data_ptr<float>();
   }
   c.stream = stream_of(stream, q);
+  c.qp = q.const_data_ptr();
+  c.kp = c.k->const_data_ptr();
+  c.vp = c.v->const_data_ptr();
   return c;
 }
 
-// The caller's scratch tensor, or one allocated here (kept alive in `hold`) when the call needs any.
-void* workspace_of(PyObject* o, const at::Tensor& q, size_t need, at::Tensor* hold, size_t* bytes) {
-  *bytes = 0;
-  if (o == Py_None) {
-    if (need == 0) return nullptr;
-    *hold = at::empty({static_cast<int64_t>(need)}, q.options().dtype(at::kByte));
-    *bytes = need;
-    return hold->data_ptr();
-  }
+// The caller's scratch tensor, if one was given.
+struct Scratch {
+  void* ptr = nullptr;
+  size_t bytes = 0;
+};
+Scratch given_scratch(PyObject* o, const at::Tensor& q) {
+  if (o == Py_None) return {};
   const at::Tensor* w = tensor_or_null(o);
   if (!side_ok(w, q, at::kByte)) bad("workspace must be a contiguous uint8 CUDA tensor on q's device");
-  *bytes = static_cast<size_t>(w->numel());
-  return w->data_ptr();
+  return {w->data_ptr(), static_cast<size_t>(w->numel())};
 }
+
+// ... or one allocated here when the call needs any.
+at::Tensor own_scratch(const at::Tensor& q, size_t need, Scratch* s) {
+  if (need == 0) return {};
+  at::Tensor t = at::empty({static_cast<int64_t>(need)}, q.options().dtype(at::kByte));
+  *s = {t.data_ptr(), need};
+  return t;
+}
+
+// Allocations and launches run without the interpreter lock: a launch waits when the stream's queue is full, and the
+// other threads of the process (one of them may be what the queue waits for) have to run meanwhile.
+class Unlocked {
+ public:
+  Unlocked() : state_(PyEval_SaveThread()) {}
+  ~Unlocked() { PyEval_RestoreThread(state_); }
+  Unlocked(const Unlocked&) = delete;
+  Unlocked& operator=(const Unlocked&) = delete;
+
+ private:
+  PyThreadState* state_;
+};
 
 void check_rc(int rc) {
   if (rc == SIGATTN_OK) return;
@@ -222,64 +244,94 @@ PyObject* guarded(F f) {
   END_HANDLE_TH_ERRORS
 }
 
+int launch_fwd(const Call& c, void* op, const Scratch& ws) {
+  switch (c.mode) {
+    case kPlain:
+      return sigattn_fwd(c.qp, c.kp, c.vp, op, c.B, c.H, c.N_q, c.D, c.scale, c.bias, c.causal, c.slopes, c.dtype, c.stream);
+    case kBiasVec:
+      return sigattn_fwd_bias_vec(c.qp, c.kp, c.vp, op, c.B, c.H, c.N_q, c.D, c.scale, c.bias_vec, c.causal, c.slopes, c.dtype,
+                                  c.stream);
+    case kGqa:
+      return sigattn_fwd_gqa(c.qp, c.kp, c.vp, op, c.B, c.H, c.H_kv, c.N_q, c.D, c.scale, c.bias, c.bias_vec, c.causal, c.slopes,
+                             c.dtype, c.stream);
+    case kNk:
+      return sigattn_fwd_nk(c.qp, c.kp, c.vp, op, c.B, c.H, c.H_kv, c.N_q, c.N_k, c.D, c.scale, c.bias, c.bias_vec, c.causal,
+                            c.slopes, c.dtype, c.stream);
+    case kShard:
+      return sigattn_fwd_shard(c.qp, c.kp, c.vp, op, c.B, c.H, c.H_kv, c.N_q, c.N_k, c.D, c.scale, c.bias, c.bias_vec, c.causal,
+                               c.pos0, c.slopes, c.dtype, c.stream);
+    case kVarlen:
+      return sigattn_fwd_varlen(c.qp, c.kp, c.vp, op, c.B, c.H, c.H_kv, c.N_q, c.D, c.scale, c.bias, c.bias_vec, c.causal,
+                                c.seqlens, c.slopes, c.dtype, c.stream);
+    case kRagged:
+      return sigattn_fwd_ragged(c.qp, c.kp, c.vp, op, c.H, c.H_kv, c.N_q, c.D, c.cu, c.n_seqs, c.scale, c.bias, c.bias_vec,
+                                c.causal, c.slopes, c.dtype, c.stream);
+    case kRowscale:
+      return sigattn_fwd_rowscale(c.qp, c.kp, c.vp, op, c.B, c.H, c.H_kv, c.N_q, c.N_k, c.D, c.scale, c.bias, c.bias_vec,
+                                  c.causal, c.row_scale, c.slopes, c.dtype, c.stream);
+    case kDecode:
+      return sigattn_fwd_decode(c.qp, c.kp, c.vp, op, c.B, c.H, c.H_kv, c.N_q, c.N_k, c.D, c.scale, c.bias, c.bias_vec, c.causal,
+                                c.slopes, c.dtype, ws.ptr, ws.bytes, c.stream);
+    default:
+      return SIGATTN_ERR_FLAG;
+  }
+}
+
+int launch_bwd(const Call& c, const void* dop, void* dq, void* dk, void* dv, float* db, float* dtemp, const Scratch& ws) {
+  switch (c.mode) {
+    case kPlain:
+      return sigattn_bwd(c.qp, c.kp, c.vp, dop, dq, dk, dv, c.B, c.H, c.N_q, c.D, c.scale, c.bias, c.causal, c.slopes, c.dtype, ws.ptr,
+                         ws.bytes, c.stream);
+    case kBiasVec:
+      return sigattn_bwd_bias_vec(c.qp, c.kp, c.vp, dop, dq, dk, dv, c.B, c.H, c.N_q, c.D, c.scale, c.bias_vec, c.causal, c.slopes,
+                                  c.dtype, db, ws.ptr, ws.bytes, c.stream);
+    case kGqa:
+      return sigattn_bwd_gqa(c.qp, c.kp, c.vp, dop, dq, dk, dv, c.B, c.H, c.H_kv, c.N_q, c.D, c.scale, c.bias, c.bias_vec, c.causal,
+                             c.slopes, c.dtype, db, ws.ptr, ws.bytes, c.stream);
+    case kNk:
+      return sigattn_bwd_nk(c.qp, c.kp, c.vp, dop, dq, dk, dv, c.B, c.H, c.H_kv, c.N_q, c.N_k, c.D, c.scale, c.bias, c.bias_vec,
+                            c.causal, c.slopes, c.dtype, db, ws.ptr, ws.bytes, c.stream);
+    case kShard:
+      return sigattn_bwd_shard(c.qp, c.kp, c.vp, dop, dq, dk, dv, c.B, c.H, c.H_kv, c.N_q, c.N_k, c.D, c.scale, c.bias, c.bias_vec,
+                               c.causal, c.pos0, c.slopes, c.dtype, db, ws.ptr, ws.bytes, c.stream);
+    case kVarlen:
+      return sigattn_bwd_varlen(c.qp, c.kp, c.vp, dop, dq, dk, dv, c.B, c.H, c.H_kv, c.N_q, c.D, c.scale, c.bias, c.bias_vec,
+                                c.causal, c.seqlens, c.slopes, c.dtype, db, ws.ptr, ws.bytes, c.stream);
+    case kRagged:
+      return sigattn_bwd_ragged(c.qp, c.kp, c.vp, dop, dq, dk, dv, c.H, c.H_kv, c.N_q, c.D, c.cu, c.n_seqs, c.scale, c.bias,
+                                c.bias_vec, c.causal, c.slopes, c.dtype, db, ws.ptr, ws.bytes, c.stream);
+    case kRowscale:
+      return sigattn_bwd_rowscale(c.qp, c.kp, c.vp, dop, dq, dk, dv, c.B, c.H, c.H_kv, c.N_q, c.N_k, c.D, c.scale, c.bias,
+                                  c.bias_vec, c.causal, c.row_scale, c.slopes, c.dtype, db, ws.ptr, ws.bytes, c.stream);
+    case kDtemp:
+      return sigattn_bwd_dtemp(c.qp, c.kp, c.vp, dop, dq, dk, dv, c.B, c.H, c.N_q, c.D, c.scale, c.bias, c.bias_vec, c.causal,
+                               c.slopes, c.dtype, db, dtemp, ws.ptr, ws.bytes, c.stream);
+    default:
+      return SIGATTN_ERR_FLAG;
+  }
+}
+
 // fwd(mode, q, k, v, scale, bias, causal, slopes, aux, workspace, out, stream) -> O
 PyObject* host_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
   return guarded([&]() -> PyObject* {
     if (n != 12) fail(PyExc_TypeError, "fwd takes 12 arguments");
     const Call c = parse(a[0], a[1], a[2], a[3], a[4], a[5], a[6], a[7], a[8], a[11]);
-    const at::Tensor& q = *c.q;
-    const c10::cuda::OptionalCUDAGuard guard(q.device());
-    at::Tensor made, hold;
-    if (a[10] == Py_None) made = at::empty_like(q);
-    else like(a[10], q, "out", "q");
-    const at::Tensor& out = a[10] == Py_None ? made : THPVariable_Unpack(a[10]);
-    const void *qp = q.const_data_ptr(), *kp = c.k->const_data_ptr(), *vp = c.v->const_data_ptr();
-    void* op = out.data_ptr();
-    int rc = SIGATTN_ERR_FLAG;
-    switch (c.mode) {
-      case kPlain:
-        rc = sigattn_fwd(qp, kp, vp, op, c.B, c.H, c.N_q, c.D, c.scale, c.bias, c.causal, c.slopes, c.dtype, c.stream);
-        break;
-      case kBiasVec:
-        rc = sigattn_fwd_bias_vec(qp, kp, vp, op, c.B, c.H, c.N_q, c.D, c.scale, c.bias_vec, c.causal, c.slopes, c.dtype,
-                                  c.stream);
-        break;
-      case kGqa:
-        rc = sigattn_fwd_gqa(qp, kp, vp, op, c.B, c.H, c.H_kv, c.N_q, c.D, c.scale, c.bias, c.bias_vec, c.causal, c.slopes,
-                             c.dtype, c.stream);
-        break;
-      case kNk:
-        rc = sigattn_fwd_nk(qp, kp, vp, op, c.B, c.H, c.H_kv, c.N_q, c.N_k, c.D, c.scale, c.bias, c.bias_vec, c.causal,
-                            c.slopes, c.dtype, c.stream);
-        break;
-      case kShard:
-        rc = sigattn_fwd_shard(qp, kp, vp, op, c.B, c.H, c.H_kv, c.N_q, c.N_k, c.D, c.scale, c.bias, c.bias_vec, c.causal,
-                               c.pos0, c.slopes, c.dtype, c.stream);
-        break;
-      case kVarlen:
-        rc = sigattn_fwd_varlen(qp, kp, vp, op, c.B, c.H, c.H_kv, c.N_q, c.D, c.scale, c.bias, c.bias_vec, c.causal,
-                                c.seqlens, c.slopes, c.dtype, c.stream);
-        break;
-      case kRagged:
-        rc = sigattn_fwd_ragged(qp, kp, vp, op, c.H, c.H_kv, c.N_q, c.D, c.cu, c.n_seqs, c.scale, c.bias, c.bias_vec,
-                                c.causal, c.slopes, c.dtype, c.stream);
-        break;
-      case kRowscale:
-        rc = sigattn_fwd_rowscale(qp, kp, vp, op, c.B, c.H, c.H_kv, c.N_q, c.N_k, c.D, c.scale, c.bias, c.bias_vec,
-                                  c.causal, c.row_scale, c.slopes, c.dtype, c.stream);
-        break;
-      case kDecode: {
-        size_t bytes = 0;
-        void* ws = workspace_of(a[9], q, sigattn_fwd_decode_workspace_bytes(c.B, c.H, c.N_q, c.D, c.dtype), &hold, &bytes);
-        rc = sigattn_fwd_decode(qp, kp, vp, op, c.B, c.H, c.H_kv, c.N_q, c.N_k, c.D, c.scale, c.bias, c.bias_vec, c.causal,
-                                c.slopes, c.dtype, ws, bytes, c.stream);
-        break;
-      }
-      default:
-        break;
+    const bool given = a[10] != Py_None, decode = c.mode == kDecode;
+    at::Tensor out;
+    if (given) out = like(a[10], *c.q, "out", "q");
+    Scratch ws = given_scratch(decode ? a[9] : Py_None, *c.q);
+    int rc;
+    {
+      const Unlocked unlocked;
+      const c10::cuda::OptionalCUDAGuard guard(c.q->device());
+      if (!given) out = at::empty_like(*c.q);
+      at::Tensor hold;
+      if (decode && a[9] == Py_None)
+        hold = own_scratch(*c.q, sigattn_fwd_decode_workspace_bytes(c.B, c.H, c.N_q, c.D, c.dtype), &ws);
+      rc = launch_fwd(c, out.data_ptr(), ws);
     }
     check_rc(rc);
-    return a[10] == Py_None ? THPVariable_Wrap(std::move(made)) : Py_NewRef(a[10]);
+    return given ? Py_NewRef(a[10]) : THPVariable_Wrap(std::move(out));
   });
 }
 
@@ -290,15 +342,10 @@ PyObject* host_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (n != 14) fail(PyExc_TypeError, "bwd takes 14 arguments");
     const Call c = parse(a[0], a[1], a[2], a[3], a[5], a[6], a[7], a[8], a[9], a[13]);
     const at::Tensor& q = *c.q;
-    const at::Tensor& d_o = like(a[4], q, "d_o", "q");
-    const c10::cuda::OptionalCUDAGuard guard(q.device());
+    const void* dop = like(a[4], q, "d_o", "q").const_data_ptr();
     at::Tensor g[3];
     std::unique_ptr<PyObject, Release> given[3];   // (an iterable other than a list or a tuple may hold no reference itself)
-    if (a[12] == Py_None) {
-      g[0] = at::empty_like(q);
-      g[1] = at::empty_like(*c.k);
-      g[2] = at::empty_like(*c.v);
-    } else {
+    if (a[12] != Py_None) {
       static const char* names[3] = {"dq", "dk", "dv"};
       const std::unique_ptr<PyObject, Release> seq(PySequence_Fast(a[12], "out must be (dq, dk, dv)"));
       if (!seq) throw PyError();
@@ -308,63 +355,30 @@ PyObject* host_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
         g[i] = like(given[i].get(), i == 0 ? q : *c.k, names[i], i == 0 ? "q" : "k");
       }
     }
-    const auto f32 = q.options().dtype(at::kFloat);
-    at::Tensor dbias, dtemp, hold;
-    if (truth(a[10])) dbias = at::empty({c.cu ? c.n_seqs : c.B, c.H}, f32);
-    if (c.mode == kDtemp) dtemp = at::empty({c.B, c.H}, f32);
-    float* db = dbias.defined() ? dbias.data_ptr<float>() : nullptr;
-    size_t bytes = 0;
-    void* ws = workspace_of(a[11], q, sigattn_bwd_workspace_bytes(c.B, c.H, c.N_q, c.D, c.dtype), &hold, &bytes);
-    const void *qp = q.const_data_ptr(), *kp = c.k->const_data_ptr(), *vp = c.v->const_data_ptr(), *dop = d_o.const_data_ptr();
-    void *dq = g[0].data_ptr(), *dk = g[1].data_ptr(), *dv = g[2].data_ptr();
-    int rc = SIGATTN_ERR_FLAG;
-    switch (c.mode) {
-      case kPlain:
-        rc = sigattn_bwd(qp, kp, vp, dop, dq, dk, dv, c.B, c.H, c.N_q, c.D, c.scale, c.bias, c.causal, c.slopes, c.dtype, ws,
-                         bytes, c.stream);
-        break;
-      case kBiasVec:
-        rc = sigattn_bwd_bias_vec(qp, kp, vp, dop, dq, dk, dv, c.B, c.H, c.N_q, c.D, c.scale, c.bias_vec, c.causal, c.slopes,
-                                  c.dtype, db, ws, bytes, c.stream);
-        break;
-      case kGqa:
-        rc = sigattn_bwd_gqa(qp, kp, vp, dop, dq, dk, dv, c.B, c.H, c.H_kv, c.N_q, c.D, c.scale, c.bias, c.bias_vec, c.causal,
-                             c.slopes, c.dtype, db, ws, bytes, c.stream);
-        break;
-      case kNk:
-        rc = sigattn_bwd_nk(qp, kp, vp, dop, dq, dk, dv, c.B, c.H, c.H_kv, c.N_q, c.N_k, c.D, c.scale, c.bias, c.bias_vec,
-                            c.causal, c.slopes, c.dtype, db, ws, bytes, c.stream);
-        break;
-      case kShard:
-        rc = sigattn_bwd_shard(qp, kp, vp, dop, dq, dk, dv, c.B, c.H, c.H_kv, c.N_q, c.N_k, c.D, c.scale, c.bias, c.bias_vec,
-                               c.causal, c.pos0, c.slopes, c.dtype, db, ws, bytes, c.stream);
-        break;
-      case kVarlen:
-        rc = sigattn_bwd_varlen(qp, kp, vp, dop, dq, dk, dv, c.B, c.H, c.H_kv, c.N_q, c.D, c.scale, c.bias, c.bias_vec,
-                                c.causal, c.seqlens, c.slopes, c.dtype, db, ws, bytes, c.stream);
-        break;
-      case kRagged:
-        rc = sigattn_bwd_ragged(qp, kp, vp, dop, dq, dk, dv, c.H, c.H_kv, c.N_q, c.D, c.cu, c.n_seqs, c.scale, c.bias,
-                                c.bias_vec, c.causal, c.slopes, c.dtype, db, ws, bytes, c.stream);
-        break;
-      case kRowscale:
-        rc = sigattn_bwd_rowscale(qp, kp, vp, dop, dq, dk, dv, c.B, c.H, c.H_kv, c.N_q, c.N_k, c.D, c.scale, c.bias,
-                                  c.bias_vec, c.causal, c.row_scale, c.slopes, c.dtype, db, ws, bytes, c.stream);
-        break;
-      case kDtemp:
-        rc = sigattn_bwd_dtemp(qp, kp, vp, dop, dq, dk, dv, c.B, c.H, c.N_q, c.D, c.scale, c.bias, c.bias_vec, c.causal,
-                               c.slopes, c.dtype, db, dtemp.data_ptr<float>(), ws, bytes, c.stream);
-        break;
-      default:
-        break;
+    const bool want_dbias = truth(a[10]), want_dtemp = c.mode == kDtemp;
+    Scratch ws = given_scratch(a[11], q);
+    at::Tensor dbias, dtemp;
+    int rc;
+    {
+      const Unlocked unlocked;
+      const c10::cuda::OptionalCUDAGuard guard(q.device());
+      for (int i = 0; i < 3; ++i)
+        if (!given[i]) g[i] = at::empty_like(i == 0 ? q : *c.k);
+      const auto f32 = q.options().dtype(at::kFloat);
+      if (want_dbias) dbias = at::empty({c.cu ? c.n_seqs : c.B, c.H}, f32);
+      if (want_dtemp) dtemp = at::empty({c.B, c.H}, f32);
+      at::Tensor hold;
+      if (a[11] == Py_None) hold = own_scratch(q, sigattn_bwd_workspace_bytes(c.B, c.H, c.N_q, c.D, c.dtype), &ws);
+      rc = launch_bwd(c, dop, g[0].data_ptr(), g[1].data_ptr(), g[2].data_ptr(), want_dbias ? dbias.data_ptr<float>() : nullptr,
+                      want_dtemp ? dtemp.data_ptr<float>() : nullptr, ws);
     }
     check_rc(rc);
-    const int extra = c.mode == kPlain ? 0 : c.mode == kDtemp ? 2 : 1;
+    const int extra = c.mode == kPlain ? 0 : want_dtemp ? 2 : 1;
     PyObject* out = PyTuple_New(3 + extra);
     if (!out) throw PyError();
     for (int i = 0; i < 3; ++i) PyTuple_SET_ITEM(out, i, given[i] ? given[i].release() : THPVariable_Wrap(std::move(g[i])));
     if (extra == 2) PyTuple_SET_ITEM(out, 3, THPVariable_Wrap(std::move(dtemp)));
-    if (extra) PyTuple_SET_ITEM(out, 2 + extra, db ? THPVariable_Wrap(std::move(dbias)) : Py_NewRef(Py_None));
+    if (extra) PyTuple_SET_ITEM(out, 2 + extra, want_dbias ? THPVariable_Wrap(std::move(dbias)) : Py_NewRef(Py_None));
     return out;
   });
 }

@@ -93,3 +93,48 @@ def test_gradients_into_any_iterable_of_three(how):
             sa.sigattn_bwd(q, k, v, d_o, *a, out=wrong)
     with pytest.raises(TypeError):
         sa.sigattn_bwd(q, k, v, d_o, *a, out=3)
+
+
+@pytest.mark.parametrize("what", ["forward", "backward"])
+def test_other_threads_run_while_a_launch_waits(what):
+    """A launch blocks when the stream's queue is full; the calls do not hold the interpreter lock meanwhile.  The stream
+    is kept busy for about half a second and more launches are queued than it takes; the longest pause of a thread that
+    only counts has to be far shorter than the wait (the interpreter's own switch interval is 5 ms)."""
+    import threading
+    import time
+    import torch
+    import paper_2409_04431_b200 as sa
+    q, k, v, d_o = _qkv()
+    o, grads = torch.empty_like(q), tuple(torch.empty_like(q) for _ in range(3))
+    a = (0.125, -3.0)
+    call = {"forward": lambda: sa.sigattn_fwd(q, k, v, *a, out=o), "backward": lambda: sa.sigattn_bwd(q, k, v, d_o, *a, out=grads)}[what]
+    call()
+    torch.cuda.synchronize()
+    stop, pauses = threading.Event(), []
+
+    def count():
+        last = time.perf_counter()
+        while not stop.is_set():
+            time.sleep(0.0005)
+            now = time.perf_counter()
+            pauses.append(now - last)
+            last = now
+
+    counter = threading.Thread(target=count)
+    counter.start()
+    try:
+        torch.cuda._sleep(1_000_000_000)
+        t0 = time.perf_counter()
+        longest = 0.0
+        for _ in range(4000):
+            t1 = time.perf_counter()
+            call()
+            longest = max(longest, time.perf_counter() - t1)
+            if time.perf_counter() - t0 > 5.0:
+                break
+    finally:
+        stop.set()
+        counter.join()
+        torch.cuda.synchronize()
+    assert longest > 0.2, longest          # some launch did wait for the queue
+    assert max(pauses) < 0.5 * longest, (max(pauses), longest)
