@@ -202,6 +202,24 @@ def _stream_ptr(stream):
     return stream.cuda_stream
 
 
+def _results(stream, device, make):
+    """make() -> a list of tensors (or None) that a call on `stream` writes: allocated as that stream's memory where it is not
+    the current one, and known to the allocator as used on the current one too."""
+    if stream is None:
+        return make()
+    handle = _stream_ptr(stream)
+    with torch.cuda.device(device):
+        current = torch.cuda.current_stream()
+        if handle in (current.cuda_stream, 1, 2):   # (1, 2: handles of the legacy and the per-thread stream)
+            return make()
+        with torch.cuda.stream(torch.cuda.ExternalStream(handle)):
+            made = make()
+        for t in made:
+            if t is not None:
+                t.record_stream(current)
+    return made
+
+
 def _dtype_code(t) -> int:
     if t.dtype == torch.bfloat16:
         return DTYPE_BF16
@@ -432,8 +450,8 @@ def sigattn_bwd_shard_acc(q, k, v, d_o, dq_acc, scale, bias, pos0, causal=False,
     vec = isinstance(bias, torch.Tensor)
     if vec:
         _check_bias_vec(bias, q)
-    dk, dv = torch.empty_like(k), torch.empty_like(v)
-    dbias = torch.empty((B, H), dtype=torch.float32, device=q.device) if want_dbias else None
+    dk, dv, dbias = _results(stream, q.device, lambda: [
+        torch.empty_like(k), torch.empty_like(v), torch.empty((B, H), dtype=torch.float32, device=q.device) if want_dbias else None])
     with torch.cuda.device(q.device):
         rc = _lib.sigattn_bwd_shard_acc(_ptr(q), _ptr(k), _ptr(v), _ptr(d_o), _ptr(dq_acc), _ptr(dk), _ptr(dv), B, H,
                                         H_kv, N_q, N_k, D, float(scale), 0.0 if vec else float(bias),
@@ -458,7 +476,7 @@ def sigattn_bwd_shard_acc_kv(q, k, v, d_o, dq_acc, dk, dv, scale, bias, pos0, ca
     vec = isinstance(bias, torch.Tensor)
     if vec:
         _check_bias_vec(bias, q)
-    dbias = torch.empty((B, H), dtype=torch.float32, device=q.device) if want_dbias else None
+    dbias, = _results(stream, q.device, lambda: [torch.empty((B, H), dtype=torch.float32, device=q.device) if want_dbias else None])
     with torch.cuda.device(q.device):
         rc = _lib.sigattn_bwd_shard_acc_kv(_ptr(q), _ptr(k), _ptr(v), _ptr(d_o), _ptr(dq_acc), _ptr(dk), _ptr(dv), B,
                                            H, H_kv, N_q, N_k, D, float(scale), 0.0 if vec else float(bias),
@@ -474,7 +492,7 @@ def sigattn_acc_to_bf16(acc, mul=1.0, out=None, stream=None):
     if not isinstance(acc, torch.Tensor) or acc.dtype != torch.float32 or not acc.is_cuda or not acc.is_contiguous():
         raise ValueError("acc must be a contiguous float32 CUDA tensor")
     if out is None:
-        out = torch.empty(acc.shape, dtype=torch.bfloat16, device=acc.device)
+        out, = _results(stream, acc.device, lambda: [torch.empty(acc.shape, dtype=torch.bfloat16, device=acc.device)])
     with torch.cuda.device(acc.device):
         rc = _lib.sigattn_acc_to_bf16(_ptr(acc), _ptr(out), acc.numel(), float(mul), _stream_ptr(stream))
     if rc != 0:
@@ -495,7 +513,7 @@ def sigattn_fwd_decode(q, k, v, scale, bias, causal=False, alibi_slopes=None, wo
 def sigattn_seqlen_norm(n_q, n_k, alpha, causal, device, stream=None):
     """The paper's row factors of the sequence-length normalisation as a float32 CUDA [n_q]:
     n_k^-alpha without a mask, (position + 1)^-alpha with the causal mask."""
-    out = torch.empty(int(n_q), dtype=torch.float32, device=device)
+    out, = _results(stream, device, lambda: [torch.empty(int(n_q), dtype=torch.float32, device=device)])
     with torch.cuda.device(out.device):
         rc = _lib.sigattn_seqlen_norm(_ptr(out), int(n_q), int(n_k), float(alpha), int(bool(causal)),
                                       _stream_ptr(stream))
@@ -567,7 +585,7 @@ def sigattn_bwd_static_scratch(q, k, v, d_o, scale, bias, causal=False, alibi_sl
     _check_same([q, k, v, d_o], ["q", "k", "v", "d_o"])
     B, H, N, D = q.shape
     if out is None:
-        dq, dk, dv = torch.empty_like(q), torch.empty_like(q), torch.empty_like(q)
+        dq, dk, dv = _results(stream, q.device, lambda: [torch.empty_like(q) for _ in range(3)])
     else:
         dq, dk, dv = out
         _check_same([q, dq, dk, dv], ["q", "dq", "dk", "dv"])

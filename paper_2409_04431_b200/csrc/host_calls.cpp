@@ -6,6 +6,7 @@
 #include <Python.h>
 
 #include <ATen/ATen.h>
+#include <c10/cuda/CUDACachingAllocator.h>
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Exceptions.h>
@@ -223,6 +224,29 @@ class Unlocked {
   PyThreadState* state_;
 };
 
+// Memory that a call allocates is used on the call's stream.  Where that is not the current one, it is made the
+// current one for the allocations: the allocator then hands out memory that is free in that stream's order, and takes
+// scratch back in that order.  Results are used on the caller's current stream as well, which the allocator is told.
+class OnStream {
+ public:
+  OnStream(const at::Tensor& q, void* stream) : device_(q.device()), current_(c10::cuda::getCurrentCUDAStream(device_.index())) {
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (s == cudaStreamPerThread) return;   // (the allocator knows no such stream)
+    if (s == cudaStreamLegacy) s = nullptr;
+    if (s != current_.stream()) other_.reset_stream(c10::cuda::getStreamFromExternal(s, device_.index()));
+  }
+  at::Tensor result(at::Tensor t) const {
+    if (other_.current_stream()) c10::cuda::CUDACachingAllocator::recordStream(t.storage().data_ptr(), current_);
+    return t;
+  }
+
+ private:
+  c10::Device device_;
+  c10::cuda::CUDAStream current_;
+  c10::cuda::CUDAGuard on_device_{device_};
+  c10::cuda::OptionalCUDAStreamGuard other_;
+};
+
 void check_rc(int rc) {
   if (rc == SIGATTN_OK) return;
   PyObject* e = PyObject_CallFunction(g_error, "i", rc);
@@ -323,8 +347,8 @@ PyObject* host_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     int rc;
     {
       const Unlocked unlocked;
-      const c10::cuda::OptionalCUDAGuard guard(c.q->device());
-      if (!given) out = at::empty_like(*c.q);
+      const OnStream on(*c.q, c.stream);
+      if (!given) out = on.result(at::empty_like(*c.q));
       at::Tensor hold;
       if (decode && a[9] == Py_None)
         hold = own_scratch(*c.q, sigattn_fwd_decode_workspace_bytes(c.B, c.H, c.N_q, c.D, c.dtype), &ws);
@@ -361,12 +385,12 @@ PyObject* host_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     int rc;
     {
       const Unlocked unlocked;
-      const c10::cuda::OptionalCUDAGuard guard(q.device());
+      const OnStream on(q, c.stream);
       for (int i = 0; i < 3; ++i)
-        if (!given[i]) g[i] = at::empty_like(i == 0 ? q : *c.k);
+        if (!given[i]) g[i] = on.result(at::empty_like(i == 0 ? q : *c.k));
       const auto f32 = q.options().dtype(at::kFloat);
-      if (want_dbias) dbias = at::empty({c.cu ? c.n_seqs : c.B, c.H}, f32);
-      if (want_dtemp) dtemp = at::empty({c.B, c.H}, f32);
+      if (want_dbias) dbias = on.result(at::empty({c.cu ? c.n_seqs : c.B, c.H}, f32));
+      if (want_dtemp) dtemp = on.result(at::empty({c.B, c.H}, f32));
       at::Tensor hold;
       if (a[11] == Py_None) hold = own_scratch(q, sigattn_bwd_workspace_bytes(c.B, c.H, c.N_q, c.D, c.dtype), &ws);
       rc = launch_bwd(c, dop, g[0].data_ptr(), g[1].data_ptr(), g[2].data_ptr(), want_dbias ? dbias.data_ptr<float>() : nullptr,

@@ -138,3 +138,57 @@ def test_other_threads_run_while_a_launch_waits(what):
         torch.cuda.synchronize()
     assert longest > 0.2, longest          # some launch did wait for the queue
     assert max(pauses) < 0.5 * longest, (max(pauses), longest)
+
+
+@pytest.mark.parametrize("how", ["object", "handle"])
+@pytest.mark.parametrize("what", ["backward", "decode", "forward", "static scratch"])
+def test_memory_of_calls_on_another_stream(what, how):
+    """An explicit stream that is not the current one, with everything allocated by the call: its scratch and results
+    share no memory with what the current stream has in use, before the call or after it."""
+    import torch
+    import paper_2409_04431_b200 as sa
+    spin = 100_000_000   # about 50 ms
+    B, H, N, D = (2, 8, 400, 64) if what != "decode" else (1, 2, 1, 128)   # the latter: sums of several clusters in scratch
+    g = torch.Generator(device="cuda").manual_seed(3)
+    q, d_o = (torch.randn((B, H, N, D), generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
+    k, v = (torch.randn((B, H, 70000 if what == "decode" else N, D), generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
+    a = (1.0 / math.sqrt(D), -math.log(k.shape[2]))
+    call = {"backward": lambda **x: sa.sigattn_bwd(q, k, v, d_o, *a, **x)[0], "forward": lambda **x: sa.sigattn_fwd(q, k, v, *a, **x),
+            "decode": lambda **x: sa.sigattn_fwd_decode(q, k, v, *a, **x),
+            "static scratch": lambda **x: sa.sigattn_bwd_static_scratch(q, k, v, d_o, *a, **x)[0]}[what]
+    ref = call()
+    side = torch.cuda.Stream()
+    stream = side if how == "object" else side.cuda_stream
+    scratch = {"backward": sa.sigattn_bwd_workspace_bytes(B, H, N, D, 0), "decode": sa.sigattn_fwd_decode_workspace_bytes(B, H, N, D, 0)}.get(what, 0)
+    sizes = [n for n in (scratch, q.numel() * 2) if n]
+
+    def close(x):
+        return float((x.float() - ref.float()).norm() / ref.float().norm()) < 1e-3   # (fp32 sums in another order)
+
+    torch.cuda.synchronize()
+    # memory that the current stream still writes when the call on the other one has long ended
+    before = [torch.empty(n, dtype=torch.uint8, device="cuda") for n in sizes for _ in range(3)]
+    torch.cuda._sleep(spin)
+    for x in before:
+        x.fill_(255)
+    del before, x
+    got = call(stream=stream)
+    torch.cuda.synchronize()
+    assert close(got)
+    # memory that the current stream takes and fills while the call's kernels have not begun
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(spin)
+    got = call(stream=stream)
+    after = [torch.full((n,), 7, dtype=torch.uint8, device="cuda") for n in sizes for _ in range(3)]
+    torch.cuda.synchronize()
+    assert close(got) and all(bool((x == 7).all()) for x in after)
+    # a result that the current stream still reads when it is dropped
+    torch.cuda.current_stream().wait_stream(side)
+    torch.cuda._sleep(spin)
+    kept = got.clone()
+    del got
+    with torch.cuda.stream(side):
+        later = [torch.zeros_like(q) for _ in range(6)]
+    torch.cuda.synchronize()
+    assert close(kept) and len(later) == 6
+    sa.sigattn_check()
