@@ -101,10 +101,10 @@ struct BwdBarriers {
   uint64_t dq_full[2], dq_empty[2];
   uint64_t dkv_full, dkv_empty;
   uint64_t stage_full, stage_empty;   // wide: the dQ staging boxes between the activation groups and the storing thread
-  // dynamic schedule (batches without padding): the TMA thread draws the next work item from a
-  // global counter and hands it to the other roles through this two-slot ring
-  uint64_t sched_full[2], sched_empty[2];
+  // dynamic schedule: the TMA thread draws the next work item and hands it to the other roles through this two-slot ring
+  uint64_t sched_full[2], sched_empty[2], sched_answer;
   int sched_item[2];
+  __align__(16) uint32_t sched_response[4];
 };
 
 struct BwdParams {
@@ -118,7 +118,7 @@ struct BwdParams {
   // bias_vec and dbias then hold one entry per (sequence, head)
   const int* cu_seqlens;
   int n_seqs;
-  int* sched_counter;   // dynamic schedule: next work item to hand out (zero at launch), or nullptr
+  int dynamic;     // 1: work items are drawn, one thread block of the grid per item (see bwd_sched_draw)
   // Few (batch, key/value head) pairs (multi-query attention at a small batch): the query heads of a
   // group are split over n_sub work items of heads_per_sub heads each, which add their dK_j, dV_j
   // (bf16 TMA reduce-adds into the cleared outputs) instead of storing them.  n_sub = 1: off.
@@ -156,21 +156,24 @@ __device__ __forceinline__ int bwd_snake_rank(int round, int n_items) {
 
 __device__ __forceinline__ int bwd_num_rounds(int n_items) { return (n_items + gridDim.x - 1) / gridDim.x; }
 
-// Dynamic schedule: the CTAs draw items from a global counter in the order of their numbers.  Used where the static
-// order above does not sort by cost: in batches without padding, where the cost follows the position of the key tile
-// inside its own sequence, and when heads are handed out in groups.  One thread per CTA draws; the MMA thread, the
-// activation groups and the drain group read the item from a two-slot ring.  false: a bounded wait expired;
-// *item < 0: none left.
+// Dynamic schedule, used where the static order above does not sort by cost: in batches without padding, where the
+// cost follows the position of the key tile inside its own sequence, and when heads are handed out in groups.  The
+// grid has one thread block per item; those that start take over the others in order (cluster launch control, as in
+// the forward).  One thread per CTA draws; the MMA thread, the activation groups and the drain group read the item
+// from a two-slot ring.  false: a bounded wait expired; *item < 0: none left.
 __device__ __forceinline__ bool bwd_sched_draw(const BwdParams& p, BwdBarriers* bars, int round, int* item,
                                                volatile int* cta_err) {
   const uint32_t slot = round & 1, phase = (round >> 1) & 1;
   if (!mbar_wait(smem_u32(&bars->sched_empty[slot]), phase ^ 1, cta_err, 70)) return false;
-  int it = atomicAdd(p.sched_counter, 1);
-  // every thread block draws until its first value >= n_items, so one launch draws n_items + gridDim.x
-  // values in all; a larger value means another launch in flight shares the counter (more launches
-  // overlapping than the library has counters): report it instead of silently skipping or repeating items
-  if (it >= p.n_items + static_cast<int>(gridDim.x)) *cta_err = 76;
-  if (it >= p.n_items) it = -1;
+  int it = blockIdx.x;
+  if (round > 0) {
+    const uint32_t response = smem_u32(bars->sched_response), bar = smem_u32(&bars->sched_answer);
+    mbar_arrive_expect_tx(bar, 16);
+    clc_try_cancel(response, bar);
+    if (!mbar_wait(bar, (round - 1) & 1, cta_err, 76)) return false;
+    it = clc_block(response);
+    fence_proxy_async_smem();   // the answer has been read before the next one is written there
+  }
   *reinterpret_cast<volatile int*>(&bars->sched_item[slot]) = it;
   mbar_arrive(smem_u32(&bars->sched_full[slot]));
   *item = it;
@@ -312,7 +315,7 @@ __device__ void bwd_load_role(const BwdParams& p, const CUtensorMap* tmQ, const 
     ++do_cnt;
     return true;
   };
-  const bool dynamic = p.sched_counter != nullptr;
+  const bool dynamic = p.dynamic != 0;
   for (int round = 0, rounds = bwd_num_rounds(p.n_items); dynamic || round < rounds; ++round) {
     int item;
     if (dynamic) {
@@ -421,7 +424,7 @@ __device__ void bwd_mma_role(const BwdParams& p, uint32_t smem_base, uint32_t tm
     return true;
   };
 
-  const bool dynamic = p.sched_counter != nullptr;
+  const bool dynamic = p.dynamic != 0;
   for (int round = 0, rounds = bwd_num_rounds(p.n_items); dynamic || round < rounds; ++round) {
     int item;
     if (dynamic) {
@@ -551,7 +554,7 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
     return true;
   };
 
-  const bool dynamic = p.sched_counter != nullptr;
+  const bool dynamic = p.dynamic != 0;
   for (int round = 0, rounds = bwd_num_rounds(p.n_items); dynamic || round < rounds; ++round) {
     int item;
     if (dynamic) {
@@ -719,7 +722,7 @@ __device__ void bwd_drain_role(const BwdParams& p, const CUtensorMap* tmW, uint8
   const int tid = threadIdx.x & 127;  // query row within the tile
   const uint32_t lane_off = static_cast<uint32_t>(((threadIdx.x >> 5) & 3) * 32) << 16;
   uint32_t step_cnt = 0;
-  const bool dynamic = p.sched_counter != nullptr;
+  const bool dynamic = p.dynamic != 0;
   for (int round = 0, rounds = bwd_num_rounds(p.n_items); dynamic || round < rounds; ++round) {
     int item;
     if (dynamic) {
@@ -780,7 +783,7 @@ __device__ void bwd_store_role(const BwdParams& p, const CUtensorMap* tmW, uint3
                                volatile int* cta_err) {
   using L = BwdSmem<D>;
   uint32_t step_cnt = 0;
-  const bool dynamic = p.sched_counter != nullptr;
+  const bool dynamic = p.dynamic != 0;
   for (int round = 0, rounds = bwd_num_rounds(p.n_items); dynamic || round < rounds; ++round) {
     int item;
     if (dynamic) {
@@ -855,6 +858,7 @@ sigattn_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       mbar_init(smem_u32(&bars.sched_full[s]), 1);
       mbar_init(smem_u32(&bars.sched_empty[s]), BwdRoles<D, WIDE>::kSchedConsumers);
     }
+    mbar_init(smem_u32(&bars.sched_answer), 1);
     fence_mbar_init();
   }
   if (warp == R::kLoadWarp && elect_one()) {
@@ -971,10 +975,6 @@ sigattn_bwd_scale_rows_kernel(const uint4* __restrict__ d_o, const float* __rest
 // What the items in work at a time may touch of Q, dO and the dQ accumulator.
 constexpr size_t kBwdL2Share = 64u << 20;
 
-// Work-item counters of the dynamic schedule: one per launch in flight, handed out round robin.
-constexpr int kBwdSchedSlots = 1024;
-__device__ int g_bwd_sched_counters[kBwdSchedSlots];
-
 template <int D, bool CAUSAL, bool ALIBI, bool DBIAS, int KIND, bool WIDE>
 int launch_bwd_variant(const CUtensorMap* maps, const BwdParams& bp, int num_sms, cudaStream_t stream,
                        cudaError_t* cuda_err) {
@@ -991,7 +991,7 @@ int launch_bwd_variant(const CUtensorMap* maps, const BwdParams& bp, int num_sms
     if (*cuda_err != cudaSuccess) return SIGATTN_ERR_CUDA;
     configured.fetch_or(bit, std::memory_order_relaxed);
   }
-  const int grid = bp.n_items < num_sms ? bp.n_items : num_sms;
+  const int grid = (bp.dynamic || bp.n_items < num_sms) ? bp.n_items : num_sms;
   *cuda_err = launch_after(kernel, dim3(grid), BwdRoles<D, WIDE>::kThreads, BwdSmem<D>::kDynBytes, stream, 0, maps[0], maps[1],
                            maps[2], maps[3], maps[4], maps[5], maps[6], bp);
   return *cuda_err == cudaSuccess ? SIGATTN_OK : SIGATTN_ERR_CUDA;
@@ -1108,7 +1108,6 @@ int launch_bwd_bf16(const void* q, const void* k, const void* v, const void* d_o
   bp.seqlens = p.seqlens;
   bp.cu_seqlens = p.cu_seqlens;
   bp.n_seqs = p.n_seqs;
-  bp.sched_counter = nullptr;
   bp.status = status;
 
   const size_t n_elems = static_cast<size_t>(BH) * p.N * p.D;
@@ -1149,15 +1148,7 @@ int launch_bwd_bf16(const void* q, const void* k, const void* v, const void* d_o
     const size_t heads = kBwdL2Share / head_bytes;
     if (heads < static_cast<size_t>(bp.BH)) bp.head_group = heads < 1 ? 1 : static_cast<int>(heads);
   }
-  if (p.cu_seqlens != nullptr || bp.head_group < bp.BH) {
-    static std::atomic<unsigned> next_slot{0};
-    int* counters = nullptr;
-    *cuda_err = cudaGetSymbolAddress(reinterpret_cast<void**>(&counters), g_bwd_sched_counters);
-    if (*cuda_err != cudaSuccess) return SIGATTN_ERR_CUDA;
-    bp.sched_counter = counters + next_slot.fetch_add(1) % kBwdSchedSlots;
-    *cuda_err = cudaMemsetAsync(bp.sched_counter, 0, sizeof(int), stream);
-    if (*cuda_err != cudaSuccess) return SIGATTN_ERR_CUDA;
-  }
+  bp.dynamic = p.cu_seqlens != nullptr || bp.head_group < bp.BH;
   if (p.row_scale != nullptr) {
     const size_t n_vec8 = n_elems / 8;
     const size_t want = n_vec8 / 256 + 1, cap = static_cast<size_t>(num_sms) * 8;

@@ -90,10 +90,10 @@ struct FwdBarriers {
   uint64_t s_full[2], p_full[2];
   uint64_t o_full[2], o_empty[2];
   uint64_t kv_full[8], kv_empty[8];
-  // dynamic schedule (batches without padding): the TMA thread draws the next work item from a
-  // global counter and hands it to the other roles through this two-slot ring
-  uint64_t sched_full[2], sched_empty[2];
+  // dynamic schedule: the TMA thread draws the next work item and hands it to the other roles through this two-slot ring
+  uint64_t sched_full[2], sched_empty[2], sched_answer;
   int sched_item[2];
+  __align__(16) uint32_t sched_response[4];
 };
 
 struct FwdParams {
@@ -113,7 +113,7 @@ struct FwdParams {
   // Q, K and V and attends only within them; bias_vec then holds one bias per (sequence, head).
   const int* cu_seqlens;    // n_seqs + 1 row offsets, or nullptr
   int n_seqs;
-  int* sched_counter;       // dynamic schedule: next work item to hand out (zero at launch), or nullptr
+  int dynamic;     // 1: work items are drawn, one thread block of the grid per item (see sched_draw)
   int n_pairs;     // work items per head: ceil(N / (128 kTiles))
   int n_kv_total;  // ceil(N / 128)
   // Keys split over several work items (packed mode only; decoding has too few (batch, head)
@@ -151,25 +151,29 @@ __device__ __forceinline__ int snake_rank(int round, int n_items) {
 
 __device__ __forceinline__ int num_rounds(int n_items) { return (n_items + gridDim.x - 1) / gridDim.x; }
 
-// Dynamic schedule (used when the launcher gives a counter).  The static snake order balances the CTAs only if the
-// items' costs fall with their rank.  In a padded batch the cost of an item also depends on the length of its sequence,
-// and in a batch without padding the cost of a causal item follows its position inside its own
-// sequence, a sawtooth over the rows.  The general instantiations therefore draw their items from
-// a global counter instead, in row order from the last row down (every sequence then hands out
-// its expensive items first, and the cheap starts come last).  One thread per CTA draws; the other
-// roles read the item from a two-slot ring in shared memory.  Returns false when a bounded wait
+// Dynamic schedule.  The static snake order balances the CTAs only if the items' costs fall with their rank.  In a
+// padded batch the cost of an item also depends on the length of its sequence, in a batch without padding the cost of a
+// causal item follows its position inside its own sequence, a sawtooth over the rows, and heads handed out in groups
+// make a sawtooth too.  Such launches have one thread block per item, in row order from the last row down (every
+// sequence then hands out its expensive items first, and the cheap starts come last).  Those that start stay: each
+// takes over the next one that has not started yet (cluster launch control), until there is none.  The order is kept
+// by the hardware, so launches share nothing, however many are in flight or captured.  One thread per CTA draws; the
+// other roles read the item from a two-slot ring in shared memory.  Returns false when a bounded wait
 // expired; *item < 0 means no items are left.
 constexpr int kSchedConsumers = 1 + kActThreads;   // the MMA thread and the activation threads
 __device__ __forceinline__ bool sched_draw(const FwdParams& p, FwdBarriers* bars, int round, int* item,
                                            volatile int* cta_err) {
   const uint32_t slot = round & 1, phase = (round >> 1) & 1;
   if (!mbar_wait(smem_u32(&bars->sched_empty[slot]), phase ^ 1, cta_err, 40)) return false;
-  int it = atomicAdd(p.sched_counter, 1);
-  // every thread block draws until its first value >= n_items, so one launch draws n_items + gridDim.x
-  // values in all; a larger value means another launch in flight shares the counter (more launches
-  // overlapping than the library has counters): report it instead of silently skipping or repeating items
-  if (it >= p.n_items + static_cast<int>(gridDim.x)) *cta_err = 46;
-  if (it >= p.n_items) it = -1;
+  int it = blockIdx.x;
+  if (round > 0) {
+    const uint32_t response = smem_u32(bars->sched_response), bar = smem_u32(&bars->sched_answer);
+    mbar_arrive_expect_tx(bar, 16);
+    clc_try_cancel(response, bar);
+    if (!mbar_wait(bar, (round - 1) & 1, cta_err, 46)) return false;
+    it = clc_block(response);
+    fence_proxy_async_smem();   // the answer has been read before the next one is written there
+  }
   *reinterpret_cast<volatile int*>(&bars->sched_item[slot]) = it;
   mbar_arrive(smem_u32(&bars->sched_full[slot]));
   *item = it;
@@ -282,7 +286,7 @@ __device__ void fwd_load_role(const FwdParams& p, const CUtensorMap* tmQ, const 
   using L = FwdSmem<D>;
   uint32_t kv_cnt = 0;
   uint32_t q_iter[2] = {0, 0};
-  const bool dynamic = GENERAL || p.sched_counter != nullptr;
+  const bool dynamic = GENERAL || p.dynamic;
   for (int round = 0, rounds = num_rounds(p.n_items); dynamic || round < rounds; ++round) {
     int item;
     if (dynamic) {
@@ -378,7 +382,7 @@ __device__ void fwd_mma_role(const FwdParams& p, uint32_t smem_base, uint32_t tm
   auto kv_addr = [&](uint32_t cnt) { return smem_base + L::kKvOff + (cnt % L::kStages) * L::kTileBytes; };
   auto kv_release = [&](uint32_t cnt) { umma_commit(smem_u32(&bars->kv_empty[cnt % L::kStages])); };
 
-  const bool dynamic = GENERAL || p.sched_counter != nullptr;
+  const bool dynamic = GENERAL || p.dynamic;
   for (int round = 0, rounds = num_rounds(p.n_items); dynamic || round < rounds; ++round) {
     int item;
     if (dynamic) {
@@ -489,7 +493,7 @@ __device__ void fwd_act_role(const FwdParams& p, const CUtensorMap* tmO, uint8_t
   const uint32_t lane_off = static_cast<uint32_t>(((threadIdx.x >> 5) & 3) * 32) << 16;
   uint32_t s_cnt0 = 0, s_cnt1 = 0, it[2] = {0, 0};
 
-  const bool dynamic = GENERAL || p.sched_counter != nullptr;
+  const bool dynamic = GENERAL || p.dynamic;
   for (int round = 0, rounds = num_rounds(p.n_items); dynamic || round < rounds; ++round) {
     int item;
     if (dynamic) {
@@ -703,6 +707,7 @@ sigattn_fwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       mbar_init(smem_u32(&bars.sched_full[s]), 1);
       mbar_init(smem_u32(&bars.sched_empty[s]), kSchedConsumers);
     }
+    mbar_init(smem_u32(&bars.sched_answer), 1);
     fence_mbar_init();
   }
   if (warp == kLoadWarp && elect_one()) {
@@ -787,15 +792,8 @@ int choose_key_splits(int base_items, int n_kv, int num_sms) {
   return best;
 }
 
-// Work-item counters of the dynamic schedule: one per launch in flight, handed out round robin
-// (1024 launches may overlap on different streams before two of them share a counter; a kernel that
-// sees its counter run past what one launch can draw sets the device status word).
-constexpr int kSchedSlots = 1024;
-
 // K and V of all heads beyond which heads are handed out in groups, and of one group.
 constexpr size_t kFwdL2Most = 80u << 20, kFwdL2Share = 32u << 20;
-
-__device__ int g_fwd_sched_counters[kSchedSlots];
 #endif
 
 template <int D, bool CAUSAL, bool ALIBI, int MODE>
@@ -815,7 +813,7 @@ int launch_fwd_variant(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUt
     configured.fetch_or(bit, std::memory_order_relaxed);
   }
   const int slots = num_sms * kCtasPerSm;
-  const int grid = fp.n_items < slots ? fp.n_items : slots;
+  const int grid = (fp.dynamic || fp.n_items < slots) ? fp.n_items : slots;
   *cuda_err = launch_after(kernel, dim3(grid), kFwdThreads, FwdSmem<D>::kDynBytes, stream, 0, tmQ, tmK, tmV, tmO, fp);
   return *cuda_err == cudaSuccess ? SIGATTN_OK : SIGATTN_ERR_CUDA;
 }
@@ -990,7 +988,6 @@ int launch_fwd_bf16(const void* q, const void* k, const void* v, void* o, const 
   fp.n_seqs = p.n_seqs;
   fp.status = status;
 
-  fp.sched_counter = nullptr;
   const bool general = !packed && (p.cu_seqlens != nullptr || p.seqlens != nullptr || p.row_scale != nullptr || accumulate ||
                                    o_splits > 1);
   if (!packed && !general && fwd_single_tile_shape(p, num_sms))
@@ -1011,15 +1008,7 @@ int launch_fwd_bf16(const void* q, const void* k, const void* v, void* o, const 
     const size_t heads = kv_bytes < kFwdL2Share ? kFwdL2Share / kv_bytes * group : group;
     if (heads < BH) fp.head_group = static_cast<int>(heads);
   }
-  if (general || fp.head_group < fp.BH) {   // (the general instantiations always draw their work items from a counter)
-    static std::atomic<unsigned> next_slot{0};
-    int* counters = nullptr;
-    *cuda_err = cudaGetSymbolAddress(reinterpret_cast<void**>(&counters), g_fwd_sched_counters);
-    if (*cuda_err != cudaSuccess) return SIGATTN_ERR_CUDA;
-    fp.sched_counter = counters + next_slot.fetch_add(1) % kSchedSlots;
-    *cuda_err = cudaMemsetAsync(fp.sched_counter, 0, sizeof(int), stream);
-    if (*cuda_err != cudaSuccess) return SIGATTN_ERR_CUDA;
-  }
+  fp.dynamic = general || fp.head_group < fp.BH;   // (the general instantiations always draw their work items)
   const size_t n_elems = static_cast<size_t>(BH) * p.N * p.D;
   if (o_splits > 1) {
     *cuda_err = cudaMemsetAsync(o, 0, n_elems * 2, stream);

@@ -335,6 +335,32 @@ __device__ __forceinline__ float4 ld_cluster_v4(uint32_t addr) {
   return v;
 }
 
+// ------------------------------------------------------------------ cluster launch control
+
+// Ask for a thread block of this grid that has not started: if there is one it never will, and the caller may do its
+// work instead.  The 16-byte answer arrives at `response` (16-byte aligned) and completes 16 bytes on `bar`.  After an
+// answer without a thread block no further request may be made.
+__device__ __forceinline__ void clc_try_cancel(uint32_t response, uint32_t bar) {
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(response),
+               "r"(bar)
+               : "memory");
+}
+
+// blockIdx.x of the thread block in the answer, -1 if there was none left.
+__device__ __forceinline__ int clc_block(uint32_t response) {
+  int x;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b128 r;\n\t"
+      "ld.shared.b128 r, [%1];\n\t"
+      "mov.b32 %0, -1;\n\t"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\t"
+      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, r;\n\t}"
+      : "=r"(x)
+      : "r"(response)
+      : "memory");
+  return x;
+}
+
 // ------------------------------------------------------------------ arithmetic helpers
 
 __device__ __forceinline__ float ex2_approx(float x) {
