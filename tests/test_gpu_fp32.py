@@ -63,3 +63,40 @@ def test_fp32_saturated_weights():
     rev = np.flip(np.cumsum(np.flip(d_o.astype(np.float64), axis=2), axis=2), axis=2)
     assert_fp32_close(to_host(gv), rev, "dV")
     assert np.max(np.abs(to_host(gq))) < 1e-9 and np.max(np.abs(to_host(gk))) < 1e-9
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+@pytest.mark.parametrize("kind", ["causal", "padded", "packed", "packed causal"])
+def test_rows_outside_a_row_s_range_do_not_reach_it(kind, value, D):
+    """Rows that share a thread block differ in what they see.  Where row `bad` of every operand is not finite, results
+    that do not depend on it are those of clean operands to the last bit."""
+    import torch
+    import paper_2409_04431_b200 as sa
+    B, H, N, bad = 1, 2, 150, 70
+    q, k, v, d_o = (torch.from_numpy(t).float().cuda() for t in inputs.random_case(B, H, N, D, 71))
+    scale, bias, causal = 1.0 / math.sqrt(D), -math.log(N), "causal" in kind
+    if kind == "padded":
+        lens = torch.tensor([bad], dtype=torch.int32, device="cuda")
+        def run(*t):
+            return [sa.sigattn_fwd_varlen(*t[:3], scale, bias, lens, causal), *sa.sigattn_bwd_varlen(*t, scale, bias, lens, causal)[:3]]
+        before, after = slice(0, bad), slice(0, bad)
+    elif kind == "causal":
+        def run(*t):
+            return [sa.sigattn_fwd(*t[:3], scale, bias, True), *sa.sigattn_bwd(*t, scale, bias, True)]
+        before, after = slice(0, bad), slice(bad + 1, N)
+    else:
+        cu = torch.tensor([0, 9, bad - 1, bad + 2, N], dtype=torch.int32, device="cuda")
+        def run(*t):
+            return [sa.sigattn_fwd_ragged(*t[:3], cu, scale, bias, causal), *sa.sigattn_bwd_ragged(*t, cu, scale, bias, causal)[:3]]
+        before, after = slice(0, bad - 1), slice(bad + 2, N)
+    clean = run(q, k, v, d_o)
+    for t in (q, k, v, d_o):
+        t[:, :, bad] = value
+    got = run(q, k, v, d_o)
+    sa.sigattn_check()
+    for i, (name, rows) in enumerate((("O", before), ("dQ", before), ("dK", after), ("dV", after))):
+        assert torch.equal(got[i][:, :, rows], clean[i][:, :, rows]), name
+    if "packed" in kind:   # the other documents, on both sides
+        for i in range(4):
+            assert torch.equal(got[i][:, :, :bad - 1], clean[i][:, :, :bad - 1]) and torch.equal(got[i][:, :, bad + 2:], clean[i][:, :, bad + 2:])
