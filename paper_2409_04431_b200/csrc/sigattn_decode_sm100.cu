@@ -57,7 +57,7 @@ struct DecodeBarriers {
 struct DecodeParams {
   int rows, rows16;       // packed rows per key/value head, and rounded up to 16
   int n_q, group;         // rows per query head, query heads per key/value head
-  int n_tiles;            // key tiles of a head
+  int n_tiles, n_keys;    // key tiles and keys of a head
   int pos0;               // position of query 0 relative to key 0
   int causal;
   int stages;             // key/value ring
@@ -71,9 +71,9 @@ struct DecodeParams {
   int* status;
 };
 
-// One weight: P = 1 / (1 + 2^-a).
+// One weight: P = 1 / (1 + 2^-a).  NaN stays NaN: a cache row that holds one is seen in the result.
 __device__ __forceinline__ float decode_weight(float a) {
-  return rcp_approx(1.0f + ex2_approx(fminf(-a, 120.0f)));
+  return rcp_approx(1.0f + ex2_approx(fmin_nan(-a, 120.0f)));
 }
 
 template <int D, bool ALIBI>
@@ -86,7 +86,7 @@ sigattn_decode_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid
   extern __shared__ uint8_t smem_raw[];
   __shared__ DecodeBarriers bars;
   __shared__ __align__(16) float row_bias[kDecMaxRows], row_slope[kDecMaxRows];   // both times log2 e
-  __shared__ __align__(16) int row_pos[kDecMaxRows];
+  __shared__ __align__(16) int row_pos[kDecMaxRows], row_last[kDecMaxRows];   // position, and of the last key it sees
   __shared__ uint32_t tmem_base_slot;
   __shared__ int cta_err_slot;
   volatile int* cta_err = &cta_err_slot;
@@ -141,6 +141,7 @@ sigattn_decode_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid
     row_bias[threadIdx.x] = p.bias_vec ? __ldg(p.bias_vec + q_head) * kDecLog2e : p.bias_log2e;
     if (ALIBI) row_slope[threadIdx.x] = __ldg(p.slopes + q_head % p.H) * kDecLog2e;
     row_pos[threadIdx.x] = r - g * p.n_q + p.pos0;
+    row_last[threadIdx.x] = p.causal ? r - g * p.n_q + p.pos0 : p.n_keys - 1;
   }
   tc_fence_before_sync();
   __syncthreads();
@@ -232,8 +233,10 @@ sigattn_decode_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid
       if (!ok) break;
       tc_fence_after_sync();
       const int key_pos = (tile0 + j) * kDecTile + key;
-      // the mask cuts only tiles that reach beyond the first query's position
-      const bool cut = p.causal && (tile0 + j + 1) * kDecTile - 1 > p.pos0;
+      // the mask cuts only tiles that reach beyond the first query's position, or beyond the last key (such rows read as
+      // zeros, and a query that holds Inf makes NaN of them)
+      const int seen = p.causal ? p.pos0 + 1 : p.n_keys;   // (causal: pos0 + 1 <= n_keys)
+      const bool cut = (tile0 + j + 1) * kDecTile > seen;
       uint8_t* p_col = smem + buf * p_bytes + (key >> 6) * p_panel + p_lo;
       // sixteen rows at a time, the rows past the end with them: straight-line code, so that the exponentials
       // and reciprocals of different rows overlap (with a test per row a tile of 32 rows took 5300 cycles)
@@ -254,7 +257,7 @@ sigattn_decode_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid
         if (cut) {
 #pragma unroll
           for (int e = 0; e < 16; ++e)
-            if (key_pos > row_pos[r0 + e]) w[e] = 0.0f;
+            if (key_pos > row_last[r0 + e]) w[e] = 0.0f;
         }
 #pragma unroll
         for (int e = 0; e < 16; ++e)
@@ -383,7 +386,8 @@ int launch_decode_bf16(const void* q, const void* k, const void* v, void* o, con
   dp.rows16 = (dp.rows + 15) & ~15;
   dp.n_q = p.N;
   dp.group = group;
-  dp.n_tiles = (p.key_rows() + kDecTile - 1) / kDecTile;
+  dp.n_keys = p.key_rows();
+  dp.n_tiles = (dp.n_keys + kDecTile - 1) / kDecTile;
   dp.pos0 = p.query_pos0();
   dp.causal = p.causal;
   dp.scale_log2e = p.scale * kDecLog2e;

@@ -375,6 +375,13 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return y;
 }
 
+// min that keeps NaN (fminf gives the other operand)
+__device__ __forceinline__ float fmin_nan(float a, float b) {
+  float y;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+  return y;
+}
+
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
   float y;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));

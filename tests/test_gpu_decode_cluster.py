@@ -60,3 +60,30 @@ def test_decode_one_cluster_per_head(B, H, H_kv, N_q, N_k, D, causal, with_slope
 def test_decode_several_clusters_per_head(B, H, H_kv, N_q, N_k, D, causal, with_slopes):
     launches, _ = _run(B, H, H_kv, N_q, N_k, D, causal, with_slopes)
     assert launches == 2      # sums in scratch, then converted
+
+
+@pytest.mark.parametrize("causal", [False, True])
+@pytest.mark.parametrize("N_k", [300, 2000, 2048])
+def test_decode_values_that_are_not_finite(N_k, causal):
+    """NaN in one cached key reaches every head that reads it; Inf in a query, whose logits are +-Inf, weighs the keys
+    with 1 and 0 (also where the last tile holds rows that do not exist)."""
+    import torch
+    import paper_2409_04431_b200 as sa
+    H, H_kv, D = 8, 2, 128
+    g = torch.Generator(device="cuda").manual_seed(N_k)
+    q = torch.randn((1, H, 1, D), generator=g, device="cuda").to(torch.bfloat16)
+    k, v = (torch.randn((1, H_kv, N_k, D), generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
+    a = (1.0 / math.sqrt(D), -math.log(N_k), causal)
+    clean = sa.sigattn_fwd_decode(q, k, v, *a)
+    bad = k.clone()
+    bad[0, 0, 17, 5] = float("nan")
+    o = sa.sigattn_fwd_decode(q, bad, v, *a)
+    assert bool(torch.isnan(o[0, :4]).all()) and torch.equal(o[0, 4:], clean[0, 4:])
+    inf = q.clone()
+    inf[0, 3, 0, 7] = float("inf")
+    o = sa.sigattn_fwd_decode(inf, k, v, *a)
+    sa.sigattn_check()
+    want = (k[0, 0, :, 7] > 0).double().cpu() @ v[0, 0].double().cpu()
+    assert rel_fro(to_host(o)[0, 3, 0], want.numpy()) < BF16_REL_FRO
+    keep = [h for h in range(H) if h != 3]
+    assert torch.equal(o[0, keep], clean[0, keep])
