@@ -1174,10 +1174,17 @@ int launch_bwd_bf16(const void* q, const void* k, const void* v, const void* d_o
   //   causal: B16 N512 97 / 90, B8 N1024 115 / 106, B8 N2048 292 / 292, B2 N4096 246 / 251;
   //   padded, lengths N/4 to N: N400 64 / 58, N1500 249 / 227, N2500 1010 / 967;
   //   packed documents: 60 in 16384 rows 337 / 291, 16 in 16384 507 / 462, 5 in 8000 253 / 280.
+  // ALiBi without a mask forms |i - j| for every element, which the 96 registers of the wide shape hold worse (120 to 232
+  // bytes spilled in its general instantiations); causal calls with grouped heads have more steps an item.  B16 H12:
+  //   ALiBi, no mask: N300 48 / 47, N577 102 / 102, N1025 256 / 268, N1250 326 / 334; H_kv4 N300 68 / 66, N577 132 / 144,
+  //   N1250 384 / 420; padded N577 113 / 110, N1250 285 / 268, N2400 1142 / 1134; 60 documents 335 / 332, 16 645 / 682;
+  //   causal H_kv4: N300 57 / 55, N577 84 / 74, N1025 158 / 160; B4 H16 H_kv4 N1900 134 / 141.
   const int typical_rows = p.cu_seqlens != nullptr ? p.N / p.n_seqs
                            : p.seqlens != nullptr  ? p.N / 2
                            : p.causal              ? p.N / 3 * 2 : p.N;
-  const bool wide = p.D == 64 && typical_rows <= 1280;
+  const bool grouped_causal = p.causal && bp.group > 1 && p.seqlens == nullptr && p.cu_seqlens == nullptr;
+  const int wide_rows = (p.slopes != nullptr && !p.causal && p.seqlens == nullptr) ? 512 : grouped_causal ? 600 : 1280;
+  const bool wide = p.D == 64 && typical_rows <= wide_rows;
 #define SIGATTN_BWD_SHAPE(DD, CC, AA, BB, KK)                                                              \
   ((DD == 64 && wide) ? launch_bwd_variant<DD, CC, AA, BB, KK, DD == 64>(maps, bp, num_sms, stream, cuda_err) \
                       : launch_bwd_variant<DD, CC, AA, BB, KK, false>(maps, bp, num_sms, stream, cuda_err))

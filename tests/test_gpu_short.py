@@ -76,3 +76,22 @@ def test_wide_backward_at_64(kind, H, H_kv, N):
     sa.sigattn_check()
     for name, g, r in zip(("dQ", "dK", "dV"), out, oracle.sigattn_bwd(q, k, v, d_o, scale, bias, causal, None, **more)):
         assert_bf16_close(to_host(g), r, name)
+
+
+@pytest.mark.parametrize("H,H_kv,N,causal", [(3, 3, 500, False), (3, 3, 530, False), (4, 2, 500, False), (4, 2, 530, False),
+                                             (4, 2, 890, True), (4, 2, 910, True)])
+def test_backward_shapes_meet_at_64(H, H_kv, N, causal):
+    """ALiBi on both sides of the lines between the wide and the narrow backward: 512 rows without a mask, 900 rows of
+    a causal call with grouped heads (two thirds of them count as typical)."""
+    import torch
+    import paper_2409_04431_b200 as sa
+    B, D = 1, 64
+    q, _, _, d_o = inputs.random_case(B, H, N, D, 600 + N)
+    _, k, v, _ = inputs.random_case(B, H_kv, N, D, 601 + N)
+    slopes = (0.5 ** np.arange(1, H + 1)).astype(np.float32)
+    tq, tk, tv, tdo = (to_device(t, "bf16") for t in (q, k, v, d_o))
+    scale, bias = 1.0 / math.sqrt(D), -math.log(N)
+    out = sa.sigattn_bwd_gqa(tq, tk, tv, tdo, scale, bias, causal, torch.from_numpy(slopes).cuda())
+    sa.sigattn_check()
+    for name, g, r in zip(("dQ", "dK", "dV"), out, oracle.sigattn_bwd(q, k, v, d_o, scale, bias, causal, slopes)):
+        assert_bf16_close(to_host(g), r, name)
