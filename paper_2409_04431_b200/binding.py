@@ -253,13 +253,9 @@ def _host_slopes_ptr(alibi_slopes, H):
 
 
 def _ws_ptr(workspace, q):
-    """Device pointer of a caller-supplied scratch tensor: uint8, on q's device, contiguous."""
-    if workspace is None:
-        return None
-    if (not isinstance(workspace, torch.Tensor) or not workspace.is_cuda or workspace.device != q.device
-            or workspace.dtype != torch.uint8 or not workspace.is_contiguous()):
-        raise ValueError("workspace must be a contiguous uint8 CUDA tensor on q's device")
-    return workspace.data_ptr()
+    """Device pointer of a caller-supplied scratch tensor after the check that every call makes of it (uint8, on q's
+    device, contiguous)."""
+    return _host.workspace_ptr(workspace, q)
 
 
 def _check_same(ts, names):

@@ -407,6 +407,16 @@ PyObject* host_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
   });
 }
 
+// workspace_ptr(workspace, q) -> the address of a scratch tensor that passes the calls' check, None for None
+PyObject* host_workspace_ptr(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return guarded([&]() -> PyObject* {
+    const at::Tensor* q = n == 2 ? tensor_or_null(a[1]) : nullptr;
+    if (!q) fail(PyExc_TypeError, "workspace_ptr takes (workspace, q)");
+    if (a[0] == Py_None) return Py_NewRef(Py_None);
+    return PyLong_FromVoidPtr(given_scratch(a[0], *q).ptr);
+  });
+}
+
 PyObject* host_set_error(PyObject*, PyObject* type) {
   Py_XSETREF(g_error, Py_NewRef(type));
   Py_RETURN_NONE;
@@ -415,6 +425,7 @@ PyObject* host_set_error(PyObject*, PyObject* type) {
 PyMethodDef g_methods[] = {
     {"fwd", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(host_fwd)), METH_FASTCALL, nullptr},
     {"bwd", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(host_bwd)), METH_FASTCALL, nullptr},
+    {"workspace_ptr", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(host_workspace_ptr)), METH_FASTCALL, nullptr},
     {"set_error", host_set_error, METH_O, nullptr},
     {nullptr, nullptr, 0, nullptr}};
 

@@ -192,3 +192,24 @@ def test_memory_of_calls_on_another_stream(what, how):
     torch.cuda.synchronize()
     assert close(kept) and len(later) == 6
     sa.sigattn_check()
+
+
+def test_refuses_scratch_the_kernels_could_not_use():
+    import torch
+    import paper_2409_04431_b200 as sa
+    q, k, v, d_o = _qkv(N=300)
+    a = (0.125, -5.0)
+    size = sa.sigattn_bwd_workspace_bytes(1, 2, 300, 64, 0)
+    ok = torch.empty(size, dtype=torch.uint8, device="cuda")
+    bad = (torch.empty(size, dtype=torch.uint8), torch.empty(size // 4, device="cuda"), torch.empty(2 * size, dtype=torch.uint8, device="cuda")[::2], size)
+    for w in bad:
+        with pytest.raises(ValueError):
+            sa.sigattn_bwd(q, k, v, d_o, *a, workspace=w)
+        with pytest.raises(ValueError):
+            sa.sigattn_fwd_decode(q[:, :, :1].contiguous(), k, v, *a, workspace=w)
+    for w, code in ((ok[:size - 1], -5), (torch.empty(size + 16, dtype=torch.uint8, device="cuda")[16:], -3)):
+        with pytest.raises(sa.SigattnError) as e:
+            sa.sigattn_bwd(q, k, v, d_o, *a, workspace=w)
+        assert e.value.code == code
+    sa.sigattn_bwd(q, k, v, d_o, *a, workspace=ok)
+    sa.sigattn_check()
