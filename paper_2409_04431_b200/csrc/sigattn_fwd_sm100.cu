@@ -771,6 +771,7 @@ sigattn_fwd_convert_o_kernel(const float4* __restrict__ ws, uint2* __restrict__ 
 // and on the benchmark configurations the two-tile shape is 5-16 % faster.  One tile per item pays when the
 // two-tile items leave more than half of the SMs empty and the sequence is too short for the keys of an item
 // to be divided (that division serves the long sequences with few heads); with N <= 128 both shapes are the same.
+// (Measured before plain calls with D = 64 and N <= 256 got a kernel of their own, which is asked first.)
 bool fwd_single_tile_shape(const Problem& p, int num_sms) {
   const bool plain_self = p.key_rows() == p.N && p.query_pos0() == 0 && p.kv_heads() == p.H;
   const long long pair_items = static_cast<long long>(p.B) * p.H * ((p.N + 2 * kBM - 1) / (2 * kBM));
