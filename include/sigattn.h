@@ -417,13 +417,16 @@ SIGATTN_API int sigattn_seqlen_norm(float* row_scale, int N_q, int N_k, float al
 
 /* Forward for generation with a cache of keys and values (where the paper measures its
  * inference gains, Appendix F.3): the same operation, arguments and result as sigattn_fwd_nk,
- * plus a scratch buffer that lets the library split the keys of one head over several thread
- * blocks when B * H_kv alone cannot fill the GPU.  Sigmoid attention has no row normalisation
- * (Section 4), so the partial outputs of the splits are plain fp32 sums - no running maximum, no
- * log-sum-exp to merge; they are added with fp32 atomics (the last bits of O may differ from run
- * to run) and converted to bf16 by a second small kernel.  The split is used when the queries of
- * a key/value head fit one pair of tiles (N_q * H / H_kv <= 256) and it shortens the run; otherwise
- * the call is sigattn_fwd_nk and leaves the workspace untouched.
+ * plus a scratch buffer.  Sigmoid attention has no row normalisation (Section 4), so the partial
+ * outputs of different keys are plain fp32 sums - no running maximum, no log-sum-exp to merge.
+ * With at most 64 query rows per key/value head (N_q * H / H_kv) the keys of a head are divided
+ * over the thread blocks of a cluster, which add their parts in a fixed order through distributed
+ * shared memory: one kernel, the scratch untouched, O the same from run to run.  Only few heads
+ * with long caches (fewer than 96 thread blocks' worth, and more than 8 to 16 tiles of 128 keys
+ * for each of them) take several clusters per head, whose sums are added in the scratch with fp32
+ * atomics (the last bits of O may differ from run to run) and converted by a second kernel.
+ * With 65 to 256 rows the general forward divides the keys over thread blocks in that second way
+ * when it shortens the run; otherwise the call is sigattn_fwd_nk and leaves the scratch untouched.
  * workspace: DEVICE scratch of at least sigattn_fwd_decode_workspace_bytes(...) bytes, 256-byte
  * aligned, owned by the caller; two calls that share it must not overlap on the device.  Errors
  * as sigattn_fwd_nk, plus SIGATTN_ERR_WORKSPACE. */
