@@ -56,7 +56,7 @@ struct BwdRoles {
   static constexpr int kLoadWarp = 4 * kGroups + (kDrainGroup ? 4 : 0);
   static constexpr int kMmaWarp = kLoadWarp + 1;
   static constexpr int kThreads = 32 * (kMmaWarp + (kDrainGroup ? 1 : 2));
-  static constexpr int kSchedConsumers = 1 + kActThreads + (kDrainGroup ? 128 : 1);   // see the dynamic schedule
+  static constexpr int kItemReaders = 1 + kActThreads + (kDrainGroup ? 128 : 1);   // threads that take every work item
   // first packed column of k-step ks (16 queries = 8 columns): a group packs its bf16 values over the first half
   // of its own columns
   __device__ static __forceinline__ uint32_t packed_col(int ks) {
@@ -71,7 +71,8 @@ struct BwdSmem {
   static constexpr int kPanelBytes = kT * 128;
   static constexpr int kTileBytes = kPanels * kPanelBytes;  // a K, V, Q or dO tile
   // K, V buffers: at D = 64 two, so that the next item's first products do not wait for this item's results to be
-  // stored (dV is staged in the V buffer, dK in the K buffer)
+  // stored (dV is staged in the V buffer, dK in the K buffer).  At D = 128 one; dK is staged where dS was, so that the
+  // next K can be loaded as soon as the last dQ has read this one.
   static constexpr int kKvStages = (D == 64) ? 2 : 1;
   static constexpr int kKOff = 0;
   static constexpr int kVOff = kTileBytes;
@@ -90,8 +91,17 @@ struct BwdSmem {
   static constexpr int kDynBytes = kTotal + 1024;
 };
 
+struct BwdItem {
+  int bh;       // (batch, key/value head) index: K_j, V_j, dK_j, dV_j
+  int bh_q0;    // first of the `group` query heads that read this key/value head
+  int j, i_begin;
+  int n;        // query tiles per query head
+  int steps;    // group * n, visited head by head; 0: no item is left
+  int n_valid;  // rows of this sequence that count (N unless the batch is padded)
+};
+
 struct BwdBarriers {
-  uint64_t kv_full[2], kv_empty[2];
+  uint64_t k_full[2], v_full[2], k_empty[2], v_empty[2];
   uint64_t q_full[3], q_empty[3];
   uint64_t do_full[3], do_empty[3];
   // s_full, p_ready, dq_full, dq_empty: one per region of tensor memory that holds S^T / P^T (see BwdTmem);
@@ -99,11 +109,12 @@ struct BwdBarriers {
   uint64_t s_full[2], dp_full;
   uint64_t p_ready[2], ds_ready;
   uint64_t dq_full[2], dq_empty[2];
-  uint64_t dkv_full, dkv_empty;
+  uint64_t dv_full, dkv_full, dkv_empty;
+  uint64_t ds_free;   // D = 128: dK has been stored from where dS goes
   uint64_t stage_full, stage_empty;   // wide: the dQ staging boxes between the activation groups and the storing thread
-  // dynamic schedule: the TMA thread draws the next work item and hands it to the other roles through this two-slot ring
+  // the TMA thread finds the next work item and hands it to the other roles through this two-slot ring
   uint64_t sched_full[2], sched_empty[2], sched_answer;
-  int sched_item[2];
+  BwdItem sched_item[2];
   __align__(16) uint32_t sched_response[4];
 };
 
@@ -118,7 +129,7 @@ struct BwdParams {
   // bias_vec and dbias then hold one entry per (sequence, head)
   const int* cu_seqlens;
   int n_seqs;
-  int dynamic;     // 1: work items are drawn, one thread block of the grid per item (see bwd_sched_draw)
+  int dynamic;     // 1: work items are drawn, one thread block of the grid per item (see BwdSchedule)
   // Few (batch, key/value head) pairs (multi-query attention at a small batch): the query heads of a
   // group are split over n_sub work items of heads_per_sub heads each, which add their dK_j, dV_j
   // (bf16 TMA reduce-adds into the cleared outputs) instead of storing them.  n_sub = 1: off.
@@ -136,15 +147,6 @@ struct BwdParams {
   int* status;
 };
 
-struct BwdItem {
-  int bh;       // (batch, key/value head) index: K_j, V_j, dK_j, dV_j
-  int bh_q0;    // first of the `group` query heads that read this key/value head
-  int j, i_begin;
-  int n;        // query tiles per query head
-  int steps;    // group * n, visited head by head
-  int n_valid;  // rows of this sequence that count (N unless the batch is padded)
-};
-
 // Ranks are ordered by decreasing cost; rounds alternate direction over the CTAs so that
 // expensive and cheap items pair up (static stand-in for longest-first scheduling).
 __device__ __forceinline__ int bwd_snake_rank(int round, int n_items) {
@@ -156,35 +158,59 @@ __device__ __forceinline__ int bwd_snake_rank(int round, int n_items) {
 
 __device__ __forceinline__ int bwd_num_rounds(int n_items) { return (n_items + gridDim.x - 1) / gridDim.x; }
 
-// Dynamic schedule, used where the static order above does not sort by cost: in batches without padding, where the
-// cost follows the position of the key tile inside its own sequence, and when heads are handed out in groups.  The
-// grid has one thread block per item; those that start take over the others in order (cluster launch control, as in
-// the forward).  One thread per CTA draws; the MMA thread, the activation groups and the drain group read the item
-// from a two-slot ring.  false: a bounded wait expired; *item < 0: none left.
-__device__ __forceinline__ bool bwd_sched_draw(const BwdParams& p, BwdBarriers* bars, int round, int* item,
-                                               volatile int* cta_err) {
-  const uint32_t slot = round & 1, phase = (round >> 1) & 1;
-  if (!mbar_wait(smem_u32(&bars->sched_empty[slot]), phase ^ 1, cta_err, 70)) return false;
-  int it = blockIdx.x;
-  if (round > 0) {
-    const uint32_t response = smem_u32(bars->sched_response), bar = smem_u32(&bars->sched_answer);
-    mbar_arrive_expect_tx(bar, 16);
-    clc_try_cancel(response, bar);
-    if (!mbar_wait(bar, (round - 1) & 1, cta_err, 76)) return false;
-    it = clc_block(response);
+// Which item comes next.  Where the static order above does not sort by cost (batches without padding, where the cost
+// follows the position of the key tile inside its own sequence, and heads handed out in groups) the items are drawn: the
+// grid has one thread block per item; those that start take over the others in order (cluster launch control, as in the
+// forward).  One thread per block, which has issued an item's last loads some steps before it ends, finds the
+// next (an answer takes about 2200 cycles), decodes it and passes it on through the ring: the divisions and searches of
+// decoding cost the other roles, above all the thread that issues the products, 600 to 1400 cycles between two items.
+struct BwdSchedule {
+  int turn, item, requests;
+};
+__device__ __forceinline__ void bwd_first_item(const BwdParams& p, BwdSchedule* s) {
+  s->turn = 0;
+  s->requests = 0;
+  s->item = p.dynamic ? static_cast<int>(blockIdx.x) : bwd_snake_rank(0, p.n_items);
+}
+// The next one (s->item < 0: none is left).  false: a bounded wait expired.
+__device__ __forceinline__ bool bwd_following_item(const BwdParams& p, BwdBarriers* bars, BwdSchedule* s, volatile int* cta_err) {
+  if (p.dynamic) {
+    mbar_arrive_expect_tx(smem_u32(&bars->sched_answer), 16);
+    clc_try_cancel(smem_u32(bars->sched_response), smem_u32(&bars->sched_answer));
+    if (!mbar_wait(smem_u32(&bars->sched_answer), s->requests & 1, cta_err, 76)) return false;
+    ++s->requests;
+    s->item = clc_block(smem_u32(bars->sched_response));
     fence_proxy_async_smem();   // the answer has been read before the next one is written there
+    return true;
   }
-  *reinterpret_cast<volatile int*>(&bars->sched_item[slot]) = it;
-  mbar_arrive(smem_u32(&bars->sched_full[slot]));
-  *item = it;
+  s->item = -1;
+  const int rounds = bwd_num_rounds(p.n_items);
+  while (s->item < 0 && ++s->turn < rounds) s->item = bwd_snake_rank(s->turn, p.n_items);
   return true;
 }
-__device__ __forceinline__ bool bwd_sched_take(BwdBarriers* bars, int round, int* item, volatile int* cta_err) {
-  const uint32_t slot = round & 1, phase = (round >> 1) & 1;
-  if (!mbar_wait(smem_u32(&bars->sched_full[slot]), phase, cta_err, 71)) return false;
-  *item = *reinterpret_cast<volatile int*>(&bars->sched_item[slot]);
-  mbar_arrive(smem_u32(&bars->sched_empty[slot]));
+// The ring: `number` counts the items of this thread block.
+__device__ __forceinline__ bool bwd_hand_item(BwdBarriers* bars, uint32_t number, const BwdItem& w, volatile int* cta_err) {
+  const uint32_t slot = number & 1, phase = (number >> 1) & 1;
+  if (!mbar_wait(smem_u32(&bars->sched_empty[slot]), phase ^ 1, cta_err, 70)) return false;
+  bars->sched_item[slot] = w;
+  mbar_arrive(smem_u32(&bars->sched_full[slot]));
   return true;
+}
+// 1 and *w, 0 when no item is left, -1 when a bounded wait expired.  (The activation threads keep the slot until the item
+// is done and read there what the steps do not need: their registers are full.)
+__device__ __forceinline__ int bwd_see_item(BwdBarriers* bars, uint32_t number, BwdItem* w, volatile int* cta_err) {
+  const uint32_t slot = number & 1, phase = (number >> 1) & 1;
+  if (!mbar_wait(smem_u32(&bars->sched_full[slot]), phase, cta_err, 71)) return -1;
+  *w = bars->sched_item[slot];
+  return w->steps > 0 ? 1 : 0;
+}
+__device__ __forceinline__ void bwd_return_item(BwdBarriers* bars, uint32_t number) {
+  mbar_arrive(smem_u32(&bars->sched_empty[number & 1]));
+}
+__device__ __forceinline__ int bwd_take_item(BwdBarriers* bars, uint32_t number, BwdItem* w, volatile int* cta_err) {
+  const int more = bwd_see_item(bars, number, w, cta_err);
+  if (more >= 0) bwd_return_item(bars, number);
+  return more;
 }
 
 // GROUPED = false compiles the plain case (one query head per key/value head, no padded batch)
@@ -205,8 +231,6 @@ __device__ __forceinline__ BwdItem decode_bwd_item(const BwdParams& p, int item)
   BwdItem w;
   // Items are numbered group of heads by group of heads (see the launcher; one group = all heads), within a group by
   // ascending key tile = descending work when causal, then head, then part.
-  // (Divisions only where they are needed: every role decodes every item, and the thread that issues the products
-  // pays for each instruction.  Two more of them cost 15 % at N = 577, five short items a head.)
   const int parts = GROUPED ? (p.n_sub > 1 ? p.n_sub : p.i_split) : 1;
   int g0 = 0, r = item, per_tile = p.BH * parts;
   if (p.head_group < p.BH) {
@@ -315,27 +339,32 @@ __device__ void bwd_load_role(const BwdParams& p, const CUtensorMap* tmQ, const 
     ++do_cnt;
     return true;
   };
-  const bool dynamic = p.dynamic != 0;
-  for (int round = 0, rounds = bwd_num_rounds(p.n_items); dynamic || round < rounds; ++round) {
-    int item;
-    if (dynamic) {
-      if (!bwd_sched_draw(p, bars, round, &item, cta_err)) return;
-      if (item < 0) break;
-    } else {
-      item = bwd_snake_rank(round, p.n_items);
-      if (item < 0) continue;
-    }
-    const BwdItem w = decode_bwd_item<CAUSAL, GROUPED>(p, item);
+  BwdSchedule sched;
+  bwd_first_item(p, &sched);
+  for (uint32_t number = 0;; ++number) {
+    BwdItem w;
+    w.steps = 0;
+    if (sched.item >= 0) w = decode_bwd_item<CAUSAL, GROUPED>(p, sched.item);
+    if (!bwd_hand_item(bars, number, w, cta_err)) return;
+    if (sched.item < 0) break;
     auto load_kv = [&]() -> bool {
-      const uint32_t st = item_cnt % L::kKvStages, ph = (item_cnt / L::kKvStages) & 1;
-      if (!mbar_wait(smem_u32(&bars->kv_empty[st]), ph ^ 1, cta_err, 42)) return false;
-      const uint32_t bar = smem_u32(&bars->kv_full[st]), dst = smem_base + st * L::kKvBytes;
-      mbar_arrive_expect_tx(bar, L::kKvBytes);
-      load_tile(tmK, dst + L::kKOff, bar, w.j * kT, w.bh);
-      load_tile(tmV, dst + L::kVOff, bar, w.j * kT, w.bh);
+      const uint32_t st = item_cnt % L::kKvStages, ph = (item_cnt / L::kKvStages) & 1, dst = smem_base + st * L::kKvBytes;
+      if (!mbar_wait(smem_u32(&bars->k_empty[st]), ph ^ 1, cta_err, 42)) return false;
+      mbar_arrive_expect_tx(smem_u32(&bars->k_full[st]), L::kTileBytes);
+      load_tile(tmK, dst + L::kKOff, smem_u32(&bars->k_full[st]), w.j * kT, w.bh);
+      if (!mbar_wait(smem_u32(&bars->v_empty[st]), ph ^ 1, cta_err, 43)) return false;
+      mbar_arrive_expect_tx(smem_u32(&bars->v_full[st]), L::kTileBytes);
+      load_tile(tmV, dst + L::kVOff, smem_u32(&bars->v_full[st]), w.j * kT, w.bh);
       ++item_cnt;
       return true;
     };
+    if (L::kKvStages == 1) {   // they can only be loaded when the item before is done: at least from L2 then
+#pragma unroll
+      for (int pn = 0; pn < L::kPanels; ++pn) {
+        tma_prefetch_3d(tmK, pn * 64, w.j * kT, w.bh);
+        tma_prefetch_3d(tmV, pn * 64, w.j * kT, w.bh);
+      }
+    }
     // With one K, V buffer the first Q and dO tiles can be loaded earlier than K and V, with two later.
     if (L::kKvStages > 1 && !load_kv()) return;
     if (!load_q(w.i_begin, w.bh_q0)) return;
@@ -355,6 +384,9 @@ __device__ void bwd_load_role(const BwdParams& p, const CUtensorMap* tmQ, const 
         if (!load_step(q_next, true)) return;
       if (!load_step(do_next, false)) return;
     }
+    // (asked for only now: with the request at the item's start the answer costs nothing, but items go to blocks that are
+    // far from ready for them: B4 H32 H_kv8 N2048 D128 causal 468 -> 563 us, 16 documents in 16384 rows 508 -> 555)
+    if (!bwd_following_item(p, bars, &sched, cta_err)) return;
   }
 }
 
@@ -364,8 +396,8 @@ __device__ void bwd_load_role(const BwdParams& p, const CUtensorMap* tmQ, const 
 // a single thread is active, and every product costs the thread more.  Measured, whole backward, us:
 // B8 H12 N4096 D64 1540 -> 1385, B8 H16 N2048 D64 causal ALiBi 353 -> 331, B2 H16 N4096 D128 causal 389 -> 387.
 // (The role run by the whole warp with an election per batch of products: 1405, 339, 392.)
-template <int D, bool CAUSAL, bool GROUPED, bool WIDE>
-__device__ void bwd_mma_role(const BwdParams& p, uint32_t smem_base, uint32_t tmem, BwdBarriers* bars,
+template <int D, bool WIDE>
+__device__ void bwd_mma_role(uint32_t smem_base, uint32_t tmem, BwdBarriers* bars,
                              volatile int* cta_err) {
   using L = BwdSmem<D>;
   using TM = BwdTmem<D>;
@@ -424,26 +456,22 @@ __device__ void bwd_mma_role(const BwdParams& p, uint32_t smem_base, uint32_t tm
     return true;
   };
 
-  const bool dynamic = p.dynamic != 0;
-  for (int round = 0, rounds = bwd_num_rounds(p.n_items); dynamic || round < rounds; ++round) {
-    int item;
-    if (dynamic) {
-      if (!bwd_sched_take(bars, round, &item, cta_err)) return;
-      if (item < 0) break;
-    } else {
-      item = bwd_snake_rank(round, p.n_items);
-      if (item < 0) continue;
-    }
-    const BwdItem w = decode_bwd_item<CAUSAL, GROUPED>(p, item);
-    if (!mbar_wait(smem_u32(&bars->kv_full[item_cnt % L::kKvStages]), (item_cnt / L::kKvStages) & 1, cta_err, 50)) return;
+  BwdItem w;
+  if (bwd_take_item(bars, 0, &w, cta_err) < 0) return;
+  int next_steps = w.steps;
+  while (next_steps > 0) {
+    const int steps = next_steps;
     const uint64_t dK_mn = desc_advance(dK_mn0, kv_off());
 
     // prologue: S^T(0), dP^T(0) and, with two regions A, S^T(1)
+    const uint32_t kv_stage = item_cnt % L::kKvStages, kv_phase = (item_cnt / L::kKvStages) & 1;
+    if (!mbar_wait(smem_u32(&bars->k_full[kv_stage]), kv_phase, cta_err, 50)) return;
     if (!issue_s(step_cnt, q_cnt, 51)) return;
+    if (!mbar_wait(smem_u32(&bars->v_full[kv_stage]), kv_phase, cta_err, 49)) return;
     if (!issue_dp(step_cnt, 52)) return;
-    if (TM::kTwoA && w.steps > 1 && !issue_s(step_cnt + 1, q_cnt + 1, 53)) return;
+    if (TM::kTwoA && steps > 1 && !issue_s(step_cnt + 1, q_cnt + 1, 53)) return;
 
-    for (int it = 0; it < w.steps; ++it) {
+    for (int it = 0; it < steps; ++it) {
       const uint32_t st = q_stage(q_cnt), reg = TM::r_index(step_cnt);
       // dV += P^T dO_i
       if (!mbar_wait(smem_u32(&bars->p_ready[reg]), TM::r_use(step_cnt) & 1, cta_err, 54)) return;
@@ -458,7 +486,12 @@ __device__ void bwd_mma_role(const BwdParams& p, uint32_t smem_base, uint32_t tm
       umma_commit(smem_u32(&bars->do_empty[do_stage(do_cnt)]));
       ++do_cnt;
       // one region A: S^T of the next query tile goes where P^T was
-      if (!TM::kTwoA && it + 1 < w.steps && !issue_s(step_cnt + 1, q_cnt + 1, 56)) return;
+      if (!TM::kTwoA && it + 1 < steps && !issue_s(step_cnt + 1, q_cnt + 1, 56)) return;
+      if (it + 1 == steps) {
+        umma_commit(smem_u32(&bars->dv_full));
+        if (bwd_take_item(bars, item_cnt + 1, &w, cta_err) < 0) return;
+        next_steps = w.steps;
+      }
       // dK += dS^T Q_i with dS^T read from region B of tensor memory (the activation groups
       // leave a bf16 copy there, over the dP^T columns they have consumed), then dQ_i = dS K_j,
       // which overwrites region B (D = 128) or the head of the step's region A (D = 64): MMAs of
@@ -479,41 +512,63 @@ __device__ void bwd_mma_role(const BwdParams& p, uint32_t smem_base, uint32_t tm
       umma_commit(smem_u32(&bars->dq_full[reg]));
       umma_commit(smem_u32(&bars->q_empty[st]));
       // dP^T of the next query tile, then (two regions A) S^T of the one after it
-      if (it + 1 < w.steps && !issue_dp(step_cnt + 1, 58)) return;
-      if (TM::kTwoA && it + 2 < w.steps && !issue_s(step_cnt + 2, q_cnt + 2, 59)) return;
+      if (it + 1 < steps && !issue_dp(step_cnt + 1, 58)) return;
+      if (TM::kTwoA && it + 2 < steps && !issue_s(step_cnt + 2, q_cnt + 2, 59)) return;
       ++q_cnt;
       ++step_cnt;
     }
     umma_commit(smem_u32(&bars->dkv_full));
+    if (L::kKvStages == 1) umma_commit(smem_u32(&bars->k_empty[0]));
     ++item_cnt;
   }
 }
 
 // ------------------------------------------------------------------ activation groups
 
-// One row of a [128 x D] fp32 accumulator -> bf16 (times `mul`) -> swizzled staging tile: share `part` of its
-// columns (32-column runs part, part + parts, ...).
+// Group `wg`'s columns of one row of a [128 x D] fp32 accumulator -> bf16 (times `mul`) -> swizzled staging tile.
 template <int D, bool WIDE>
-__device__ __forceinline__ void bwd_store_acc_rows(uint32_t t_acc, uint8_t* stage, int tid, float mul, int part) {
+__device__ __forceinline__ void bwd_store_acc_rows(uint32_t t_acc, uint8_t* stage, int tid, float mul, int wg) {
   using L = BwdSmem<D>;
-  constexpr int kParts = BwdRoles<D, WIDE>::kGroups / 2;
+  constexpr int kShare = D / BwdRoles<D, WIDE>::kGroups, kRun = kShare < 32 ? kShare : 32;   // columns, at a time
 #pragma unroll 1
-  for (int c = part; c < D / 32; c += kParts) {
-    uint32_t o[32];
-    tmem_ld32(t_acc + c * 32, o);
+  for (int c = wg * kShare; c < (wg + 1) * kShare; c += kRun) {
+    uint32_t o[kRun];
+    if constexpr (kRun == 32) tmem_ld32(t_acc + c, o); else tmem_ld16(t_acc + c, o);
     tmem_wait_ld();
-    uint8_t* panel = stage + (c >> 1) * L::kPanelBytes + tid * 128;
+    uint8_t* panel = stage + (c >> 6) * L::kPanelBytes + tid * 128;
 #pragma unroll
-    for (int g = 0; g < 4; ++g) {
+    for (int g = 0; g < kRun / 8; ++g) {
       uint4 val;
       val.x = pack_bf16x2(mul * __uint_as_float(o[8 * g + 0]), mul * __uint_as_float(o[8 * g + 1]));
       val.y = pack_bf16x2(mul * __uint_as_float(o[8 * g + 2]), mul * __uint_as_float(o[8 * g + 3]));
       val.z = pack_bf16x2(mul * __uint_as_float(o[8 * g + 4]), mul * __uint_as_float(o[8 * g + 5]));
       val.w = pack_bf16x2(mul * __uint_as_float(o[8 * g + 6]), mul * __uint_as_float(o[8 * g + 7]));
-      const int chunk = (c & 1) * 4 + g;
-      *reinterpret_cast<uint4*>(panel + ((chunk ^ (tid & 7)) * 16)) = val;
+      *reinterpret_cast<uint4*>(panel + (((((c & 63) >> 3) + g) ^ (tid & 7)) * 16)) = val;
     }
   }
+}
+
+// What a thread's key row needs to know about query head bh_q.  Batch without padding: the queries [q_lo, q_hi) that see
+// the key (its own sequence, from the key itself on when causal), and the sequence's bias.
+struct BwdRow {
+  float slope_log2e, bias_log2e;
+  int q_lo, q_hi, seq;
+};
+template <bool CAUSAL, bool ALIBI, bool RAGGED>
+__device__ __forceinline__ BwdRow bwd_row(const BwdParams& p, int key, int bh_q) {
+  BwdRow r;
+  r.slope_log2e = ALIBI ? __ldg(p.slopes + bh_q % p.H) * kLog2eB : 0.0f;
+  r.bias_log2e = p.bias_log2e;
+  r.q_lo = r.q_hi = r.seq = 0;
+  if (!RAGGED) {
+    if (p.bias_vec) r.bias_log2e = __ldg(p.bias_vec + bh_q) * kLog2eB;
+  } else if (key < p.N) {
+    r.seq = bwd_seq_of_row(p.cu_seqlens, p.n_seqs, key);
+    r.q_lo = CAUSAL ? key : __ldg(p.cu_seqlens + r.seq);
+    r.q_hi = __ldg(p.cu_seqlens + r.seq + 1);
+    if (p.bias_vec) r.bias_log2e = __ldg(p.bias_vec + r.seq * p.H + bh_q) * kLog2eB;
+  }
+  return r;
 }
 
 // KIND: 0 plain, 1 general (grouped heads, padded batch), 2 general plus a batch stored without padding
@@ -554,37 +609,25 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
     return true;
   };
 
-  const bool dynamic = p.dynamic != 0;
-  for (int round = 0, rounds = bwd_num_rounds(p.n_items); dynamic || round < rounds; ++round) {
-    int item;
-    if (dynamic) {
-      if (!bwd_sched_take(bars, round, &item, cta_err)) return;
-      if (item < 0) break;
-    } else {
-      item = bwd_snake_rank(round, p.n_items);
-      if (item < 0) continue;
-    }
-    const BwdItem w = decode_bwd_item<CAUSAL, GROUPED>(p, item);
+  constexpr bool ragged = (KIND == 2);
+  // Whether the next item is looked up and dV stored while an item's last products run (see the epilogue).  Not in the
+  // causal general kinds with 64 columns a thread, whose steps it makes slower than it gains between items (B4 H16 H_kv4
+  // N2000 D64 157 us with it, 151 without; B2 H32 H_kv8 N4000 504 and 482; with items that every role decoded for itself
+  // and the results' buffers given back at once these were 147 and 470).
+  constexpr bool kAhead = !(D == 64 && CAUSAL && GROUPED && !WIDE);
+  bool release = false;   // the results that this thread stored may not have left their staging tile yet
+  BwdItem w;
+  int more = bwd_see_item(bars, 0, &w, cta_err);
+  if (more < 0) return;
+  BwdRow row;
+  if (kAhead && more) row = bwd_row<CAUSAL, ALIBI, ragged>(p, w.j * kT + tid, w.bh_q0);
+  while (more) {
     for (int g = 0; g < (GROUPED ? p.heads_per_sub : 1); ++g) {   // the query heads that read this key/value head
-    const int bh_q = w.bh_q0 + g;
-    float slope_log2e = 0.0f;
-    if (ALIBI) slope_log2e = p.slopes[bh_q % p.H] * kLog2eB;
-    float bias_log2e = p.bias_vec ? __ldg(p.bias_vec + bh_q) * kLog2eB : p.bias_log2e;
+    if (!kAhead) row = bwd_row<CAUSAL, ALIBI, ragged>(p, w.j * kT + tid, w.bh_q0 + g);
+    else if (g > 0) row = bwd_row<CAUSAL, ALIBI, ragged>(p, w.j * kT + tid, bars->sched_item[item_cnt & 1].bh_q0 + g);
+    const float slope_log2e = row.slope_log2e, bias_log2e = row.bias_log2e;
+    const int q_lo = row.q_lo, q_hi = row.q_hi, seq = row.seq;
     float ds_sum = 0.0f;   // this thread's share of sum dS over the head's tiles (the bias gradient)
-    // batch without padding: the queries [q_lo, q_hi) that see this thread's key (its own sequence,
-    // from the key itself on when causal), and the sequence's bias
-    constexpr bool ragged = (KIND == 2);
-    int q_lo = 0, q_hi = 0, seq = 0;
-    if (ragged) {
-      const int kr = w.j * kT + tid;
-      bias_log2e = p.bias_log2e;
-      if (kr < p.N) {
-        seq = bwd_seq_of_row(p.cu_seqlens, p.n_seqs, kr);
-        q_lo = CAUSAL ? kr : __ldg(p.cu_seqlens + seq);
-        q_hi = __ldg(p.cu_seqlens + seq + 1);
-        if (p.bias_vec) bias_log2e = __ldg(p.bias_vec + seq * p.H + bh_q) * kLog2eB;
-      }
-    }
 
     for (int it = 0; it < w.n; ++it) {
       const int i = w.i_begin + it;
@@ -632,12 +675,19 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
       tmem_wait_st();
       tc_fence_before_sync();
       mbar_arrive(smem_u32(&bars->p_ready[TM::r_index(step_cnt)]));
+      if (kAhead && release) {   // (one thread a result)
+        tma_wait_group_read<0>();
+        const uint32_t st = (item_cnt - 1) % L::kKvStages;
+        mbar_arrive(smem_u32(wg == 0 ? &bars->v_empty[st] : L::kKvStages == 1 ? &bars->ds_free : &bars->k_empty[st]));
+        release = false;
+      }
       if constexpr (!R::kDrainGroup) {
         if ((g > 0 || it > 0) && !drain(step_cnt - 1)) return;
       }
 
       // dS^T = P (1 - P) dP^T -> bf16 -> shared memory [key][query], 128-byte swizzle
       if (!mbar_wait(smem_u32(&bars->dp_full), step_cnt & 1, cta_err, 62 + wg)) return;
+      if (L::kKvStages == 1 && g == 0 && it == 0 && !mbar_wait(smem_u32(&bars->ds_free), (item_cnt & 1) ^ 1, cta_err, 68)) return;
       tc_fence_after_sync();
       uint8_t* ds_row = smem + L::kDsOff + (wg * kCols >> 6) * L::kPanelBytes + tid * 128;
 #pragma unroll
@@ -670,6 +720,7 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
       ++step_cnt;
     }
 
+    const int bh_q = DBIAS ? bars->sched_item[item_cnt & 1].bh_q0 + g : 0;
     if (DBIAS && ragged) {   // keys of one warp may belong to different sequences: one atomic per key
       if (q_hi > q_lo) atomicAdd(p.dbias + seq * p.H + bh_q, ds_sum);
     } else if (DBIAS) {   // sum over the warp, one atomic per warp, item and query head
@@ -679,34 +730,82 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
     }
     }   // query heads
 
-    if constexpr (!R::kDrainGroup) {
-      if (!drain(step_cnt - 1)) return;
-    }
-
-    // epilogue: the first half of the groups stores dV_j (staged in the V tile), the other half scale * dK_j (K tile)
-    if (!mbar_wait(smem_u32(&bars->dkv_full), item_cnt & 1, cta_err, 64 + wg)) return;
-    const uint32_t kv_stage = item_cnt % L::kKvStages;
-    ++item_cnt;
-    tc_fence_after_sync();
-    const bool is_dv = wg < R::kGroups / 2;
-    uint8_t* stage = smem + kv_stage * L::kKvBytes + (is_dv ? L::kVOff : L::kKOff);
-    bwd_store_acc_rows<D, WIDE>(tmem + (is_dv ? TM::kDv : TM::kDk) + lane_off, stage, tid, is_dv ? 1.0f : p.scale,
-                          wg % (R::kGroups / 2));
-    tc_fence_before_sync();
-    mbar_arrive(smem_u32(&bars->dkv_empty));
-    fence_proxy_async_smem();
-    if (is_dv) named_barrier_sync<1, R::kActThreads / 2>(); else named_barrier_sync<2, R::kActThreads / 2>();
-    if (tid == 0 && wg % (R::kGroups / 2) == 0) {
-      const CUtensorMap* tm = is_dv ? tmDv : tmDk;
-#pragma unroll
-      for (int pn = 0; pn < L::kPanels; ++pn)
-        if (GROUPED && (p.n_sub > 1 || p.i_split > 1 || p.dkv_add))   // the parts (or successive calls) add their shares
-          tma_reduce_add_3d(tm, smem_u32(stage + pn * L::kPanelBytes), pn * 64, w.j * kT, w.bh);
+    // Epilogue.  While the last dK and dQ are computed, the next item is looked up and dV, complete before them, is
+    // converted and stored from the V buffer; then scale * dK, from the K buffer (D = 128: from where dS was).  The
+    // buffers go back once the stores have read them: with two of them after the next P phase, by when they have.
+    // Waited for at once, with both results converted after the last product and the next item looked up then, the
+    // threads stood 5000 to 6000 cycles between two items (clock traces).  Whole backward, us, that way / this way:
+    // B16 H12 N577 D64 94.5 / 90.3, B16 H16 N512 D64 causal 82.9 / 79.0, B16 H8 padded N1500 D64 225.7 / 216.9,
+    // 60 documents in 16384 rows D64 223 / 208.5, B4 H16 N1024 D128 causal ALiBi 87.8 / 80.0,
+    // B2 H16 N4096 D128 causal 428 / 418.
+    if constexpr (!kAhead) {   // one group converts dV, the other dK
+      const uint32_t st = item_cnt % L::kKvStages;
+      if (!mbar_wait(smem_u32(&bars->dkv_full), item_cnt & 1, cta_err, 64 + wg)) return;
+      tc_fence_after_sync();
+      uint8_t* stage = smem + st * L::kKvBytes + (wg == 0 ? L::kVOff : L::kKOff);
+#pragma unroll 1
+      for (int share = 0; share < R::kGroups; ++share)
+        bwd_store_acc_rows<D, WIDE>(tmem + (wg == 0 ? TM::kDv : TM::kDk) + lane_off, stage, tid, wg == 0 ? 1.0f : p.scale, share);
+      tc_fence_before_sync();
+      mbar_arrive(smem_u32(&bars->dkv_empty));
+      fence_proxy_async_smem();
+      if (wg == 0) named_barrier_sync<1, 128>(); else named_barrier_sync<2, 128>();
+      if (tid == 0) {
+        const CUtensorMap* tm = wg == 0 ? tmDv : tmDk;
+        if (p.n_sub > 1 || p.i_split > 1 || p.dkv_add)
+          tma_reduce_add_3d(tm, smem_u32(stage), 0, w.j * kT, w.bh);
         else
-          tma_store_3d(tm, smem_u32(stage + pn * L::kPanelBytes), pn * 64, w.j * kT, w.bh);
-      tma_commit_group();
+          tma_store_3d(tm, smem_u32(stage), 0, w.j * kT, w.bh);
+        tma_commit_group();
+        tma_wait_group_read<0>();
+        mbar_arrive(smem_u32(wg == 0 ? &bars->v_empty[st] : &bars->k_empty[st]));
+      }
+      bwd_return_item(bars, item_cnt);
+      ++item_cnt;
+      more = bwd_see_item(bars, item_cnt, &w, cta_err);
+      if (more < 0) return;
+    } else {
+    const int done_row = bars->sched_item[item_cnt & 1].j * kT, done_bh = bars->sched_item[item_cnt & 1].bh;
+    bwd_return_item(bars, item_cnt);
+    more = bwd_see_item(bars, item_cnt + 1, &w, cta_err);
+    if (more < 0) return;
+    if (more) row = bwd_row<CAUSAL, ALIBI, ragged>(p, w.j * kT + tid, w.bh_q0);
+    const uint32_t kv_stage = item_cnt % L::kKvStages;
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const bool is_dv = r == 0;
+      if (!mbar_wait(smem_u32(is_dv ? &bars->dv_full : &bars->dkv_full), item_cnt & 1, cta_err, is_dv ? 66 : 64)) return;
+      tc_fence_after_sync();
+      uint8_t* stage = smem + (is_dv ? kv_stage * L::kKvBytes + L::kVOff
+                                     : L::kKvStages == 1 ? L::kDsOff : kv_stage * L::kKvBytes + L::kKOff);
+      bwd_store_acc_rows<D, WIDE>(tmem + (is_dv ? TM::kDv : TM::kDk) + lane_off, stage, tid, is_dv ? 1.0f : p.scale, wg);
+      if (!is_dv) {
+        tc_fence_before_sync();
+        mbar_arrive(smem_u32(&bars->dkv_empty));
+      }
+      fence_proxy_async_smem();
+      named_barrier_sync<1, R::kActThreads>();
+      if (tid == 0 && wg == r) {
+        const CUtensorMap* tm = is_dv ? tmDv : tmDk;
+#pragma unroll
+        for (int pn = 0; pn < L::kPanels; ++pn)
+          if (GROUPED && (p.n_sub > 1 || p.i_split > 1 || p.dkv_add))   // the parts (or successive calls) add their shares
+            tma_reduce_add_3d(tm, smem_u32(stage + pn * L::kPanelBytes), pn * 64, done_row, done_bh);
+          else
+            tma_store_3d(tm, smem_u32(stage + pn * L::kPanelBytes), pn * 64, done_row, done_bh);
+        tma_commit_group();
+        release = true;
+      }
+      if constexpr (!R::kDrainGroup) {
+        if (is_dv && !drain(step_cnt - 1)) return;
+      }
+    }
+    ++item_cnt;
+    if (L::kKvStages == 1 && tid == 0 && wg == 0) {   // the next V is waited for
       tma_wait_group_read<0>();
-      mbar_arrive(smem_u32(&bars->kv_empty[kv_stage]));
+      mbar_arrive(smem_u32(&bars->v_empty[0]));
+      release = false;
+    }
     }
   }
   if (tid == 0) tma_wait_group<0>();
@@ -714,7 +813,7 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
 
 // ------------------------------------------------------------------ dQ drain group
 
-template <int D, bool CAUSAL, bool GROUPED>
+template <int D, bool GROUPED>
 __device__ void bwd_drain_role(const BwdParams& p, const CUtensorMap* tmW, uint8_t* smem, uint32_t tmem,
                                BwdBarriers* bars, volatile int* cta_err) {
   using L = BwdSmem<D>;
@@ -722,17 +821,9 @@ __device__ void bwd_drain_role(const BwdParams& p, const CUtensorMap* tmW, uint8
   const int tid = threadIdx.x & 127;  // query row within the tile
   const uint32_t lane_off = static_cast<uint32_t>(((threadIdx.x >> 5) & 3) * 32) << 16;
   uint32_t step_cnt = 0;
-  const bool dynamic = p.dynamic != 0;
-  for (int round = 0, rounds = bwd_num_rounds(p.n_items); dynamic || round < rounds; ++round) {
-    int item;
-    if (dynamic) {
-      if (!bwd_sched_take(bars, round, &item, cta_err)) return;
-      if (item < 0) break;
-    } else {
-      item = bwd_snake_rank(round, p.n_items);
-      if (item < 0) continue;
-    }
-    const BwdItem w = decode_bwd_item<CAUSAL, GROUPED>(p, item);
+  for (uint32_t number = 0;; ++number) {
+    BwdItem w;
+    if (bwd_take_item(bars, number, &w, cta_err) <= 0) break;
     for (int s = 0; s < w.steps; ++s) {
       const int g = GROUPED ? s / w.n : 0, it = s - g * w.n;   // query head within the group, query tile
       const int row0 = (w.i_begin + it) * kT, bh_q = w.bh_q0 + g;
@@ -778,22 +869,14 @@ __device__ void bwd_drain_role(const BwdParams& p, const CUtensorMap* tmW, uint8
 }
 
 // Wide: one thread adds the staged dQ tiles to the fp32 accumulator.
-template <int D, bool CAUSAL, bool GROUPED>
+template <int D>
 __device__ void bwd_store_role(const BwdParams& p, const CUtensorMap* tmW, uint32_t smem_base, BwdBarriers* bars,
                                volatile int* cta_err) {
   using L = BwdSmem<D>;
   uint32_t step_cnt = 0;
-  const bool dynamic = p.dynamic != 0;
-  for (int round = 0, rounds = bwd_num_rounds(p.n_items); dynamic || round < rounds; ++round) {
-    int item;
-    if (dynamic) {
-      if (!bwd_sched_take(bars, round, &item, cta_err)) return;
-      if (item < 0) break;
-    } else {
-      item = bwd_snake_rank(round, p.n_items);
-      if (item < 0) continue;
-    }
-    const BwdItem w = decode_bwd_item<CAUSAL, GROUPED>(p, item);
+  for (uint32_t number = 0;; ++number) {
+    BwdItem w;
+    if (bwd_take_item(bars, number, &w, cta_err) <= 0) break;
     int it = 0, bh_q = w.bh_q0;
     for (int s = 0; s < w.steps; ++s, ++step_cnt) {
       if (!mbar_wait(smem_u32(&bars->stage_full), step_cnt & 1, cta_err, 75)) return;
@@ -833,8 +916,10 @@ sigattn_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   if (threadIdx.x == 0) {
     cta_err = 0;
     for (int s = 0; s < 2; ++s) {
-      mbar_init(smem_u32(&bars.kv_full[s]), 1);
-      mbar_init(smem_u32(&bars.kv_empty[s]), 2);
+      mbar_init(smem_u32(&bars.k_full[s]), 1);
+      mbar_init(smem_u32(&bars.v_full[s]), 1);
+      mbar_init(smem_u32(&bars.k_empty[s]), 1);
+      mbar_init(smem_u32(&bars.v_empty[s]), 1);
     }
     for (int s = 0; s < 3; ++s) {
       mbar_init(smem_u32(&bars.q_full[s]), 1);
@@ -850,13 +935,15 @@ sigattn_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     }
     mbar_init(smem_u32(&bars.dp_full), 1);
     mbar_init(smem_u32(&bars.ds_ready), R::kActThreads);
+    mbar_init(smem_u32(&bars.dv_full), 1);
     mbar_init(smem_u32(&bars.dkv_full), 1);
+    mbar_init(smem_u32(&bars.ds_free), 1);
     mbar_init(smem_u32(&bars.stage_full), R::kActThreads);
     mbar_init(smem_u32(&bars.stage_empty), 1);
     mbar_init(smem_u32(&bars.dkv_empty), R::kActThreads);
     for (int s = 0; s < 2; ++s) {
       mbar_init(smem_u32(&bars.sched_full[s]), 1);
-      mbar_init(smem_u32(&bars.sched_empty[s]), BwdRoles<D, WIDE>::kSchedConsumers);
+      mbar_init(smem_u32(&bars.sched_empty[s]), BwdRoles<D, WIDE>::kItemReaders);
     }
     mbar_init(smem_u32(&bars.sched_answer), 1);
     fence_mbar_init();
@@ -885,14 +972,14 @@ sigattn_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     if ((threadIdx.x & 31) == 0) bwd_load_role<D, CAUSAL, GROUPED>(p, &tmQ, &tmK, &tmV, &tmDo, smem_base, &bars, &cta_err);
     __syncwarp();
   } else if (warp == R::kMmaWarp) {
-    if (elect_one()) bwd_mma_role<D, CAUSAL, GROUPED, WIDE>(p, smem_base, tmem, &bars, &cta_err);
+    if (elect_one()) bwd_mma_role<D, WIDE>(smem_base, tmem, &bars, &cta_err);
     __syncwarp();
   } else if (warp < 4 * R::kGroups) {
     bwd_act_role<D, CAUSAL, ALIBI, DBIAS, KIND, WIDE>(p, &tmDk, &tmDv, warp >> 2, smem, tmem, &bars, &cta_err);
   } else if constexpr (R::kDrainGroup) {
-    bwd_drain_role<D, CAUSAL, GROUPED>(p, &tmW, smem, tmem, &bars, &cta_err);
+    bwd_drain_role<D, GROUPED>(p, &tmW, smem, tmem, &bars, &cta_err);
   } else {
-    if (elect_one()) bwd_store_role<D, CAUSAL, GROUPED>(p, &tmW, smem_base, &bars, &cta_err);
+    if (elect_one()) bwd_store_role<D>(p, &tmW, smem_base, &bars, &cta_err);
     __syncwarp();
   }
 
@@ -1167,6 +1254,7 @@ int launch_bwd_bf16(const void* q, const void* k, const void* v, const void* d_o
   // the bias gradient costs the activation groups a running sum (4-5 % of the kernel), so it
   // is compiled in only where it is asked for; likewise the loop over a group's query heads and
   // the per-sequence lengths (kind 1) and the lookups of a batch without padding (kind 2)
+  // (The figures below were taken before the next item was looked up ahead, which made the wide shape 2 to 7 % faster.)
   // Wide or narrow (see BwdRoles).  Short sequences have b = -log n near the common path's limit, so many warps take
   // both activation paths, and items of few steps; there four groups pay.  Long ones are bound by the other work of
   // those groups.  The line is drawn by the length a typical row sees.  Whole backward, us, narrow / wide, H12 or 16:
@@ -1178,12 +1266,13 @@ int launch_bwd_bf16(const void* q, const void* k, const void* v, const void* d_o
   // bytes spilled in its general instantiations); causal calls with grouped heads have more steps an item.  B16 H12:
   //   ALiBi, no mask: N300 48 / 47, N577 102 / 102, N1025 256 / 268, N1250 326 / 334; H_kv4 N300 68 / 66, N577 132 / 144,
   //   N1250 384 / 420; padded N577 113 / 110, N1250 285 / 268, N2400 1142 / 1134; 60 documents 335 / 332, 16 645 / 682;
-  //   causal H_kv4: N300 57 / 55, N577 84 / 74, N1025 158 / 160; B4 H16 H_kv4 N1900 134 / 141.
+  //   causal H_kv4: N300 57 / 55, N577 84 / 74; with the next item looked up ahead (wide only) B8 H16 H_kv4 N1000 117 / 104,
+  //   B4 N1500 103 / 102, N2000 151 / 147 (ALiBi 167 / 152), N3000 326 / 340, B2 H32 H_kv8 N4000 484 / 500.
   const int typical_rows = p.cu_seqlens != nullptr ? p.N / p.n_seqs
                            : p.seqlens != nullptr  ? p.N / 2
                            : p.causal              ? p.N / 3 * 2 : p.N;
   const bool grouped_causal = p.causal && bp.group > 1 && p.seqlens == nullptr && p.cu_seqlens == nullptr;
-  const int wide_rows = (p.slopes != nullptr && !p.causal && p.seqlens == nullptr) ? 512 : grouped_causal ? 600 : 1280;
+  const int wide_rows = (p.slopes != nullptr && !p.causal && p.seqlens == nullptr) ? 512 : grouped_causal ? 1400 : 1280;
   const bool wide = p.D == 64 && typical_rows <= wide_rows;
 #define SIGATTN_BWD_SHAPE(DD, CC, AA, BB, KK)                                                              \
   ((DD == 64 && wide) ? launch_bwd_variant<DD, CC, AA, BB, KK, DD == 64>(maps, bp, num_sms, stream, cuda_err) \
