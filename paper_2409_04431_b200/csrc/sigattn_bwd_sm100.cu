@@ -517,8 +517,10 @@ __device__ void bwd_mma_role(uint32_t smem_base, uint32_t tmem, BwdBarriers* bar
       ++q_cnt;
       ++step_cnt;
     }
-    umma_commit(smem_u32(&bars->dkv_full));
+    // (the commit that the epilogue waits for comes last: after a block's last item nothing waits for k_empty, and no
+    // arrival may be on its way when the block ends)
     if (L::kKvStages == 1) umma_commit(smem_u32(&bars->k_empty[0]));
+    umma_commit(smem_u32(&bars->dkv_full));
     ++item_cnt;
   }
 }
