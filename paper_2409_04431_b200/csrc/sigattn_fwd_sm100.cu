@@ -278,6 +278,15 @@ __device__ __forceinline__ Item decode_item(const FwdParams& p, int item) {
   return w;
 }
 
+// Whether the polls of a wait are unrolled (see mbar_wait_limit).  Plain calls without a mask at D = 64 are bound by the
+// chain from a tile's logits to the next product and small enough for the instruction cache; there a loop of single polls,
+// which answers a little later, costs more than its shorter code gains.  Forward, us, all unrolled / loop / the activation
+// threads' unrolled and eight at a time in the issuing thread: B8 H12 N4096 563 / 572 / 566, B2 H12 N8100 620 / 630 / 620,
+// B4 H16 N3000 243 / 246 / 243, N2048 168.6 / 169.6 / 167.7, B16 H12 N1025 113.7 / 112.9 / 111.7, B4 H12 N577 15.5 / 14.8 / 15.0.
+// Everywhere else the loop is the fastest: causal ALiBi B8 H16 N2048 133.9 / 127.6 / 128.7 (eight at a time in all roles),
+// padded B16 H8 N1500 103.5 / 94.6 / 95.5, 16 documents in 16384 rows D64 185.9 / 168.8 / 170.3.
+__host__ __device__ constexpr bool fwd_polls_unrolled(int D, bool masked_or_general) { return D == 64 && !masked_or_general; }
+
 // ------------------------------------------------------------------ producer
 
 template <int D, bool CAUSAL, bool GENERAL>   // GENERAL: always dynamic
@@ -346,6 +355,7 @@ __device__ void fwd_mma_role(const FwdParams& p, uint32_t smem_base, uint32_t tm
   using L = FwdSmem<D>;
   constexpr uint32_t kIdescS = make_idesc_bf16(kBM, kBN, 0, 0);
   constexpr uint32_t kIdescPV = make_idesc_bf16(kBM, D, 0, 1);
+  constexpr int kPolls = fwd_polls_unrolled(D, CAUSAL || GENERAL) ? 8 : 1;
   uint32_t kv_cnt = 0;
   uint32_t it[2] = {0, 0};      // items seen per query tile
   uint32_t p_cnt[2] = {0, 0};   // P tiles consumed per query tile
@@ -377,7 +387,7 @@ __device__ void fwd_mma_role(const FwdParams& p, uint32_t smem_base, uint32_t tm
   };
   auto kv_wait = [&](uint32_t cnt) -> bool {
     const uint32_t stage = cnt % L::kStages, phase = (cnt / L::kStages) & 1;
-    return mbar_wait(smem_u32(&bars->kv_full[stage]), phase, cta_err, 20);
+    return mbar_wait<kPolls>(smem_u32(&bars->kv_full[stage]), phase, cta_err, 20);
   };
   auto kv_addr = [&](uint32_t cnt) { return smem_base + L::kKvOff + (cnt % L::kStages) * L::kTileBytes; };
   auto kv_release = [&](uint32_t cnt) { umma_commit(smem_u32(&bars->kv_empty[cnt % L::kStages])); };
@@ -399,14 +409,14 @@ __device__ void fwd_mma_role(const FwdParams& p, uint32_t smem_base, uint32_t tm
     auto v_cnt = [&](int j) { return base_cnt + 2 * j + 1; };
 
     // first logits
-    if (!mbar_wait(smem_u32(&bars->q_full[0]), it[0] & 1, cta_err, 21)) return;
+    if (!mbar_wait<kPolls>(smem_u32(&bars->q_full[0]), it[0] & 1, cta_err, 21)) return;
     if (!kv_wait(k_cnt(0))) return;
     tc_fence_after_sync();
     issue_s(0, kv_addr(k_cnt(0)));
     umma_commit(smem_u32(&bars->s_full[0]));
     if (L::kOStaged && w.n[0] == 1) umma_commit(smem_u32(&bars->q_empty[0]));   // Q_0 no longer needed
     if (w.n[1] > 0) {
-      if (!mbar_wait(smem_u32(&bars->q_full[1]), it[1] & 1, cta_err, 22)) return;
+      if (!mbar_wait<kPolls>(smem_u32(&bars->q_full[1]), it[1] & 1, cta_err, 22)) return;
       tc_fence_after_sync();
       issue_s(1, kv_addr(k_cnt(0)));
       umma_commit(smem_u32(&bars->s_full[1]));
@@ -414,14 +424,14 @@ __device__ void fwd_mma_role(const FwdParams& p, uint32_t smem_base, uint32_t tm
     }
     kv_release(k_cnt(0));
     // accumulators of the previous item must have been read out before the first PV overwrites them
-    if (!mbar_wait(smem_u32(&bars->o_empty[0]), (it[0] & 1) ^ 1, cta_err, 23)) return;
-    if (w.n[1] > 0 && !mbar_wait(smem_u32(&bars->o_empty[1]), (it[1] & 1) ^ 1, cta_err, 24)) return;
+    if (!mbar_wait<kPolls>(smem_u32(&bars->o_empty[0]), (it[0] & 1) ^ 1, cta_err, 23)) return;
+    if (w.n[1] > 0 && !mbar_wait<kPolls>(smem_u32(&bars->o_empty[1]), (it[1] & 1) ^ 1, cta_err, 24)) return;
 
     for (int j = 0; j < w.n_kv; ++j) {
       if (!kv_wait(v_cnt(j))) return;
       const bool more = (j + 1 < w.n_kv);
       if (j < w.n[0]) {
-        if (!mbar_wait(smem_u32(&bars->p_full[0]), p_cnt[0] & 1, cta_err, 25)) return;
+        if (!mbar_wait<kPolls>(smem_u32(&bars->p_full[0]), p_cnt[0] & 1, cta_err, 25)) return;
         ++p_cnt[0];
         tc_fence_after_sync();
         issue_pv(0, kv_addr(v_cnt(j)), j > 0);
@@ -435,7 +445,7 @@ __device__ void fwd_mma_role(const FwdParams& p, uint32_t smem_base, uint32_t tm
         if (L::kOStaged && j + 2 == w.n[0]) umma_commit(smem_u32(&bars->q_empty[0]));
       }
       if (j < w.n[1]) {
-        if (!mbar_wait(smem_u32(&bars->p_full[1]), p_cnt[1] & 1, cta_err, 26)) return;
+        if (!mbar_wait<kPolls>(smem_u32(&bars->p_full[1]), p_cnt[1] & 1, cta_err, 26)) return;
         ++p_cnt[1];
         tc_fence_after_sync();
         issue_pv(1, kv_addr(v_cnt(j)), j > 0);
@@ -491,6 +501,7 @@ __device__ void fwd_act_role(const FwdParams& p, const CUtensorMap* tmO, uint8_t
   const int g = threadIdx.x >> 7;            // column group of the tile
   const int tid = threadIdx.x & 127;         // row of the tile
   const uint32_t lane_off = static_cast<uint32_t>(((threadIdx.x >> 5) & 3) * 32) << 16;
+  constexpr int kPolls = fwd_polls_unrolled(D, CAUSAL || MODE != 0) ? 64 : 1;
   uint32_t s_cnt0 = 0, s_cnt1 = 0, it[2] = {0, 0};
 
   const bool dynamic = GENERAL || p.dynamic;
@@ -546,7 +557,7 @@ __device__ void fwd_act_role(const FwdParams& p, const CUtensorMap* tmO, uint8_t
       for (int t = 0; t < kTiles; ++t) {
         if (j >= w.n[t]) continue;
         uint32_t& cnt = t ? s_cnt1 : s_cnt0;
-        if (!mbar_wait(smem_u32(&bars->s_full[t]), cnt & 1, cta_err, 30 + t)) return;
+        if (!mbar_wait<kPolls>(smem_u32(&bars->s_full[t]), cnt & 1, cta_err, 30 + t)) return;
         ++cnt;
         tc_fence_after_sync();
         const int jk = (PACKED || GENERAL) ? w.j0 + j : j;   // key tile (split keys, unpadded batches: items start later)
@@ -600,7 +611,7 @@ __device__ void fwd_act_role(const FwdParams& p, const CUtensorMap* tmO, uint8_t
 #pragma unroll
     for (int t = 0; t < kTiles; ++t) {
       if (w.n[t] == 0) continue;
-      if (!mbar_wait(smem_u32(&bars->o_full[t]), it[t] & 1, cta_err, 32 + t)) return;
+      if (!mbar_wait<kPolls>(smem_u32(&bars->o_full[t]), it[t] & 1, cta_err, 32 + t)) return;
       ++it[t];
       tc_fence_after_sync();
       uint8_t* stage = smem + (L::kOStaged ? L::kOOff : L::kQOff) + t * L::kTileBytes;

@@ -62,8 +62,10 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 // failure, the wait gives up, records the failure in `*cta_error` (shared memory) and
 // returns false.  Callers leave their loops on false and fall through to the common
 // tear-down, so the kernel always terminates and frees its tensor memory.
+// UNROLL: how many of 64 polls follow one another in the code.
 constexpr long long kWaitLimitCycles = 2000000000LL;  // about one second
 
+template <int UNROLL = 1>
 __device__ __forceinline__ bool mbar_wait_limit(uint32_t bar, uint32_t parity, volatile int* cta_error, int where,
                                                 long long limit_cycles) {
   if (mbar_try_wait(bar, parity)) return true;
@@ -74,7 +76,7 @@ __device__ __forceinline__ bool mbar_wait_limit(uint32_t bar, uint32_t parity, v
     // D = 64, code 148 -> 88 KB, warps stalled for instructions 1.79 -> 0.93 of those issued (B8 H8 N2700 padded).
     // Whole backward, us, unrolled / loop: B8 H8 N2700 D64 padded 362 / 300, B4 H32 H_kv8 N3000 D64 causal ALiBi 699 / 639,
     // B8 H16 N2048 D64 causal ALiBi 325 / 302, 60 documents in 16384 rows D64 208 / 187, D128 313 / 286.
-#pragma unroll 1
+#pragma unroll UNROLL
     for (int i = 0; i < 64; ++i) {
       if (mbar_try_wait(bar, parity)) return true;
     }
@@ -86,8 +88,9 @@ __device__ __forceinline__ bool mbar_wait_limit(uint32_t bar, uint32_t parity, v
   }
 }
 
+template <int UNROLL = 1>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* cta_error, int where) {
-  return mbar_wait_limit(bar, parity, cta_error, where, kWaitLimitCycles);
+  return mbar_wait_limit<UNROLL>(bar, parity, cta_error, where, kWaitLimitCycles);
 }
 
 // Four consecutive floats added to global memory (16-byte aligned), no return value.
