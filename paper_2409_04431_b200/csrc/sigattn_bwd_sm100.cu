@@ -196,20 +196,22 @@ __device__ __forceinline__ bool bwd_hand_item(BwdBarriers* bars, uint32_t number
   mbar_arrive(smem_u32(&bars->sched_full[slot]));
   return true;
 }
-// 1 and *w, 0 when no item is left, -1 when a bounded wait expired.  (The activation threads keep the slot until the item
-// is done and read there what the steps do not need: their registers are full.)
-__device__ __forceinline__ int bwd_see_item(BwdBarriers* bars, uint32_t number, BwdItem* w, volatile int* cta_err) {
+// 1 when the slot holds an item, 0 when none is left, -1 when a bounded wait expired.  The activation threads keep the
+// slot until the item is done and read its fields there, also at each step: their registers are full.  With the item
+// copied (seven values, and a row's sequence, in every thread) the general instantiations at D = 64 spilled 32 to 56 bytes.
+__device__ __forceinline__ int bwd_see_item(BwdBarriers* bars, uint32_t number, volatile int* cta_err) {
   const uint32_t slot = number & 1, phase = (number >> 1) & 1;
   if (!mbar_wait(smem_u32(&bars->sched_full[slot]), phase, cta_err, 71)) return -1;
-  *w = bars->sched_item[slot];
-  return w->steps > 0 ? 1 : 0;
+  return bars->sched_item[slot].steps > 0 ? 1 : 0;
 }
 __device__ __forceinline__ void bwd_return_item(BwdBarriers* bars, uint32_t number) {
   mbar_arrive(smem_u32(&bars->sched_empty[number & 1]));
 }
 __device__ __forceinline__ int bwd_take_item(BwdBarriers* bars, uint32_t number, BwdItem* w, volatile int* cta_err) {
-  const int more = bwd_see_item(bars, number, w, cta_err);
-  if (more >= 0) bwd_return_item(bars, number);
+  const int more = bwd_see_item(bars, number, cta_err);
+  if (more < 0) return more;
+  *w = bars->sched_item[number & 1];
+  bwd_return_item(bars, number);
   return more;
 }
 
@@ -550,25 +552,26 @@ __device__ __forceinline__ void bwd_store_acc_rows(uint32_t t_acc, uint8_t* stag
   }
 }
 
-// What a thread's key row needs to know about query head bh_q.  Batch without padding: the queries [q_lo, q_hi) that see
-// the key (its own sequence, from the key itself on when causal), and the sequence's bias.
+// What a thread's key row needs to know about the item's query head g.  Batch without padding: the queries [q_lo, q_hi)
+// that see the key (its own sequence, from the key itself on when causal), and the sequence's bias.
 struct BwdRow {
   float slope_log2e, bias_log2e;
-  int q_lo, q_hi, seq;
+  int q_lo, q_hi;
 };
 template <bool CAUSAL, bool ALIBI, bool RAGGED>
-__device__ __forceinline__ BwdRow bwd_row(const BwdParams& p, int key, int bh_q) {
+__device__ __forceinline__ BwdRow bwd_row(const BwdParams& p, const BwdItem& w, int tid, int g) {
+  const int key = w.j * kT + tid, bh_q = w.bh_q0 + g;
   BwdRow r;
   r.slope_log2e = ALIBI ? __ldg(p.slopes + bh_q % p.H) * kLog2eB : 0.0f;
   r.bias_log2e = p.bias_log2e;
-  r.q_lo = r.q_hi = r.seq = 0;
+  r.q_lo = r.q_hi = 0;
   if (!RAGGED) {
     if (p.bias_vec) r.bias_log2e = __ldg(p.bias_vec + bh_q) * kLog2eB;
   } else if (key < p.N) {
-    r.seq = bwd_seq_of_row(p.cu_seqlens, p.n_seqs, key);
-    r.q_lo = CAUSAL ? key : __ldg(p.cu_seqlens + r.seq);
-    r.q_hi = __ldg(p.cu_seqlens + r.seq + 1);
-    if (p.bias_vec) r.bias_log2e = __ldg(p.bias_vec + r.seq * p.H + bh_q) * kLog2eB;
+    const int seq = bwd_seq_of_row(p.cu_seqlens, p.n_seqs, key);
+    r.q_lo = CAUSAL ? key : __ldg(p.cu_seqlens + seq);
+    r.q_hi = __ldg(p.cu_seqlens + seq + 1);
+    if (p.bias_vec) r.bias_log2e = __ldg(p.bias_vec + seq * p.H + bh_q) * kLog2eB;
   }
   return r;
 }
@@ -576,8 +579,8 @@ __device__ __forceinline__ BwdRow bwd_row(const BwdParams& p, int key, int bh_q)
 // KIND: 0 plain, 1 general (grouped heads, padded batch), 2 general plus a batch stored without padding
 template <int D, bool CAUSAL, bool ALIBI, bool DBIAS, int KIND, bool WIDE>
 __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const CUtensorMap* tmDv,
-                             int wg,
-                             uint8_t* smem, uint32_t tmem, BwdBarriers* bars, volatile int* cta_err) {
+                             int wg, uint8_t* smem, uint32_t smem_base, uint32_t tmem, BwdBarriers* bars,
+                             volatile int* cta_err) {
   using L = BwdSmem<D>;
   using TM = BwdTmem<D>;
   using R = BwdRoles<D, WIDE>;
@@ -601,38 +604,31 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
     tc_fence_before_sync();
     mbar_arrive(smem_u32(&bars->dq_empty[reg]));
     if (!mbar_wait(smem_u32(&bars->stage_empty), (step & 1) ^ 1, cta_err, 74)) return false;
-    uint8_t* box = smem + L::kDqOff + (wg >> 1) * L::kPanelBytes + tid * 128;
+    const uint32_t box = smem_base + L::kDqOff + (wg >> 1) * L::kPanelBytes + tid * 128;
 #pragma unroll
-    for (int e = 0; e < 4; ++e)
-      *reinterpret_cast<uint4*>(box + ((((wg & 1) * 4 + e) ^ (tid & 7)) * 16)) =
-          make_uint4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]);
+    for (int e = 0; e < 4; ++e) st_shared_v4(box + ((((wg & 1) * 4 + e) ^ (tid & 7)) * 16), o + 4 * e);
     fence_proxy_async_smem();
     mbar_arrive(smem_u32(&bars->stage_full));
     return true;
   };
 
   constexpr bool ragged = (KIND == 2);
-  // Whether the next item is looked up and dV stored while an item's last products run (see the epilogue).  Not in the
-  // causal general kinds with 64 columns a thread, whose steps it makes slower than it gains between items (B4 H16 H_kv4
-  // N2000 D64 157 us with it, 151 without; B2 H32 H_kv8 N4000 504 and 482; with items that every role decoded for itself
-  // and the results' buffers given back at once these were 147 and 470).
-  constexpr bool kAhead = !(D == 64 && CAUSAL && GROUPED && !WIDE);
+  auto item = [&]() -> const BwdItem& { return bars->sched_item[item_cnt & 1]; };
   bool release = false;   // the results that this thread stored may not have left their staging tile yet
-  BwdItem w;
-  int more = bwd_see_item(bars, 0, &w, cta_err);
+  int more = bwd_see_item(bars, 0, cta_err);
   if (more < 0) return;
   BwdRow row;
-  if (kAhead && more) row = bwd_row<CAUSAL, ALIBI, ragged>(p, w.j * kT + tid, w.bh_q0);
+  if (more) row = bwd_row<CAUSAL, ALIBI, ragged>(p, item(), tid, 0);
   while (more) {
     for (int g = 0; g < (GROUPED ? p.heads_per_sub : 1); ++g) {   // the query heads that read this key/value head
-    if (!kAhead) row = bwd_row<CAUSAL, ALIBI, ragged>(p, w.j * kT + tid, w.bh_q0 + g);
-    else if (g > 0) row = bwd_row<CAUSAL, ALIBI, ragged>(p, w.j * kT + tid, bars->sched_item[item_cnt & 1].bh_q0 + g);
+    if (g > 0) row = bwd_row<CAUSAL, ALIBI, ragged>(p, item(), tid, g);
     const float slope_log2e = row.slope_log2e, bias_log2e = row.bias_log2e;
-    const int q_lo = row.q_lo, q_hi = row.q_hi, seq = row.seq;
+    const int q_lo = row.q_lo, q_hi = row.q_hi;
     float ds_sum = 0.0f;   // this thread's share of sum dS over the head's tiles (the bias gradient)
 
-    for (int it = 0; it < w.n; ++it) {
-      const int i = w.i_begin + it;
+    const int i_first = item().i_begin, i_end = i_first + item().n;
+    for (int i = i_first; i < i_end; ++i) {
+      const BwdItem& w = item();
       // this thread's key index minus the position of the tile's first query
       const float col_rel = static_cast<float>((w.j - i) * kT + tid - p.pos0);
       // the mask cuts through the tile unless even its first query sits at or after the last key:
@@ -677,21 +673,23 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
       tmem_wait_st();
       tc_fence_before_sync();
       mbar_arrive(smem_u32(&bars->p_ready[TM::r_index(step_cnt)]));
-      if (kAhead && release) {   // (one thread a result)
+      if (release) {   // (one thread a result)
         tma_wait_group_read<0>();
         const uint32_t st = (item_cnt - 1) % L::kKvStages;
         mbar_arrive(smem_u32(wg == 0 ? &bars->v_empty[st] : L::kKvStages == 1 ? &bars->ds_free : &bars->k_empty[st]));
         release = false;
       }
       if constexpr (!R::kDrainGroup) {
-        if ((g > 0 || it > 0) && !drain(step_cnt - 1)) return;
+        if ((g > 0 || i > i_first) && !drain(step_cnt - 1)) return;
       }
 
       // dS^T = P (1 - P) dP^T -> bf16 -> shared memory [key][query], 128-byte swizzle
       if (!mbar_wait(smem_u32(&bars->dp_full), step_cnt & 1, cta_err, 62 + wg)) return;
-      if (L::kKvStages == 1 && g == 0 && it == 0 && !mbar_wait(smem_u32(&bars->ds_free), (item_cnt & 1) ^ 1, cta_err, 68)) return;
+      if (L::kKvStages == 1 && g == 0 && i == i_first &&
+          !mbar_wait(smem_u32(&bars->ds_free), (item_cnt & 1) ^ 1, cta_err, 68))
+        return;
       tc_fence_after_sync();
-      uint8_t* ds_row = smem + L::kDsOff + (wg * kCols >> 6) * L::kPanelBytes + tid * 128;
+      const uint32_t ds_row = smem_base + L::kDsOff + (wg * kCols >> 6) * L::kPanelBytes + tid * 128;
 #pragma unroll
       for (int c = 0; c < kCols / 16; ++c) {  // 16 queries at a time
         uint32_t dp[16];
@@ -709,8 +707,7 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
 #pragma unroll
         for (int g = 0; g < 2; ++g) {
           const int chunk = ((wg * kCols & 63) >> 3) + c * 2 + g;
-          *reinterpret_cast<uint4*>(ds_row + ((chunk ^ (tid & 7)) * 16)) =
-              make_uint4(ds[4 * g + 0], ds[4 * g + 1], ds[4 * g + 2], ds[4 * g + 3]);
+          st_shared_v4(ds_row + ((chunk ^ (tid & 7)) * 16), ds + 4 * g);
         }
         // ... and one to tensor memory (A operand of dK), over dP^T columns already consumed
         tmem_st8(tmem + TM::kB + lane_off + wg * kCols + c * 8, ds);
@@ -722,9 +719,10 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
       ++step_cnt;
     }
 
-    const int bh_q = DBIAS ? bars->sched_item[item_cnt & 1].bh_q0 + g : 0;
+    const int bh_q = DBIAS ? item().bh_q0 + g : 0;
     if (DBIAS && ragged) {   // keys of one warp may belong to different sequences: one atomic per key
-      if (q_hi > q_lo) atomicAdd(p.dbias + seq * p.H + bh_q, ds_sum);
+      if (q_hi > q_lo)
+        atomicAdd(p.dbias + bwd_seq_of_row(p.cu_seqlens, p.n_seqs, item().j * kT + tid) * p.H + bh_q, ds_sum);
     } else if (DBIAS) {   // sum over the warp, one atomic per warp, item and query head
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) ds_sum += __shfl_xor_sync(0xffffffffu, ds_sum, off);
@@ -740,43 +738,17 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
     // B16 H12 N577 D64 94.5 / 90.3, B16 H16 N512 D64 causal 82.9 / 79.0, B16 H8 padded N1500 D64 225.7 / 216.9,
     // 60 documents in 16384 rows D64 223 / 208.5, B4 H16 N1024 D128 causal ALiBi 87.8 / 80.0,
     // B2 H16 N4096 D128 causal 428 / 418.
-    if constexpr (!kAhead) {   // one group converts dV, the other dK
-      const uint32_t st = item_cnt % L::kKvStages;
-      if (!mbar_wait(smem_u32(&bars->dkv_full), item_cnt & 1, cta_err, 64 + wg)) return;
-      tc_fence_after_sync();
-      uint8_t* stage = smem + st * L::kKvBytes + (wg == 0 ? L::kVOff : L::kKOff);
-#pragma unroll 1
-      for (int share = 0; share < R::kGroups; ++share)
-        bwd_store_acc_rows<D, WIDE>(tmem + (wg == 0 ? TM::kDv : TM::kDk) + lane_off, stage, tid, wg == 0 ? 1.0f : p.scale, share);
-      tc_fence_before_sync();
-      mbar_arrive(smem_u32(&bars->dkv_empty));
-      fence_proxy_async_smem();
-      if (wg == 0) named_barrier_sync<1, 128>(); else named_barrier_sync<2, 128>();
-      if (tid == 0) {
-        const CUtensorMap* tm = wg == 0 ? tmDv : tmDk;
-        if (p.n_sub > 1 || p.i_split > 1 || p.dkv_add)
-          tma_reduce_add_3d(tm, smem_u32(stage), 0, w.j * kT, w.bh);
-        else
-          tma_store_3d(tm, smem_u32(stage), 0, w.j * kT, w.bh);
-        tma_commit_group();
-        tma_wait_group_read<0>();
-        mbar_arrive(smem_u32(wg == 0 ? &bars->v_empty[st] : &bars->k_empty[st]));
-      }
-      bwd_return_item(bars, item_cnt);
-      ++item_cnt;
-      more = bwd_see_item(bars, item_cnt, &w, cta_err);
-      if (more < 0) return;
-    } else {
-    const int done_row = bars->sched_item[item_cnt & 1].j * kT, done_bh = bars->sched_item[item_cnt & 1].bh;
+    const int done_row = item().j * kT, done_bh = item().bh;
+    const uint32_t done = item_cnt & 1, kv_stage = item_cnt % L::kKvStages;
     bwd_return_item(bars, item_cnt);
-    more = bwd_see_item(bars, item_cnt + 1, &w, cta_err);
+    ++item_cnt;
+    more = bwd_see_item(bars, item_cnt, cta_err);
     if (more < 0) return;
-    if (more) row = bwd_row<CAUSAL, ALIBI, ragged>(p, w.j * kT + tid, w.bh_q0);
-    const uint32_t kv_stage = item_cnt % L::kKvStages;
+    if (more) row = bwd_row<CAUSAL, ALIBI, ragged>(p, item(), tid, 0);
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const bool is_dv = r == 0;
-      if (!mbar_wait(smem_u32(is_dv ? &bars->dv_full : &bars->dkv_full), item_cnt & 1, cta_err, is_dv ? 66 : 64)) return;
+      if (!mbar_wait(smem_u32(is_dv ? &bars->dv_full : &bars->dkv_full), done, cta_err, is_dv ? 66 : 64)) return;
       tc_fence_after_sync();
       uint8_t* stage = smem + (is_dv ? kv_stage * L::kKvBytes + L::kVOff
                                      : L::kKvStages == 1 ? L::kDsOff : kv_stage * L::kKvBytes + L::kKOff);
@@ -802,12 +774,10 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
         if (is_dv && !drain(step_cnt - 1)) return;
       }
     }
-    ++item_cnt;
     if (L::kKvStages == 1 && tid == 0 && wg == 0) {   // the next V is waited for
       tma_wait_group_read<0>();
       mbar_arrive(smem_u32(&bars->v_empty[0]));
       release = false;
-    }
     }
   }
   if (tid == 0) tma_wait_group<0>();
@@ -977,7 +947,7 @@ sigattn_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     if (elect_one()) bwd_mma_role<D, WIDE>(smem_base, tmem, &bars, &cta_err);
     __syncwarp();
   } else if (warp < 4 * R::kGroups) {
-    bwd_act_role<D, CAUSAL, ALIBI, DBIAS, KIND, WIDE>(p, &tmDk, &tmDv, warp >> 2, smem, tmem, &bars, &cta_err);
+    bwd_act_role<D, CAUSAL, ALIBI, DBIAS, KIND, WIDE>(p, &tmDk, &tmDv, warp >> 2, smem, smem_base, tmem, &bars, &cta_err);
   } else if constexpr (R::kDrainGroup) {
     bwd_drain_role<D, GROUPED>(p, &tmW, smem, tmem, &bars, &cta_err);
   } else {

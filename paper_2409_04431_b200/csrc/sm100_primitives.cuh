@@ -27,6 +27,11 @@ __device__ __forceinline__ bool elect_one() {
   return pred != 0;
 }
 
+// 16 bytes to shared memory by its 32-bit address (a generic pointer costs two registers).
+__device__ __forceinline__ void st_shared_v4(uint32_t addr, const uint32_t* v) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+}
+
 // ------------------------------------------------------------------ mbarrier
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
