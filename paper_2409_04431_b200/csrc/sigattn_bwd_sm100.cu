@@ -42,8 +42,7 @@ constexpr int kT = 128;  // tile edge: keys per item (TMEM lanes) and queries pe
 // Warp roles.  Narrow: two activation groups of four warps (64 query columns a thread) and a drain group.  Wide
 // (D = 64): four activation groups (32 query columns a thread) that also drain dQ, and a thread that issues its adds.
 // Four warps per scheduler instead of two cover the latency of the activation and feed the exponentials evenly where
-// the warps take different paths, and each path's code is half as long (two chunks of 32 logits on both paths do not
-// fit the instruction cache well); but 512 threads wait, drain and arrive where 256 and 128 did.  The launcher
+// the warps take different paths; but 512 threads wait, drain and arrive where 256 and 128 did.  The launcher
 // chooses (see there).  The 512 activation threads have 96 registers each: room for 32 columns and no more.
 template <int D, bool WIDE>
 struct BwdRoles {
@@ -1226,29 +1225,38 @@ int launch_bwd_bf16(const void* q, const void* k, const void* v, const void* d_o
   // the bias gradient costs the activation groups a running sum (4-5 % of the kernel), so it
   // is compiled in only where it is asked for; likewise the loop over a group's query heads and
   // the per-sequence lengths (kind 1) and the lookups of a batch without padding (kind 2)
-  // (The figures below were taken before the next item was looked up ahead, which made the wide shape 2 to 7 % faster.)
-  // Wide or narrow (see BwdRoles).  Short sequences have b = -log n near the common path's limit, so many warps take
-  // both activation paths, and items of few steps; there four groups pay.  Long ones are bound by the other work of
-  // those groups.  The line is drawn by the length a typical row sees.  Whole backward, us, narrow / wide, H12 or 16:
-  //   no mask: B16 N300 54 / 52, B16 N577 122 / 101, B16 N1025 250 / 245, B16 N1500 387 / 401, B8 N2048 335 / 353;
-  //   causal: B16 N512 97 / 90, B8 N1024 115 / 106, B8 N2048 292 / 292, B2 N4096 246 / 251;
-  //   padded, lengths N/4 to N: N400 64 / 58, N1500 249 / 227, N2500 1010 / 967;
-  //   packed documents: 60 in 16384 rows 337 / 291, 16 in 16384 507 / 462, 5 in 8000 253 / 280.
-  // ALiBi without a mask forms |i - j| for every element, which the 96 registers of the wide shape hold worse (120 to 232
-  // bytes spilled in its general instantiations); causal calls with grouped heads have more steps an item.  B16 H12:
-  //   ALiBi, no mask: N300 48 / 47, N577 102 / 102, N1025 256 / 268, N1250 326 / 334; H_kv4 N300 68 / 66, N577 132 / 144,
-  //   N1250 384 / 420; padded N577 113 / 110, N1250 285 / 268, N2400 1142 / 1134; 60 documents 335 / 332, 16 645 / 682;
-  //   causal H_kv4: N300 57 / 55, N577 84 / 74; with the next item looked up ahead (wide only) B8 H16 H_kv4 N1000 117 / 104,
-  //   B4 N1500 103 / 102, N2000 151 / 147 (ALiBi 167 / 152), N3000 326 / 340, B2 H32 H_kv8 N4000 484 / 500.
+  // Wide or narrow at D = 64 (see BwdRoles).  Short sequences have b = -log n near the common path's limit, so many warps
+  // take both activation paths, and their items have few steps, few of them unmasked; there four groups pay.  Elsewhere
+  // the other work of those groups costs more.  The line is drawn by the length a typical row sees, where the two cross
+  // (whole backward, us, narrow / wide; lengths of padded batches N/4 to N, packed documents in 16384 rows):
+  //   no mask, B16 H12:        N300 43.0 / 41.0, 385 62.7 / 64.4, 577 86.6 / 87.5, 1100 225 / 237, 2048 347 / 371
+  //     ALiBi:                 N260 41.3 / 42.6, 350 42.8 / 43.0, 577 88.2 / 94.1, 1025 245 / 255
+  //     H16 H_kv4:             N300 70.4 / 63.5, 400 98.2 / 90.9, 600 137 / 140, 1500 270 / 290
+  //     the same with ALiBi:   N200 48.6 / 43.1, 385 106 / 102, 520 151 / 156, 1025 344 / 355
+  //   causal, H16:             N300 53.8 / 53.2, 512 79.2 / 75.7, 700 66.2 / 63.7, 850 75.0 / 76.4, 1024 89 / 92, 2048 272 / 280
+  //     ALiBi:                 N300 51.9 / 49.2, 512 72.4 / 71.5, 850 74.8 / 76.1, 2048 280 / 290
+  //     H_kv4:                 N300 62.5 / 59.4, 512 51.9 / 49.7, 577 108 / 113, 1000 94.6 / 98.6, 2000 137 / 145, 3000 309 / 333
+  //     query tiles divided:   B1 H2 N500 19.2 / 19.2, 700 19.4 / 21.1, 2000 27.5 / 29.6
+  //   padded, H8:              N400 51.2 / 49.2, 800 100 / 94, 1000 115 / 118, 1500 203 / 208, 2700 303 / 311
+  //     causal:                N400 47.8 / 47.3, 800 83.8 / 77.9, 1200 132 / 140, 1500 146 / 139, 1800 94.1 / 93.4, 2500 168 / 176
+  //     ALiBi without a mask:  N200 30.7 / 30.2, 400 55.3 / 53.3, 577 72 / 73, 1250 226 / 237
+  //   packed, causal, H16:     120 documents 178 / 162, 60 218 / 186, 20 317 / 299, 14 320 / 310, 12 346 / 343, 10 404 / 404, 8 490 / 499
+  //     H_kv4:                 60 229 / 205, 20 454 / 444, 14 337 / 324, 12 383 / 388, 8 500 / 504;  no mask 60 298 / 252, 12 570 / 579
+  //     ALiBi without a mask:  60 297 / 272, 20 608 / 596, 16 525 / 527, 12 669 / 680
   const int typical_rows = p.cu_seqlens != nullptr ? p.N / p.n_seqs
                            : p.seqlens != nullptr  ? p.N / 2
                            : p.causal              ? p.N / 3 * 2 : p.N;
-  const bool grouped_causal = p.causal && bp.group > 1 && p.seqlens == nullptr && p.cu_seqlens == nullptr;
-  const int wide_rows = (p.slopes != nullptr && !p.causal && p.seqlens == nullptr) ? 512 : grouped_causal ? 1400 : 1280;
+  const bool alibi_no_mask = alibi && !p.causal;
+  const int wide_rows = p.cu_seqlens != nullptr            ? (alibi_no_mask ? 900 : 1280)
+                        : p.seqlens != nullptr             ? (alibi_no_mask ? 250 : 450)
+                        : bp.group > 1                     ? (p.causal ? 360 : 480)
+                        : alibi_no_mask || bp.i_split > 1  ? 0
+                                                           : (p.causal ? 500 : 320);
   const bool wide = p.D == 64 && typical_rows <= wide_rows;
+  // (plain calls with ALiBi and no mask never take the wide shape: it is not compiled for them)
 #define SIGATTN_BWD_SHAPE(DD, CC, AA, BB, KK)                                                              \
-  ((DD == 64 && wide) ? launch_bwd_variant<DD, CC, AA, BB, KK, DD == 64>(maps, bp, num_sms, stream, cuda_err) \
-                      : launch_bwd_variant<DD, CC, AA, BB, KK, false>(maps, bp, num_sms, stream, cuda_err))
+  (wide ? launch_bwd_variant<DD, CC, AA, BB, KK, DD == 64 && !(KK == 0 && AA && !CC)>(maps, bp, num_sms, stream, cuda_err) \
+        : launch_bwd_variant<DD, CC, AA, BB, KK, false>(maps, bp, num_sms, stream, cuda_err))
 #define SIGATTN_BWD_KIND(DD, CC, AA, KK)                                                                   \
   ((p.dbias != nullptr) ? SIGATTN_BWD_SHAPE(DD, CC, AA, true, KK) : SIGATTN_BWD_SHAPE(DD, CC, AA, false, KK))
 #define SIGATTN_BWD_CASE(DD, CC, AA)                                                                       \

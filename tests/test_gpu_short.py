@@ -54,8 +54,8 @@ def test_short_many_heads_equal_the_general_kernels(B, N, causal):
     ("plain", 3, 3, 300), ("causal", 3, 3, 700), ("grouped", 4, 2, 385), ("padded", 2, 2, 520), ("packed", 2, 1, 900),
 ])
 def test_wide_backward_at_64(kind, H, H_kv, N):
-    """The four-group shape of the backward (typical sequences up to 1280 rows, heads of 64): every kind of call that
-    reaches it, with a ragged last tile, several query tiles per item and several items per thread block."""
+    """The four-group shape of the backward (short sequences, heads of 64): every kind of call that reaches it, with a
+    ragged last tile and several query tiles per item."""
     import torch
     import paper_2409_04431_b200 as sa
     B, D, causal = (1 if kind == "packed" else 2), 64, kind in ("causal", "packed")
@@ -81,8 +81,7 @@ def test_wide_backward_at_64(kind, H, H_kv, N):
 @pytest.mark.parametrize("H,H_kv,N,causal", [(3, 3, 500, False), (3, 3, 530, False), (4, 2, 500, False), (4, 2, 530, False),
                                              (4, 2, 890, True), (4, 2, 910, True)])
 def test_backward_shapes_meet_at_64(H, H_kv, N, causal):
-    """ALiBi on both sides of the lines between the wide and the narrow backward: 512 rows without a mask, 900 rows of
-    a causal call with grouped heads (two thirds of them count as typical)."""
+    """ALiBi at lengths of 500 and 900 rows, where both shapes of the backward have served."""
     import torch
     import paper_2409_04431_b200 as sa
     B, D = 1, 64
@@ -94,4 +93,43 @@ def test_backward_shapes_meet_at_64(H, H_kv, N, causal):
     out = sa.sigattn_bwd_gqa(tq, tk, tv, tdo, scale, bias, causal, torch.from_numpy(slopes).cuda())
     sa.sigattn_check()
     for name, g, r in zip(("dQ", "dK", "dV"), out, oracle.sigattn_bwd(q, k, v, d_o, scale, bias, causal, slopes)):
+        assert_bf16_close(to_host(g), r, name)
+
+
+@pytest.mark.parametrize("kind,N,causal,with_slopes", [
+    ("plain", 320, False, False), ("plain", 321, False, False),       # wide up to 320 rows
+    ("plain", 752, True, False), ("plain", 753, True, True),          # 500, two thirds of the rows count as typical
+    ("grouped", 480, False, True), ("grouped", 481, False, False),
+    ("grouped", 542, True, True), ("grouped", 543, True, False),      # 360
+    ("padded", 901, False, False), ("padded", 902, True, False),      # 450, half of the rows
+    ("padded", 501, False, True), ("padded", 502, False, True),       # 250
+    ("packed", 1280, True, False), ("packed", 1281, True, False),     # rows per document
+    ("packed", 900, False, True), ("packed", 901, False, True),
+])
+def test_backward_on_both_sides_of_the_wide_shapes_lines(kind, N, causal, with_slopes):
+    """The last length that the wide shape of the backward serves and the first of the narrow one, for each kind of call."""
+    import torch
+    import paper_2409_04431_b200 as sa
+    B, D = (1 if kind == "packed" else 2), 64
+    H, H_kv = (4, 2) if kind == "grouped" else (2, 2)
+    q, _, _, d_o = inputs.random_case(B, H, N, D, 700 + N)
+    _, k, v, _ = inputs.random_case(B, H_kv, N, D, 701 + N)
+    slopes = (0.5 ** np.arange(1, H + 1)).astype(np.float32) if with_slopes else None
+    sl = None if slopes is None else torch.from_numpy(slopes).cuda()
+    t = [to_device(x, "bf16") for x in (q, k, v, d_o)]
+    scale, bias, more = 1.0 / math.sqrt(D), -math.log(N), {}
+    if kind == "padded":
+        lens = [N, N // 3]
+        out = sa.sigattn_bwd_varlen(*t, scale, bias, torch.tensor(lens, dtype=torch.int32, device="cuda"), causal, sl)
+        more = {"seqlens": lens}
+    elif kind == "packed":
+        cu = np.array([0, N], dtype=np.int32)
+        out = sa.sigattn_bwd_ragged(*t, torch.from_numpy(cu).cuda(), scale, bias, causal, sl)
+        more = {"cu_seqlens": cu}
+    elif kind == "grouped":
+        out = sa.sigattn_bwd_gqa(*t, scale, bias, causal, sl)
+    else:
+        out = sa.sigattn_bwd(*t, scale, bias, causal, sl)
+    sa.sigattn_check()
+    for name, g, r in zip(("dQ", "dK", "dV"), out, oracle.sigattn_bwd(q, k, v, d_o, scale, bias, causal, slopes, **more)):
         assert_bf16_close(to_host(g), r, name)
