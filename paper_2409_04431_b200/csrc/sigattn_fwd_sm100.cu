@@ -278,14 +278,20 @@ __device__ __forceinline__ Item decode_item(const FwdParams& p, int item) {
   return w;
 }
 
-// Whether the polls of a wait are unrolled (see mbar_wait_limit).  Plain calls without a mask at D = 64 are bound by the
-// chain from a tile's logits to the next product and small enough for the instruction cache; there a loop of single polls,
-// which answers a little later, costs more than its shorter code gains.  Forward, us, all unrolled / loop / the activation
-// threads' unrolled and eight at a time in the issuing thread: B8 H12 N4096 563 / 572 / 566, B2 H12 N8100 620 / 630 / 620,
-// B4 H16 N3000 243 / 246 / 243, N2048 168.6 / 169.6 / 167.7, B16 H12 N1025 113.7 / 112.9 / 111.7, B4 H12 N577 15.5 / 14.8 / 15.0.
-// Everywhere else the loop is the fastest: causal ALiBi B8 H16 N2048 133.9 / 127.6 / 128.7 (eight at a time in all roles),
-// padded B16 H8 N1500 103.5 / 94.6 / 95.5, 16 documents in 16384 rows D64 185.9 / 168.8 / 170.3.
-__host__ __device__ constexpr bool fwd_polls_unrolled(int D, bool masked_or_general) { return D == 64 && !masked_or_general; }
+// How many polls of a wait are unrolled (see mbar_wait_limit).  Where the chain from a tile's logits to the next product
+// bounds a kernel that is small enough for the instruction cache, a loop of single polls, which answers a little later, costs
+// more than its shorter code gains: plain calls without a mask at D = 64, and without ALiBi at D = 128.  Forward, us, all
+// unrolled / all a loop / this:
+//   D = 64 without a mask: B8 H12 N4096 563 / 573 / 566, B2 H12 N8100 617 / 629 / 616, B4 H16 N2048 167.6 / 169.4 / 166.8,
+//     B16 H12 N1025 113.6 / 112.9 / 111.0, B4 H12 N577 15.3 / 14.8 / 14.9
+//   D = 128: B1 H8 N16384 causal 497 / 511 / 498, without a mask B4 H16 N2048 152 / 153 / 152, N600 causal 36.0 / 35.5 / 35.5;
+//     ALiBi: B4 H16 N1024 32.1 / 30.7 / 30.8, 299 queries on 12176 keys 102.4 / 104 / 103
+//   others: causal ALiBi B8 H16 N2048 D64 134 / 127.6 / 126.6, causal B2 H16 N4096 111 / 108.4 / 107.3, padded B16 H8 N1500
+//     104 / 94.7 / 94.5, 16 documents in 16384 rows D64 187 / 168.3 / 167.3, 1500 queries on 6000 keys D64 232 / 230 / 227
+__host__ __device__ constexpr int fwd_act_polls(int D, bool causal, bool alibi, int mode) {
+  return (mode == 0 && (D == 64 ? !causal : !alibi)) ? 64 : 1;
+}
+__host__ __device__ constexpr int fwd_mma_polls(int D, bool general) { return (D == 128 && !general) ? 64 : 8; }
 
 // ------------------------------------------------------------------ producer
 
@@ -355,7 +361,7 @@ __device__ void fwd_mma_role(const FwdParams& p, uint32_t smem_base, uint32_t tm
   using L = FwdSmem<D>;
   constexpr uint32_t kIdescS = make_idesc_bf16(kBM, kBN, 0, 0);
   constexpr uint32_t kIdescPV = make_idesc_bf16(kBM, D, 0, 1);
-  constexpr int kPolls = fwd_polls_unrolled(D, CAUSAL || GENERAL) ? 8 : 1;
+  constexpr int kPolls = fwd_mma_polls(D, GENERAL);
   uint32_t kv_cnt = 0;
   uint32_t it[2] = {0, 0};      // items seen per query tile
   uint32_t p_cnt[2] = {0, 0};   // P tiles consumed per query tile
@@ -501,7 +507,7 @@ __device__ void fwd_act_role(const FwdParams& p, const CUtensorMap* tmO, uint8_t
   const int g = threadIdx.x >> 7;            // column group of the tile
   const int tid = threadIdx.x & 127;         // row of the tile
   const uint32_t lane_off = static_cast<uint32_t>(((threadIdx.x >> 5) & 3) * 32) << 16;
-  constexpr int kPolls = fwd_polls_unrolled(D, CAUSAL || MODE != 0) ? 64 : 1;
+  constexpr int kPolls = fwd_act_polls(D, CAUSAL, ALIBI, MODE);
   uint32_t s_cnt0 = 0, s_cnt1 = 0, it[2] = {0, 0};
 
   const bool dynamic = GENERAL || p.dynamic;

@@ -13,8 +13,9 @@
 //
 // What bounds it: the activation (W / 128 * 1024 MUFU cycles a unit and SM, more where unnormalised logits send
 // warps through both evaluations) and the chain around it.  It serves every plain call of its size: measured
-// against the general kernel, us: B32 H12 (no mask) N = 64 14.4 -> 10.3, 128 16.2 -> 14.3, 129 24.7 -> 18.6,
-// 197 28.7 -> 25.8, 256 29.5 -> 28.8; causal B64 H16 N200 59.7 -> 47.7; B1 H12 N50 8.3 -> 6.2, N197 10.3 -> 9.8.
+// against the general kernel when it was new, us: B32 H12 (no mask) N = 64 14.4 -> 10.3, 128 16.2 -> 14.3, 129 24.7 -> 18.6,
+// 197 28.7 -> 25.8, 256 29.5 -> 28.8; causal B64 H16 N200 59.7 -> 47.7; B1 H12 N50 8.3 -> 6.2, N197 10.3 -> 9.8.  Now, one call
+// after the other: 6.1, 9.3, 13.1, 17.9, 20.2; 42.7; 5.1, 5.9.
 #include <atomic>
 
 #include "launch.h"
@@ -90,6 +91,10 @@ sigattn_short_fwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __g
 
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t smem_base = smem_u32(smem);
+  // How many polls of a wait are unrolled (see mbar_wait_limit); forward, us, all / a loop / 8: causal B64 H16 N200
+  // 42.66 / 42.93 / 42.92, B32 H12 N140 15.30 / 15.48 / 15.56; without a mask B64 H16 N200 39.6 / 39.4 / 39.1, B32 H12 N64
+  // 6.24 / 6.15 / 6.06; causal ALiBi B64 H16 N200 40.7 / 40.4 / 40.2.
+  constexpr int kPolls = (CAUSAL && !ALIBI) ? 64 : 8;
   const int warp = threadIdx.x >> 5;
   // contiguous runs of units per thread block: the units of a head share K and V
   const int u0 = static_cast<int>(static_cast<long long>(blockIdx.x) * p.n_units / gridDim.x);
@@ -138,11 +143,11 @@ sigattn_short_fwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __g
         const ShortUnit w = short_unit<CAUSAL>(p, u);
         const uint32_t i = u - u0;
         // unit i - 1 has computed its logits: Q and K may be overwritten; its O: V may be
-        if (i > 0 && !mbar_wait(smem_u32(&bars.qk_empty), (i - 1) & 1, cta_err, 10)) break;
+        if (i > 0 && !mbar_wait<kPolls>(smem_u32(&bars.qk_empty), (i - 1) & 1, cta_err, 10)) break;
         if (w.head != last_head) load_kv(&tmK, kSfK, &bars.k_full, w.head);
         mbar_arrive_expect_tx(smem_u32(&bars.q_full), kSfTileBytes);
         tma_load_3d(smem_base + kSfQ, &tmQ, smem_u32(&bars.q_full), 0, w.row0, w.head);
-        if (i > 0 && !mbar_wait(smem_u32(&bars.v_empty), (i - 1) & 1, cta_err, 11)) break;
+        if (i > 0 && !mbar_wait<kPolls>(smem_u32(&bars.v_empty), (i - 1) & 1, cta_err, 11)) break;
         if (w.head != last_head) load_kv(&tmV, kSfV, &bars.v_full, w.head);
         last_head = w.head;
       }
@@ -162,9 +167,9 @@ sigattn_short_fwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __g
         const bool new_head = w.head != last_head;
         last_head = w.head;
         if (new_head) ++heads;
-        if (new_head && !mbar_wait(smem_u32(&bars.k_full), (heads - 1) & 1, cta_err, 20)) break;
-        if (!mbar_wait(smem_u32(&bars.q_full), par, cta_err, 21)) break;
-        if (i > 0 && !mbar_wait(smem_u32(&bars.o_empty), par ^ 1, cta_err, 22)) break;   // tensor memory free again
+        if (new_head && !mbar_wait<kPolls>(smem_u32(&bars.k_full), (heads - 1) & 1, cta_err, 20)) break;
+        if (!mbar_wait<kPolls>(smem_u32(&bars.q_full), par, cta_err, 21)) break;
+        if (i > 0 && !mbar_wait<kPolls>(smem_u32(&bars.o_empty), par ^ 1, cta_err, 22)) break;   // tensor memory free again
         tc_fence_after_sync();
         const uint32_t idesc_s = make_idesc_bf16(kSfRows, 0, 0, 0) | (static_cast<uint32_t>(w.width >> 3) << 17);
 #pragma unroll
@@ -172,8 +177,8 @@ sigattn_short_fwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __g
           umma_ss(tmem, desc_advance(q_desc, ks * 32), desc_advance(k_desc, ks * 32), idesc_s, ks > 0);
         umma_commit(smem_u32(&bars.s_full));
         umma_commit(smem_u32(&bars.qk_empty));
-        if (new_head && !mbar_wait(smem_u32(&bars.v_full), (heads - 1) & 1, cta_err, 23)) break;
-        if (!mbar_wait(smem_u32(&bars.p_full), par, cta_err, 24)) break;
+        if (new_head && !mbar_wait<kPolls>(smem_u32(&bars.v_full), (heads - 1) & 1, cta_err, 23)) break;
+        if (!mbar_wait<kPolls>(smem_u32(&bars.p_full), par, cta_err, 24)) break;
         tc_fence_after_sync();
         const int h16 = w.half >> 4, n16 = w.width >> 4;
 #pragma unroll 4
@@ -200,7 +205,7 @@ sigattn_short_fwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __g
       const float bias = p.bias_vec ? __ldg(p.bias_vec + w.head) * kSfLog2e : p.bias_log2e;
       const int col0 = g ? w.half : 0;
       const int runs = ((g ? w.width : w.half) - col0) >> 5;
-      if (!mbar_wait(smem_u32(&bars.s_full), par, cta_err, 30)) break;
+      if (!mbar_wait<kPolls>(smem_u32(&bars.s_full), par, cta_err, 30)) break;
       tc_fence_after_sync();
       if (live) {
         const uint32_t t0 = tmem + lane_off + col0;
@@ -221,7 +226,7 @@ sigattn_short_fwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __g
       mbar_arrive(smem_u32(&bars.p_full));
 
       // O: 32 of the 64 columns per group
-      if (!mbar_wait(smem_u32(&bars.o_full), par, cta_err, 31)) break;
+      if (!mbar_wait<kPolls>(smem_u32(&bars.o_full), par, cta_err, 31)) break;
       tc_fence_after_sync();
       if (live) {
         uint32_t o[32];
