@@ -359,7 +359,9 @@ __device__ void bwd_load_role(const BwdParams& p, const CUtensorMap* tmQ, const 
       ++item_cnt;
       return true;
     };
-    if (L::kKvStages == 1) {   // they can only be loaded when the item before is done: at least from L2 then
+    // They can only be loaded when the item before is done: at least from L2 then (D = 128, whole backward, us, without /
+    // with: 120 documents in 16384 rows 244 / 240, B4 H16 N1024 causal ALiBi 80.4 / 79.5; longer items the same).
+    if (L::kKvStages == 1) {
 #pragma unroll
       for (int pn = 0; pn < L::kPanels; ++pn) {
         tma_prefetch_3d(tmK, pn * 64, w.j * kT, w.bh);
@@ -733,7 +735,8 @@ __device__ void bwd_act_role(const BwdParams& p, const CUtensorMap* tmDk, const 
     // converted and stored from the V buffer; then scale * dK, from the K buffer (D = 128: from where dS was).  The
     // buffers go back once the stores have read them: with two of them after the next P phase, by when they have.
     // Waited for at once, with both results converted after the last product and the next item looked up then, the
-    // threads stood 5000 to 6000 cycles between two items (clock traces).  Whole backward, us, that way / this way:
+    // threads stood 5000 to 6000 cycles between two items (clock traces).  Whole backward, us, that way / this way (both
+    // with the polls of all waits unrolled, see mbar_wait_limit):
     // B16 H12 N577 D64 94.5 / 90.3, B16 H16 N512 D64 causal 82.9 / 79.0, B16 H8 padded N1500 D64 225.7 / 216.9,
     // 60 documents in 16384 rows D64 223 / 208.5, B4 H16 N1024 D128 causal ALiBi 87.8 / 80.0,
     // B2 H16 N4096 D128 causal 428 / 418.

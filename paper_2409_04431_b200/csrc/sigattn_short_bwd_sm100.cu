@@ -18,10 +18,10 @@
 //
 // Sixteen activation warps (32 columns a thread; four per scheduler hide the chain's latency); the epilogues are
 // theirs too, so registers allow them.  What bounds it: the activation phases of a step (P, then dS) and the wait
-// for the next S^T between them (at B32 H12 N197 38 % of the issue slots, 25 % of the MUFU pipe and 15 % of the tensor
-// pipe are in use).  Measured, whole backward, us, clear + general kernel + conversion / this: B32 H12 N197 61.8 / 36.9,
-// N64 28.7 / 12.7, N128 32.8 / 16.5, N256 74.2 / 43.2; causal B64 H16 N200 143 / 84.6; B1 H12 N50 13.6 / 7.2, N197
-// 19.5 / 15.2.
+// for the next S^T between them (at B32 H12 N197 43 % of the issue slots, 29 % of the MUFU pipe and 17 % of the tensor
+// pipe are in use).  Measured when it was new, whole backward, us, clear + general kernel + conversion / this: B32 H12 N197
+// 61.8 / 36.9, N64 28.7 / 12.7, N128 32.8 / 16.5, N256 74.2 / 43.2; causal B64 H16 N200 143 / 84.6; B1 H12 N50 13.6 / 7.2,
+// N197 19.5 / 15.2.  Now, one call after the other: 32.5, 9.6, 13.0, 36.2; 74.2; 7.5, 12.6.
 #include <atomic>
 
 #include "launch.h"

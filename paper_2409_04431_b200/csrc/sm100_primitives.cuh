@@ -67,7 +67,8 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 // failure, the wait gives up, records the failure in `*cta_error` (shared memory) and
 // returns false.  Callers leave their loops on false and fall through to the common
 // tear-down, so the kernel always terminates and frees its tensor memory.
-// UNROLL: how many of 64 polls follow one another in the code.
+// UNROLL: how many of 64 polls follow one another in the code.  One, except in small kernels whose time is a chain of
+// waits, which then answer 10 to 20 cycles sooner (see their callers).
 constexpr long long kWaitLimitCycles = 2000000000LL;  // about one second
 
 template <int UNROLL = 1>
@@ -78,9 +79,10 @@ __device__ __forceinline__ bool mbar_wait_limit(uint32_t bar, uint32_t parity, v
   while (true) {
     // Kept a loop: unrolled, the 64 polls are 2 to 3 KB of code at every wait, half of a kernel's code, and warps that
     // wait walk through them while others run the steps; the instruction cache then loses the steps.  Backward at
-    // D = 64, code 148 -> 88 KB, warps stalled for instructions 1.79 -> 0.93 of those issued (B8 H8 N2700 padded).
-    // Whole backward, us, unrolled / loop: B8 H8 N2700 D64 padded 362 / 300, B4 H32 H_kv8 N3000 D64 causal ALiBi 699 / 639,
-    // B8 H16 N2048 D64 causal ALiBi 325 / 302, 60 documents in 16384 rows D64 208 / 187, D128 313 / 286.
+    // D = 64, code 148 -> 88 KB; warps stalled for an instruction for each one that issues 1.79 -> 0.45 (padded B8 H8 N2700)
+    // and 1.14 -> 0.41 (causal ALiBi B2 H16 H_kv4 N4000).  Whole backward, us, unrolled / loop: B8 H8 N2700 D64 padded
+    // 362 / 300, B4 H32 H_kv8 N3000 D64 causal ALiBi 699 / 639, B8 H16 N2048 D64 causal ALiBi 325 / 302, 60 documents in
+    // 16384 rows D64 208 / 187, D128 313 / 286.
 #pragma unroll UNROLL
     for (int i = 0; i < 64; ++i) {
       if (mbar_try_wait(bar, parity)) return true;
