@@ -433,6 +433,8 @@ __device__ void fwd_mma_role(const FwdParams& p, uint32_t smem_base, uint32_t tm
     if (!mbar_wait<kPolls>(smem_u32(&bars->o_empty[0]), (it[0] & 1) ^ 1, cta_err, 23)) return;
     if (w.n[1] > 0 && !mbar_wait<kPolls>(smem_u32(&bars->o_empty[1]), (it[1] & 1) ^ 1, cta_err, 24)) return;
 
+    // (an item's last commit is an o_full: the activation threads wait for it before the block can end, while nothing waits
+    // for the last V buffer of a block's last item)
     for (int j = 0; j < w.n_kv; ++j) {
       if (!kv_wait(v_cnt(j))) return;
       const bool more = (j + 1 < w.n_kv);
@@ -441,7 +443,10 @@ __device__ void fwd_mma_role(const FwdParams& p, uint32_t smem_base, uint32_t tm
         ++p_cnt[0];
         tc_fence_after_sync();
         issue_pv(0, kv_addr(v_cnt(j)), j > 0);
-        if (j == w.n[0] - 1) umma_commit(smem_u32(&bars->o_full[0]));
+        if (j == w.n[0] - 1) {
+          if (!more && j >= w.n[1]) kv_release(v_cnt(j));
+          umma_commit(smem_u32(&bars->o_full[0]));
+        }
       }
       if (more && !kv_wait(k_cnt(j + 1))) return;
       if (j + 1 < w.n[0]) {
@@ -455,9 +460,12 @@ __device__ void fwd_mma_role(const FwdParams& p, uint32_t smem_base, uint32_t tm
         ++p_cnt[1];
         tc_fence_after_sync();
         issue_pv(1, kv_addr(v_cnt(j)), j > 0);
-        if (j == w.n[1] - 1) umma_commit(smem_u32(&bars->o_full[1]));
+        if (j == w.n[1] - 1) {
+          if (!more) kv_release(v_cnt(j));
+          umma_commit(smem_u32(&bars->o_full[1]));
+        }
       }
-      kv_release(v_cnt(j));
+      if (more) kv_release(v_cnt(j));
       if (j + 1 < w.n[1]) {
         issue_s(1, kv_addr(k_cnt(j + 1)));
         umma_commit(smem_u32(&bars->s_full[1]));

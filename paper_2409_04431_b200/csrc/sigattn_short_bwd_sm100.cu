@@ -260,8 +260,6 @@ sigattn_short_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __g
           umma_ss(tmem + kSbDq + s.i * kSbD, desc_advance(ds_mn, ks * 2048), desc_advance(k_mn, ks * 2048), kIdescDq,
                   (s.j > 0 || ks > 0));
         if (last_of_j) {
-          umma_commit(smem_u32(&bars.acc_full));
-          ++n_acc;
           umma_commit(smem_u32(&bars.empty[slot(k_tile(s.j), s.h)]));
           umma_commit(smem_u32(&bars.empty[slot(v_tile(s.j), s.h)]));
         }
@@ -270,6 +268,10 @@ sigattn_short_bwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __g
         if (s.j == n_tiles - 1 && (one_tile || s.i == 1)) {
           umma_commit(smem_u32(&bars.empty[slot(q_tile(s.i), s.h)]));
           umma_commit(smem_u32(&bars.empty[slot(do_tile(s.i), s.h)]));
+        }
+        if (last_of_j) {   // after the others: nothing waits for the slots of a block's last head
+          umma_commit(smem_u32(&bars.acc_full));
+          ++n_acc;
         }
         if (more) ok = issue_dp(next);
         s = next;

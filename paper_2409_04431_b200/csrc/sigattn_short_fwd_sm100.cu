@@ -186,8 +186,8 @@ sigattn_short_fwd_bf16_kernel(const __grid_constant__ CUtensorMap tmQ, const __g
           const uint32_t p_col = ks < h16 ? ks * 8 : w.half + (ks - h16) * 8;
           umma_ts(tmem + w.o_col, tmem + p_col, desc_advance(v_desc, ks * 2048), kIdescPV, ks > 0);
         }
-        umma_commit(smem_u32(&bars.o_full));
         umma_commit(smem_u32(&bars.v_empty));
+        umma_commit(smem_u32(&bars.o_full));   // last: nothing waits for the v_empty of a block's last unit
       }
     }
     __syncwarp();
